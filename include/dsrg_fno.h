@@ -54,8 +54,8 @@ typedef enum {
  * tensor cores (tcgen05) with exact float32 level sums, merged into
  * double-float accumulators (float32 hi + lo pairs, about 48 bits); the
  * regulariser and the dressing of this form run in double-float, the energy
- * and D_vv sums in float64.  In both forms the NO eigensolve runs in
- * double-float.  On the workloads here the two forms agree to a few 1e-9 E_h
+ * and D_vv sums in float64.  In both forms the NO eigensolve runs in float64
+ * (double-float below 33 rows).  On the workloads here the two forms agree to a few 1e-9 E_h
  * in energies; ONs are tested to agree within 1e-8. */
 /* BF16X3 and TF32 are the literal forms of the precision study: only the
  * contractions of B with B (nu^{ij}_{ab} = sum_Q B^Q_{ia} B^Q_{jb}, Eq. A7, of
@@ -214,7 +214,7 @@ int dsrg_fno_cut(int32_t nvir, const double* ons, int32_t mode, double threshold
  * may synchronise the device, is not acceptable.  This call does the same
  * eigensolve and cut as dsrg_fno_truncate with the same arguments, but its
  * scratch is one fixed file-scope device array of the library (5 nvir^2
- * doubles and a few KB for nvir up to 512, about 10.5 MB), held by every device that loads
+ * doubles and about 110 KB for nvir up to 512, about 10.6 MB), held by every device that loads
  * the library until the process exits.
  *   - nvir > 512 returns DSRG_FNO_ERR_ARG, with the limit named in a message
  *     to the log callback (dsrg_fno_set_log_callback).  dvv, on_out and
@@ -264,7 +264,7 @@ int dsrg_fno_ladder(int32_t nv, int32_t naux, const double* B_vv, int32_t npairs
  *   threshold  absolute eigenvalue threshold (w > threshold kept).
  *   precision  DSRG_FNO_FP64, or DSRG_FNO_SLICED_BF16 (digit-plane
  *              contractions: 5 planes for W, 6 for B'); the eigensolve is the
- *              double-float Jacobi solver in both.
+ *              same in both.
  *   B_out      device [naux][nh][np], caller-allocated: its first naux'
  *              slices receive B' (the rest is left untouched).
  *   w_out      device [naux] or NULL: every eigenvalue of W, descending.

@@ -78,9 +78,9 @@ int dsrg_fno_debug_set_fused_epilogue(int32_t on);
  * problem's count).  Affects later calls of this process. */
 int dsrg_fno_debug_set_syrk_planes(int32_t nslices);
 
-/* on != 0 (the default): symmetric eigensolves above 80 x 80 run on the
- * column-pair Jacobi kernel; 0: on the round-parallel kernel over A in
- * global memory (for comparison).  Affects later calls of this process. */
+/* on != 0 (the default): symmetric eigensolves above 32 x 32 run on the
+ * divide-and-conquer solver; 0: on the Jacobi kernels (up to 80 x 80 in shared
+ * memory, above that round-parallel over A in global memory; for comparison).  Affects later calls of this process. */
 int dsrg_fno_debug_set_eig_colpair(int32_t on);
 
 /* Symmetric eigensolves of `count` (1..4) matrices at once, as the density

@@ -454,5 +454,5 @@ def dsrg_fno_debug_set_syrk_planes(nslices: int):
 
 
 def dsrg_fno_debug_set_eig_colpair(on: bool):
-    """Column-pair Jacobi kernel (True, default) or the round-parallel one."""
+    """Divide-and-conquer eigensolver (True, default) or the Jacobi kernels."""
     _check("dsrg_fno_debug_set_eig_colpair", load().dsrg_fno_debug_set_eig_colpair(1 if on else 0))

@@ -1,4 +1,10 @@
-// Symmetric eigensolver (Eq. 8: Gamma V = n V) and helpers.
+// Symmetric eigensolver (Eq. 8: Gamma V = n V) and helpers: the dispatch, the
+// Jacobi kernels and the sorting.  From EIG_DC_MIN_N = 33 rows on the solver is
+// divide and conquer in float64 (eig_dc.cu): at 34 rows it takes 0.72 ms
+// against 0.78 ms here, at 80 1.3 against 5.1, at 203 3.1 against 9.1, at 1200
+// 27 against 97 (D_vv-like matrices; errors 2e-15 of the largest eigenvalue
+// against 1e-13).  The Jacobi kernels keep the smaller matrices, those above
+// EIG_DC_MAX_N, and the density step's, which share one launch.
 //
 // Cyclic two-sided Jacobi with round-robin pair ordering: in each round the
 // indices form m/2 disjoint pairs (m = n rounded up to even, a padding index
@@ -18,6 +24,7 @@
 // is not the exact annihilating angle, and the next sweep removes what is
 // left of a_pq.  A is double-buffered (every block of A' reads four entries
 // of A); V is updated in place (a thread owns a column pair).
+#include <algorithm>
 #include <atomic>
 
 #include "dd.cuh"
@@ -374,249 +381,6 @@ __global__ void __launch_bounds__(JNT, 1) jacobi_smem_batch_kernel(const __grid_
 }
 
 
-// The rotation (c, s) that annihilates a_pq (a_pp, a_qq, a_pq double-float):
-// t from float32 arithmetic on the double-float difference, c and s in
-// double-float renormalised so that c^2 + s^2 = 1 to working precision.
-__device__ __forceinline__ float4 jacobi_rotation(dd app, dd aqq, dd apq) {
-  if (apq.hi == 0.0f) return make_float4(1.f, 0.f, 0.f, 0.f);
-  const dd d = dd_sub(aqq, app);
-  const float th = d.hi / (2.0f * apq.hi);
-  const float t = (th >= 0.0f ? 1.0f : -1.0f) / (fabsf(th) + sqrtf(fmaf(th, th, 1.0f)));
-  dd c = dd_rsqrt12(dd_add_f(two_prod(t, t), 1.0f));
-  dd sn = dd_mul_f(c, t);
-  const float g = dd_sub(dd_add(dd_mul(c, c), dd_mul(sn, sn)), dd_make(1.0f)).hi;
-  c = dd_add(c, dd_mul_f(c, -0.5f * g));
-  sn = dd_add(sn, dd_mul_f(sn, -0.5f * g));
-  return make_float4(c.hi, c.lo, sn.hi, sn.lo);
-}
-
-// position of index j in round r of the round-robin ordering (inverse of rr_index)
-__device__ __forceinline__ int rr_position(int j, int r, int m) {
-  return j == 0 ? 0 : ((j - 1 - r) % (m - 1) + (m - 1)) % (m - 1) + 1;
-}
-
-// ---------------------------------------------------------------------------
-// Column-pair Jacobi.  The same cyclic two-sided Jacobi with round-robin
-// pairs, organised around column pairs: in a round, block b owns the column
-// pairs k in [b cp, (b+1) cp) of A and V.  For its pair (p, q) it reads
-// columns p and q (A in column-major double-float; A stays symmetric), forms
-// M = A J on them, then A' = J^T M for every row pair of the round (the
-// rotations of all pairs are known to every block), rotates V's columns p, q,
-// and writes the columns back.  With the new columns it publishes a_jj and
-// a_{partner(j), j} for the next round's pairing, from which every block
-// forms all rotations of the next round: one grid barrier per round, the
-// matrix moving through L2 once per round.
-struct ColPairArgs {
-  int n, m, half, cp, cpc;  // pairs per block, pairs held in shared memory at a time
-  const double* A_in;
-  double* A_out;
-  double* V_out;
-  float2* Ac;    // [n][n]: Ac[j][i] = A[i][j]
-  float2* Vc;    // [n][n]: Vc[j][i] = V[i][j]
-  float2* pub;   // [2][2][m]: per parity, a_jj and a_{partner(j), j}
-  double* nrm2;  // [n] squared column norms of V
-  double* red;   // 2 * gridDim.x partial norms
-  unsigned* bar;
-  int* status;   // [0] 1 = no convergence, [1] 1 = barrier wait expired, [2] sweeps
-  int max_sweeps;
-};
-
-// threads per block of the column-pair kernel: one block per SM, so the
-// latency of its column loads is hidden by the warps of that one block
-constexpr int CPT = 1024;
-
-// the round that follows round r of sweep `sw` (the next sweep starts at round 0)
-__device__ __forceinline__ int next_round(int r, int m) { return r + 1 < m - 1 ? r + 1 : 0; }
-
-__global__ void __launch_bounds__(CPT) jacobi_colpair_kernel(ColPairArgs P) {
-  extern __shared__ float4 s_rot[];                              // [half]
-  int2* s_pair = reinterpret_cast<int2*>(s_rot + P.half);       // [half]
-  float2* colP = reinterpret_cast<float2*>(s_pair + P.half);   // [2 cpc][n]: p and q columns of each pair
-  const int n = P.n, m = P.m, half = P.half;
-  const long n2 = (long)n * n;
-  // ---- set-up: A (symmetrised) and V = 1 in columns, round 0's inputs
-  for (long idx = blockIdx.x * (long)CPT + threadIdx.x; idx < n2; idx += (long)gridDim.x * CPT) {
-    const int j = (int)(idx / n), i = (int)(idx % n);
-    const dd a = dd_from_double(0.5 * (P.A_in[(long)i * n + j] + P.A_in[(long)j * n + i]));
-    P.Ac[idx] = make_float2(a.hi, a.lo);
-    P.Vc[idx] = make_float2(i == j ? 1.0f : 0.0f, 0.0f);
-  }
-  for (int j = blockIdx.x * CPT + threadIdx.x; j < n; j += gridDim.x * CPT) {
-    const int pos = rr_position(j, 0, m);
-    const int pj = rr_index(m - 1 - pos, 0, m);
-    const double a = 0.5 * (P.A_in[(long)j * n + j] + P.A_in[(long)j * n + j]);
-    const dd djj = dd_from_double(a);
-    dd off = dd_make(0.0f);
-    if (pj < n) off = dd_from_double(0.5 * (P.A_in[(long)pj * n + j] + P.A_in[(long)j * n + pj]));
-    P.pub[j] = make_float2(djj.hi, djj.lo);
-    P.pub[m + j] = make_float2(off.hi, off.lo);
-  }
-  if (!grid_barrier_at(P.bar, P.status)) return;
-  const double tol = fmax(1e-30, ((double)n * 4e-15) * ((double)n * 4e-15));
-  double prev = -1.0;
-  int converged = 0, sweeps_done = 0, cur = 0;
-  for (int sweep = 0; sweep <= P.max_sweeps; ++sweep) {
-    sweeps_done = sweep;
-    // ---- convergence: off-diagonal and total squared norms (fixed order)
-    {
-      __shared__ double s_o[CPT], s_t[CPT];
-      double o = 0.0, t = 0.0;
-      for (long idx = blockIdx.x * (long)CPT + threadIdx.x; idx < n2; idx += (long)gridDim.x * CPT) {
-        const float2 v = __ldcg(P.Ac + idx);
-        const double a = (double)v.x + (double)v.y;
-        t += a * a;
-        if (idx / n != idx % n) o += a * a;
-      }
-      s_o[threadIdx.x] = o;
-      s_t[threadIdx.x] = t;
-      __syncthreads();
-      for (int w = CPT / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) {
-          s_o[threadIdx.x] += s_o[threadIdx.x + w];
-          s_t[threadIdx.x] += s_t[threadIdx.x + w];
-        }
-        __syncthreads();
-      }
-      if (threadIdx.x == 0) {
-        __stcg(P.red + 2 * blockIdx.x, s_o[0]);
-        __stcg(P.red + 2 * blockIdx.x + 1, s_t[0]);
-      }
-      if (!grid_barrier_at(P.bar, P.status)) return;
-      double so = 0.0, st = 0.0;
-      for (int b = 0; b < (int)gridDim.x; ++b) {
-        so += __ldcg(P.red + 2 * b);
-        st += __ldcg(P.red + 2 * b + 1);
-      }
-      if (st == 0.0 || so <= tol * st || (so <= 1e-22 * st && prev >= 0.0 && so > 0.25 * prev)) {
-        converged = 1;
-        break;
-      }
-      prev = so;
-      if (sweep == P.max_sweeps) break;
-    }
-    for (int r = 0; r < m - 1; ++r) {
-      const float2* pd = P.pub + (size_t)cur * 2 * m;      // a_jj
-      const float2* po = pd + m;                             // a_{partner(j), j}
-      // ---- all rotations of this round, from the published entries
-      for (int k = threadIdx.x; k < half; k += CPT) {
-        const int i1 = rr_index(k, r, m), i2 = rr_index(m - 1 - k, r, m);
-        const int p = min(i1, i2), q = max(i1, i2);
-        float4 cs = make_float4(1.f, 0.f, 0.f, 0.f);
-        if (q < n) {
-          const float2 dp = __ldcg(pd + p), dq = __ldcg(pd + q), op = __ldcg(po + p), oq = __ldcg(po + q);
-          const dd apq = dd_mul_f(dd_add(dd{op.x, op.y}, dd{oq.x, oq.y}), 0.5f);
-          cs = jacobi_rotation(dd{dp.x, dp.y}, dd{dq.x, dq.y}, apq);
-        }
-        s_rot[k] = cs;
-        s_pair[k] = make_int2(p, q);
-      }
-      __syncthreads();
-      float2* nd = P.pub + (size_t)(cur ^ 1) * 2 * m;
-      float2* no = nd + m;
-      const int rn = next_round(r, m);
-      const int k0 = blockIdx.x * P.cp;
-      const int kend = min(k0 + P.cp, half);
-      // this block's pairs, P.cpc at a time (as many as shared memory holds)
-      for (int kb = k0; kb < kend; kb += P.cpc) {
-        const int nk = min(P.cpc, kend - kb);
-        // M = A J on columns p, q of each pair (colP / colQ rows of length n)
-        for (int idx = threadIdx.x; idx < nk * n; idx += CPT) {
-          const int kk = idx / n, i = idx - kk * n;
-          const int2 pq = s_pair[kb + kk];
-          const float4 cc = s_rot[kb + kk];
-          const dd c = {cc.x, cc.y}, sn = {cc.z, cc.w};
-          const float2 a = __ldcg(P.Ac + (long)pq.x * n + i);
-          float2* cP = colP + (size_t)kk * 2 * n;
-          if (pq.y < n) {
-            const float2 b = __ldcg(P.Ac + (long)pq.y * n + i);
-            const dd ap = {a.x, a.y}, aq = {b.x, b.y};
-            const dd mp = rot_combine(c, ap, sn, aq, true), mq = rot_combine(sn, ap, c, aq, false);
-            cP[i] = make_float2(mp.hi, mp.lo);
-            cP[n + i] = make_float2(mq.hi, mq.lo);
-            // V J on the same columns (rows are independent)
-            const float2 va = __ldcg(P.Vc + (long)pq.x * n + i), vb = __ldcg(P.Vc + (long)pq.y * n + i);
-            const dd vp = {va.x, va.y}, vq = {vb.x, vb.y};
-            const dd wp = rot_combine(c, vp, sn, vq, true), wq = rot_combine(sn, vp, c, vq, false);
-            __stcg(P.Vc + (long)pq.x * n + i, make_float2(wp.hi, wp.lo));
-            __stcg(P.Vc + (long)pq.y * n + i, make_float2(wq.hi, wq.lo));
-          } else {
-            cP[i] = a;
-          }
-        }
-        __syncthreads();
-        // A' = J^T M: every row pair of the round, on every loaded column, in place
-        for (int idx = threadIdx.x; idx < nk * 2 * half; idx += CPT) {
-          const int col = idx / half, k2 = idx - col * half;   // col: 2 kk + (0: p, 1: q)
-          const int kk = col >> 1;
-          if ((col & 1) && s_pair[kb + kk].y >= n) continue;
-          const int2 rq = s_pair[k2];
-          if (rq.y >= n) continue;
-          const float4 rc = s_rot[k2];
-          const dd cr = {rc.x, rc.y}, sr = {rc.z, rc.w};
-          float2* cc = colP + (size_t)col * n;
-          const float2 x = cc[rq.x], y = cc[rq.y];
-          const dd xp = {x.x, x.y}, yq = {y.x, y.y};
-          const dd u = rot_combine(cr, xp, sr, yq, true), v = rot_combine(sr, xp, cr, yq, false);
-          cc[rq.x] = make_float2(u.hi, u.lo);
-          cc[rq.y] = make_float2(v.hi, v.lo);
-        }
-        __syncthreads();
-        for (int idx = threadIdx.x; idx < nk * 2 * n; idx += CPT) {
-          const int col = idx / n, i = idx - col * n;
-          const int2 pq = s_pair[kb + (col >> 1)];
-          const int j = (col & 1) ? pq.y : pq.x;
-          if (j < n) __stcg(P.Ac + (long)j * n + i, colP[(size_t)col * n + i]);
-        }
-        // the next round's inputs of the loaded columns
-        for (int col = threadIdx.x; col < 2 * nk; col += CPT) {
-          const int2 pq = s_pair[kb + (col >> 1)];
-          const int j = (col & 1) ? pq.y : pq.x;
-          if (j >= n) continue;
-          const float2* cc = colP + (size_t)col * n;
-          const int pj = rr_index(m - 1 - rr_position(j, rn, m), rn, m);
-          __stcg(nd + j, cc[j]);
-          __stcg(no + j, pj < n ? cc[pj] : make_float2(0.f, 0.f));
-        }
-        __syncthreads();
-      }
-      if (!grid_barrier_at(P.bar, P.status)) return;
-      cur ^= 1;
-    }
-  }
-  // ---- output: Rayleigh quotients and eigenvectors normalised by the
-  // column norms of V (they drift from 1 by rounding of the rotations)
-  double* nrm2 = P.nrm2;
-  for (int j = blockIdx.x; j < n; j += gridDim.x) {
-    __shared__ double s_r[CPT];
-    double acc = 0.0;
-    for (int i = threadIdx.x; i < n; i += CPT) {
-      const float2 v = __ldcg(P.Vc + (long)j * n + i);
-      const dd vv = dd_mul(dd{v.x, v.y}, dd{v.x, v.y});
-      acc += dd_to_double(vv);
-    }
-    s_r[threadIdx.x] = acc;
-    __syncthreads();
-    for (int w = CPT / 2; w > 0; w >>= 1) {
-      if (threadIdx.x < w) s_r[threadIdx.x] += s_r[threadIdx.x + w];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) __stcg(nrm2 + j, s_r[0]);
-    __syncthreads();
-  }
-  if (!grid_barrier_at(P.bar, P.status)) return;
-  for (long idx = blockIdx.x * (long)CPT + threadIdx.x; idx < n2; idx += (long)gridDim.x * CPT) {
-    const int i = (int)(idx / n), j = (int)(idx % n);
-    const float2 a = __ldcg(P.Ac + (long)j * n + i), v = __ldcg(P.Vc + (long)j * n + i);
-    const double nj = __ldcg(nrm2 + j), ni = __ldcg(nrm2 + i);
-    P.A_out[idx] = ((double)a.x + (double)a.y) / (i == j ? nj : sqrt(nj * ni));
-    P.V_out[idx] = ((double)v.x + (double)v.y) / sqrt(nj);
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    P.status[0] = converged ? 0 : 1;
-    P.status[2] = sweeps_done;
-  }
-}
-
 // ranks by (value descending | ascending, index ascending)
 __global__ void eig_rank_kernel(int n, const double* __restrict__ A, bool descending, int* rank) {
   int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -675,68 +439,18 @@ static thread_local bool t_device_shared = false;
 SharedDeviceScope::SharedDeviceScope(bool shared) : prev(t_device_shared) { t_device_shared = shared; }
 SharedDeviceScope::~SharedDeviceScope() { t_device_shared = prev; }
 
-// A (n x n, symmetric) is destroyed: on return its diagonal holds the
-// eigenvalues; V (n x n) receives the eigenvectors (column j <-> A[j][j]).
-// work: eig_work_doubles(n) doubles.  status_dev: four ints of device memory.
-// Matrices above the shared-memory size: the column-pair kernel (default) or
-// the round-parallel kernel over A in global memory (test hook, comparison).
-static std::atomic<int> g_eig_colpair{1};
-void set_eig_colpair(bool on) { g_eig_colpair.store(on ? 1 : 0); }
+// Matrices of EIG_DC_MIN_N to EIG_DC_MAX_N rows: divide and conquer (default)
+// or Jacobi like the others (test hook, comparison).
+static std::atomic<int> g_eig_dc{1};
+void set_eig_colpair(bool on) { g_eig_dc.store(on ? 1 : 0); }
 
-static int eig_colpair(int n, int m, double* A, double* V, double* work, int* status_dev, int max_sweeps,
-                       cudaStream_t st) {
-  const long n2 = (long)n * n;
-  ColPairArgs P;
-  P.n = n;
-  P.m = m;
-  P.half = m / 2;
-  P.A_in = A;
-  P.A_out = A;
-  P.V_out = V;
-  P.Ac = reinterpret_cast<float2*>(work);
-  P.Vc = reinterpret_cast<float2*>(work + 2 * n2);
-  P.pub = reinterpret_cast<float2*>(work + n2);
-  P.nrm2 = work + n2 + 4 * (long)m + 16;
-  P.red = work + 3 * n2;
-  P.bar = reinterpret_cast<unsigned*>(work + 3 * n2 + 2 * JMAX_BLOCKS);
-  P.status = status_dev;
-  P.max_sweeps = max_sweeps;
-  const size_t table = (sizeof(float4) + sizeof(int2)) * (size_t)P.half;
-  const size_t per_pair = 2 * sizeof(float2) * (size_t)n;
-  const size_t cap = 200 * 1024;
-  if (table + per_pair > cap || n2 < 4 * (long)m + 16 + n) return DSRG_FNO_ERR_UNSUPPORTED;
-  auto kern = jacobi_colpair_kernel;
-  int dev = 0, sms = 0;
-  DSRG_CUDA(cudaGetDevice(&dev));
-  DSRG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  // one block per SM: a round ends in a grid barrier whose arrivals are
-  // serialised atomics, so more blocks make every round slower; the pairs of
-  // a block are rotated together, as many at a time as shared memory holds
-  // (half the SMs when batch workers share the device: their solves overlap)
-  const int G = std::max(1, std::min(std::min(t_device_shared ? sms / 2 : sms, JMAX_BLOCKS), P.half));
-  P.cp = (P.half + G - 1) / G;
-  P.cpc = (int)std::max<size_t>(1, std::min<size_t>((size_t)P.cp, (cap - table) / per_pair));
-  const size_t smem = table + per_pair * (size_t)P.cpc;
-  if (smem > 48 * 1024) DSRG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap));
-  int occ = 0;
-  DSRG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, CPT, smem));
-  if (occ < 1) return DSRG_FNO_ERR_UNSUPPORTED;
-  const int grid = (P.half + P.cp - 1) / P.cp;
-  void* args[] = {&P};
-  DSRG_CUDA(cudaLaunchCooperativeKernel((const void*)kern, dim3(grid), dim3(CPT), args, smem, st));
-  DSRG_LAUNCH_CHECK();
-  int h[3] = {0, 0, 0};
-  DSRG_CUDA(cudaMemcpyAsync(h, status_dev, 3 * sizeof(int), cudaMemcpyDeviceToHost, st));
-  DSRG_CUDA(cudaStreamSynchronize(st));
-  prof_count(n >= 256 ? "eig_sweeps_large" : "eig_sweeps_small", (double)h[2]);
-  if (h[1]) return DSRG_FNO_ERR_TIMEOUT;
-  return h[0] ? DSRG_FNO_ERR_NOCONV : DSRG_FNO_OK;
-}
+static std::atomic<long long> g_spin_limit{BAR_SPIN_LIMIT};  // host copy of g_bar_spin_limit
 
 // Spin limit of the grid barrier on the current device; spins <= 0 restores
 // the default (test hook: a tiny limit makes the barrier's wait run out).
 int eig_set_barrier_limit(long long spins) {
   const long long v = spins > 0 ? spins : BAR_SPIN_LIMIT;
+  g_spin_limit.store(v);
   DSRG_CUDA(cudaMemcpyToSymbol(g_bar_spin_limit, &v, sizeof(v)));
   return DSRG_FNO_OK;
 }
@@ -761,6 +475,16 @@ int eig_sym_jacobi(int n, double* A, double* V, double* work, int* status_dev, i
   P.max_sweeps = max_sweeps;
   DSRG_CUDA(cudaMemsetAsync(P.bar, 0, 2 * sizeof(unsigned), st));
   DSRG_CUDA(cudaMemsetAsync(status_dev, 0, 4 * sizeof(int), st));
+  if (n >= EIG_DC_MIN_N && n <= EIG_DC_MAX_N && g_eig_dc.load()) {
+    // its barrier polls without naps: an eighth of the spins is about as long
+    const long long lim = std::max(1LL, g_spin_limit.load() / 8);
+    DSRG_TRY(eig_dc(n, A, V, work, P.bar, status_dev, lim, t_device_shared, st));
+    int h[2] = {0, 0};
+    DSRG_CUDA(cudaMemcpyAsync(h, status_dev, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
+    DSRG_CUDA(cudaStreamSynchronize(st));
+    if (h[1]) return DSRG_FNO_ERR_TIMEOUT;
+    return h[0] ? DSRG_FNO_ERR_NOCONV : DSRG_FNO_OK;
+  }
   if ((long)n * n >= (1L << 31)) return DSRG_FNO_ERR_UNSUPPORTED;  // 32-bit element offsets
   constexpr int SMEM_CEILING = 200 * 1024;
   // small matrices: one block with A, its copy and V in shared memory
@@ -768,12 +492,6 @@ int eig_sym_jacobi(int n, double* A, double* V, double* work, int* status_dev, i
   const size_t smem = in_smem ? sizeof(float4) * (size_t)m + 3 * sizeof(float2) * (size_t)n * n
                               : (sizeof(float4) + sizeof(int2)) * (size_t)(m / 2);
   if (smem > (size_t)SMEM_CEILING) return DSRG_FNO_ERR_UNSUPPORTED;
-  // (the column-pair kernel stages two columns of n per pair: above n of
-  // about 7000 it does not fit, and the round-parallel kernel takes the matrix)
-  if (!in_smem && g_eig_colpair.load()) {
-    const int rc = eig_colpair(n, m, A, V, work, status_dev, max_sweeps, st);
-    if (rc != DSRG_FNO_ERR_UNSUPPORTED) return rc;
-  }
   auto kern = in_smem ? jacobi_coop_kernel<true> : jacobi_coop_kernel<false>;
   // one fixed ceiling for every launch: concurrent callers (batch workers)
   // never lower it under one another

@@ -8,7 +8,7 @@
 // In the fast form both contractions run on the digit-plane kernel: W with
 // 5 planes (its entries are sums of nh np products), B' with 6 (B' enters
 // every integral, as the rotation to the frozen natural orbitals does);
-// the eigensolve is the double-float Jacobi solver of the natural orbitals.
+// the eigensolve is that of the natural orbitals.
 #include <math.h>
 
 #include <vector>
