@@ -33,11 +33,24 @@ DEFAULT_WORKLOAD = "sa_cas10_ncore60_nvir1200_naux3600"
 # 64 independent instances of ragged size (synth.problems.batch_sizes, seed 3)
 BATCH_WORKLOAD = "ragged_batch64_seed3"
 BATCH_CUT = 98.5
-PHASES = ("sliced_gemm_pair", "sliced_gemm_syrk", "sliced_gemm_plain", "phase_stage_b", "phase_pair_epilogue",
+PHASES = ("residue_gemm_pair", "residue_gemm_syrk", "residue_gemm_plain", "sliced_gemm_pair", "sliced_gemm_syrk",
+          "sliced_gemm_plain", "phase_stage_b", "phase_pair_epilogue",
           "phase_dress", "phase_stage_sig", "phase_small_terms", "phase_no_eigen", "phase_density_eigen",
           "phase_recanon_and_rotate")
 COUNTERS = ("eig_sweeps_large", "eig_sweeps_small")
 METRIC = "DSRG-PT2 D_vv+E2 solves/sec & GFLOP/s, fast vs FP64 GPU form at ≤1e-7 Eh"
+
+
+def gemm_query(pkg, kind):
+    """(ms, launches, executed flops) of the contraction kernel in one of its
+    modes (pair, syrk, plain): the residue form (5 planes) or digit planes."""
+    q = pkg.dsrg_fno_profile_query("residue_gemm_" + kind)
+    return q if q[1] else pkg.dsrg_fno_profile_query("sliced_gemm_" + kind)
+
+
+def dtype_of(nslices):
+    return ("bf16 residues modulo 10 coprimes -> exact f32 sums -> f64" if nslices in (0, 5) else
+            f"bf16 digit planes (k={nslices}) -> exact f32 level sums -> f64")
 
 
 def parse():
@@ -534,9 +547,9 @@ def main():
         _, n_c, total = pkg.dsrg_fno_profile_query(nm)
         phases[nm] = {"calls": n_c, "mean": total / max(n_c, 1)}
     ons_last = on.cpu().numpy()
-    pair_ms, pair_n, pair_fl = pkg.dsrg_fno_profile_query("sliced_gemm_pair")
-    syrk_ms, syrk_n, syrk_fl = pkg.dsrg_fno_profile_query("sliced_gemm_syrk")
-    plain_ms, plain_n, plain_fl = pkg.dsrg_fno_profile_query("sliced_gemm_plain")
+    pair_ms, pair_n, pair_fl = gemm_query(pkg, "pair")
+    syrk_ms, syrk_n, syrk_fl = gemm_query(pkg, "syrk")
+    plain_ms, plain_n, plain_fl = gemm_query(pkg, "plain")
     ms_max = max_over_ranks(ms, dist, dev)
     value = replica_rate(args.steps, world, ms_max)
     flops = algorithmic_flops(p)
@@ -632,7 +645,7 @@ def main():
     line = {
         "metric": METRIC, "value": value, "unit": "solves/s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_max / args.steps, "higher_is_better": True, "scaling": "weak",
-        "vs_baseline": None, "dtype": f"bf16 digit planes (k={args.nslices}) -> exact f32 level sums -> f64",
+        "vs_baseline": None, "dtype": dtype_of(args.nslices),
         "data": "synthetic",
         "config": dict(single_config(p, args.workload, cuts, args.nslices),
                        epilogue="fused" if args.fused_epilogue else "separate kernel"),
@@ -661,7 +674,7 @@ def main():
 def mr_energy_timing(pkg, p, gp, dev, steps=2):
     """The full second-order energy over every amplitude class
     (dsrg_fno_pt2_energy_mr) on the headline workload, with a seeded synthetic
-    3-cumulant: E_vv on the digit-plane path, the rest (doubles with an active
+    3-cumulant: E_vv on the tensor-core path, the rest (doubles with an active
     particle, singles, cumulant couplings) in float64; timed beside E_vv alone.
     rest_gemm_flops: the float64 integral GEMM of the rest, 2 nh np nh nact naux."""
     import torch
@@ -682,13 +695,13 @@ def mr_energy_timing(pkg, p, gp, dev, steps=2):
 
     s_full, (e2, evv) = timed(lambda: pkg.dsrg_fno_pt2_energy_mr(gp, l3))
     s_vv, _ = timed(lambda: pkg.dsrg_fno_pt2_energy(gp))
-    # phases of one more call: the integral GEMM (digit planes) and the element stages of the rest
+    # phases of one more call: the integral GEMM and the element stages of the rest
     pkg.dsrg_fno_profile_enable(True)
     pkg.dsrg_fno_pt2_energy_mr(gp, l3)
     torch.cuda.synchronize()
     pkg.dsrg_fno_profile_enable(False)
     ph = {nm: pkg.dsrg_fno_profile_query(nm)[0] / 1e3 for nm in ("phase_mr_integrals", "phase_mr_terms")}
-    g_ms, _, g_fl = pkg.dsrg_fno_profile_query("sliced_gemm_plain")
+    g_ms, _, g_fl = gemm_query(pkg, "plain")
     flops = 2.0 * p.nh * p.np_ * p.nh * p.nact * p.naux
     return {"s_full": s_full, "s_vv_only": s_vv, "s_rest": s_full - s_vv, "e2": e2, "e_vv": evv,
             "e_rest": e2 - evv, "lambda3": "seeded synthetic 3-cumulant (scale 0.03)", "steps": steps,
@@ -888,19 +901,22 @@ PEAKS_OWN = {"fp64_dgemm_tflops": 1.0988, "tf32_tflops": 1027.07}
 
 def roofline_of(pair_ms, pair_n, pair_fl, syrk, plain, step_ms, workload=None, alg_flops=None, nslices=5):
     """Roofline of the pair contraction (the dominant kernel).  `frac` counts
-    the algorithmic pair flops times the k(k+1)/2 digit products of k planes
-    (no tile padding); `frac_executed` the flops the tensor cores executed
-    (every 128 x N tile in full, K padded to 64)."""
+    the algorithmic pair flops times the products the form takes (10 moduli in
+    the residue form of 5 planes, k(k+1)/2 digit products of k = 3, 4 planes; no
+    tile padding); `frac_executed` the flops the tensor cores executed
+    (whole output tiles, K padded to 64)."""
     peaks, peak_kind = measured_peaks()
     peak = peaks.get("bf16_tflops_sustained", peaks.get("bf16_tflops"))
     achieved_exec = (pair_fl / (pair_ms / 1e3) / 1e12) if pair_ms > 0 else None
-    prods = nslices * (nslices + 1) / 2
+    residue = nslices in (0, 5)
+    prods = 10 if residue else nslices * (nslices + 1) / 2
     achieved = (alg_flops * prods / (pair_ms / 1e3) / 1e12) if (pair_ms > 0 and alg_flops) else None
     tf = lambda q: (q[2] / (q[0] / 1e3) / 1e12) if q[0] > 0 else None  # noqa: E731
-    return {"bound": "tensor", "kernel": "sliced_gemm_kernel (pair contraction, tcgen05 bf16 digit planes)",
+    return {"bound": "tensor", "kernel": ("residue_gemm_kernel (pair contraction, tcgen05 modulo 10 coprimes)" if residue else
+                                           "sliced_gemm_kernel (pair contraction, tcgen05 bf16 digit planes)"),
             "achieved": achieved, "peak": peak, "peak_kind": f"bf16 dense sustained, {peak_kind}",
             "unit": "TFLOP/s", "frac": (achieved / peak) if achieved else None,
-            "count": f"algorithmic pair flops (2 naux nv^2 per hole pair i <= j) x {prods:.0f} digit products",
+            "count": f"algorithmic pair flops (2 naux nv^2 per hole pair i <= j) x {prods:.0f} products",
             "achieved_executed": achieved_exec, "frac_executed": (achieved_exec / peak) if achieved_exec else None,
             "padding": (pair_fl / (alg_flops * prods)) if alg_flops else None,
             "traffic": traffic_per_launch(workload, pair_fl / max(pair_n, 1)) if pair_n else None,
@@ -976,7 +992,7 @@ def batch_arm(args):
         step(gps)
     barrier()
     pkg.dsrg_fno_profile_enable(False)
-    q = {nm: pkg.dsrg_fno_profile_query(nm) for nm in ("sliced_gemm_pair", "sliced_gemm_syrk", "sliced_gemm_plain")}
+    q = {nm: gemm_query(pkg, nm) for nm in ("pair", "syrk", "plain")}
     # stream time per step summed over the concurrent workers
     phases = {}
     for nm in PHASES:
@@ -1061,13 +1077,13 @@ def batch_arm(args):
                                     "nkept_equal": all(a["nkept"] == b["nkept"] for a, b in zip(rf, r64))}}
 
     alg = sum(pair_alg_flops(pp, [r["nkept"]]) for pp, r in zip(probs, res)) * args.steps
-    roofline = roofline_of(*q["sliced_gemm_pair"], q["sliced_gemm_syrk"], q["sliced_gemm_plain"], ms,
+    roofline = roofline_of(*q["pair"], q["syrk"], q["plain"], ms,
                            alg_flops=alg, nslices=args.nslices)
     roofline["note"] = "kernel times from a second, profiled run of the same steps"
     line = {
         "metric": METRIC, "value": value, "unit": "instances/s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_max / args.steps, "higher_is_better": True, "scaling": "weak",
-        "vs_baseline": None, "dtype": f"bf16 digit planes (k={args.nslices}) -> exact f32 level sums -> f64",
+        "vs_baseline": None, "dtype": dtype_of(args.nslices),
         "data": "synthetic",
         "config": batch_config(args.nslices),
         "workers": workers,

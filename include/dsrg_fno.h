@@ -49,10 +49,14 @@ typedef enum {
 } dsrg_fno_status;
 
 /* Arithmetic of the integral contractions.  FP64: plain float64 on the CUDA
- * cores.  SLICED_BF16: each float64 row is split into `nslices` exact bfloat16
- * digit planes with a per-row power-of-two scale; digit products run on the
- * tensor cores (tcgen05) with exact float32 level sums, merged into
- * double-float accumulators (float32 hi + lo pairs, about 48 bits); the
+ * cores.  SLICED_BF16: each float64 row becomes integers with a per-row
+ * power-of-two scale, whose products run on the tensor cores (tcgen05) with
+ * exact float32 sums.  With 5 planes (the default) the pair contractions are
+ * formed modulo 10 coprime numbers (residue form, rows scaled to a 2-norm of
+ * 2^44) and put together by the Chinese remainder theorem; otherwise the
+ * integers are split into `nslices` exact bfloat16 digit planes, whose level
+ * sums are merged into double-float accumulators (float32 hi + lo pairs, about
+ * 48 bits); the
  * regulariser and the dressing of this form run in double-float, the energy
  * and D_vv sums in float64.  In both forms the NO eigensolve runs in float64
  * (double-float below 33 rows).  On the workloads here the two forms agree to a few 1e-9 E_h

@@ -69,8 +69,10 @@ int dsrg_fno_debug_set_barrier_limit(int64_t spins);
 
 /* on != 0: the fast form's Eq. A7 regulariser runs in the output stage of
  * the pair-contraction kernel; 0 (the default, faster on GB300): in a
- * separate kernel over the stored contraction tiles.  Affects later calls of
- * this process. */
+ * separate kernel over the stored contraction tiles.  The digit forms of 3 and
+ * 4 planes and the literal forms only: with 5 planes the kernel that puts the
+ * residues together applies the regulariser.  Affects later calls of this
+ * process. */
 int dsrg_fno_debug_set_fused_epilogue(int32_t on);
 
 /* Digit planes of the dressed matrices in the fast form's rank-K update of

@@ -58,6 +58,7 @@ struct Plan {
   std::vector<DressDesc> desc;
   std::vector<Batch> batches;
   int max_pairs = 0, max_desc = 0, max_out = 0;
+  int res_cap = 0;  // residue form: output tiles whose residues are held at a time
 };
 
 static void build_plan(int nc, int na, long cap_pairs, Plan& P) {
@@ -202,6 +203,9 @@ struct PassBuffers {
   float2* hp;        // [nh np] eps_i - eps_a, double-float (fused epilogue)
   const RegTables* reg;
   bool fused;        // Eq. A7 epilogue inside the contraction kernel
+  bool residue;      // B.B contraction in the residue form
+  uint16_t* res;     // residues of res_cap output tiles
+  int res_cap;
   int2* tiles;       // output tiles of the pair contraction, all batches
   int* slot_of;      // [batch][nh][nh] slot of pair (i, j) in the batch, -1 outside
   std::vector<long> tile_begin;
@@ -255,10 +259,18 @@ static int2 pair_form_of(const dsrg_fno_problem* p, int ks) {
 
 static size_t doubles(size_t n) { return ws_bytes(n, sizeof(double)); }
 
-static long pair_cap_for_budget(int nv, int np, int ks, size_t budget) {
-  // tau + kappa + two dressed matrices per pair (+ nu and the dressed planes in the fast form)
+// The B.B contraction of five planes runs in the residue form (10 products
+// instead of 15 and no dropped ones); 3 and 4 planes stay digit planes.
+static bool residue_form(int ks, int2 pform) { return ks == 5 && pform.x == FORM_DIGITS; }
+static int pair_tile_rows(int ks, int2 pform) { return residue_form(ks, pform) ? RES_TILE : PAIR_TILE_M; }
+static int pair_tile_cols(int ks, int2 pform) {
+  return residue_form(ks, pform) ? RES_TILE : pair_tile_n(pform.x, pform.y);
+}
+
+static long pair_cap_for_budget(int nv, int np, int ks, bool residue, size_t budget) {
+  // tau + kappa + two dressed matrices per pair (+ the dressed planes and, outside the residue form, nu in the fast form)
   double per_pair = 4.0 * (double)nv * nv * 8.0 + 1024.0;
-  if (ks) per_pair += (double)np * np * 8.0 + 2.0 * ks * 2.0 * (double)nv * (nv + 64);
+  if (ks) per_pair += (residue ? 0.0 : (double)np * np * 8.0) + 2.0 * ks * 2.0 * (double)nv * (nv + 64);
   long cap = (long)(budget / per_pair);
   return std::max<long>(cap, 1);
 }
@@ -277,6 +289,22 @@ size_t device_budget(size_t held) {
 }
 
 static size_t plan_budget(const Workspace& ws) { return device_budget(ws.cap); }
+
+// Batches of pairs that fit the budget.  The residues of 4096 output tiles (5.4
+// GB, 54 rounds of units on 76 pairs of SMs) lose nothing to the launches' last
+// rounds; a small budget holds an eighth of itself, at least 64 tiles.
+static void make_plan(const Geometry& g, int ks, int2 pform, size_t budget, Plan& P) {
+  const bool rf = residue_form(ks, pform);
+  const size_t tile = residue_tile_bytes(RES_MOD);
+  if (rf) P.res_cap = (int)std::max<size_t>(64, std::min<size_t>(4096, budget / 8 / tile));
+  const size_t held = rf ? std::min(budget / 8, (size_t)P.res_cap * tile) : 0;
+  build_plan(g.nc, g.na, pair_cap_for_budget(g.nv, g.np, ks, rf, budget - held), P);
+  if (rf) {
+    int most = 1;
+    for (const Batch& b : P.batches) most = std::max(most, pair_tile_bound(RES_TILE, RES_TILE, g, b.npairs));
+    P.res_cap = std::min(P.res_cap, most);
+  }
+}
 
 static int run_pass(const Geometry& g, const double* B, const double* eps, const double* gamma1,
                     const double* lambda2, const Plan& P, PassBuffers& W, bool want_d, double* D,
@@ -306,17 +334,23 @@ static int run_pass(const Geometry& g, const double* B, const double* eps, const
     // digit planes of B: rows (hole, particle), contraction over Q
     const long rows = (long)g.nh * g.np;
     DSRG_PHASE("phase_stage_b", st);
-    if (W.pform.x == FORM_DIGITS)
+    if (W.residue)
+      DSRG_TRY(residue_stage(RES_MOD, B, rows, g.nq, 1, rows, W.kpad_q, W.planes_b, W.exps_b, st));
+    else if (W.pform.x == FORM_DIGITS)
       DSRG_TRY(slice_rows(W.ks, B, rows, g.nq, 1, rows, W.kpad_q, W.planes_b, W.exps_b, st));
     else
       DSRG_TRY(stage_literal(W.pform.x, W.pform.y, B, rows, g.nq, 1, rows, W.kpad_q, W.planes_b, W.exps_b, st));
     DSRG_TRY(eps_to_dd(g.nh + g.nv, eps, W.eps_dd, st));
-    if (W.fused) DSRG_TRY(hole_particle_dd(g, eps, W.hp, st));
+    if (W.fused || W.residue) DSRG_TRY(hole_particle_dd(g, eps, W.hp, st));
   }
   for (size_t bi = 0; bi < P.batches.size(); ++bi) {
     const Batch& b = P.batches[bi];
     double* ts = want_d ? W.ts : nullptr;
-    if (W.ks && W.fused) {
+    if (W.residue) {
+      DSRG_TRY(residue_pair(g, W.planes_b, W.exps_b, W.kpad_q, W.tiles + W.tile_begin[bi], W.tile_count[bi],
+                            W.slot_of + bi * (size_t)g.nh * g.nh, W.hp, W.res, W.res_cap, as_dd(W.tau), as_dd(W.kap), ts,
+                            W.err, st));
+    } else if (W.ks && W.fused) {
       PairEpilogue epi{};
       epi.hp = W.hp;
       epi.reg = W.reg;
@@ -421,16 +455,18 @@ static size_t pass_bytes(const Geometry& g, const Plan& P, bool want_d, int nspl
   b += ws_bytes(16, sizeof(int));
   if (ks) {
     const size_t rows = (size_t)g.nh * g.np;
-    b += ws_bytes((size_t)ks * rows * pad64(g.nq), 2) + ws_bytes(rows, sizeof(int));
-    b += doubles((size_t)P.max_pairs * g.np * g.np);
+    const bool rf = residue_form(ks, pform);
+    b += ws_bytes((size_t)(rf ? RES_MOD : ks) * rows * pad64(g.nq), 2) +
+         (rf ? residue_exps_bytes(rows) : ws_bytes(rows, sizeof(int)));
+    b += rf ? ws_bytes(P.res_cap * residue_tile_bytes(RES_MOD), 1) : doubles((size_t)P.max_pairs * g.np * g.np);
     b += doubles((size_t)g.nh + g.nv);
     b += doubles((size_t)g.nh * g.np);
     if (want_d)
       b += ws_bytes((size_t)ks * P.max_out * g.nv * pad64(g.nv), 2) + 2 * ws_bytes((size_t)P.max_out * g.nv, sizeof(int));
     b += ws_bytes(8, sizeof(int));
     size_t tiles = 0;
-    const int bn = pair_tile_n(pform.x, pform.y);
-    for (const Batch& bt : P.batches) tiles += (size_t)pair_tile_bound(bn, g, bt.npairs);
+    const int bm = pair_tile_rows(ks, pform), bn = pair_tile_cols(ks, pform);
+    for (const Batch& bt : P.batches) tiles += (size_t)pair_tile_bound(bm, bn, g, bt.npairs);
     b += ws_bytes(tiles + 1, sizeof(int2)) + ws_bytes(P.batches.size() * (size_t)g.nh * g.nh + 1, sizeof(int));
   }
   return b;
@@ -471,12 +507,19 @@ static int carve_pass(Workspace& ws, const Geometry& g, const Plan& P, bool want
     const size_t rows = (size_t)g.nh * g.np;
     W.kpad_q = pad64(g.nq);
     W.kpad_v = pad64(g.nv);
-    W.planes_b = ws_take<__nv_bfloat16>(ws, (size_t)ks * rows * W.kpad_q);
-    W.exps_b = ws_take<int>(ws, rows);
-    W.nu = ws_take<float2>(ws, (size_t)P.max_pairs * g.np * g.np);
+    W.residue = residue_form(ks, pform);
+    W.planes_b = ws_take<__nv_bfloat16>(ws, (size_t)(W.residue ? RES_MOD : ks) * rows * W.kpad_q);
+    if (W.residue) {
+      W.exps_b = reinterpret_cast<int*>(ws_take<char>(ws, residue_exps_bytes(rows)));
+      W.res = reinterpret_cast<uint16_t*>(ws_take<char>(ws, P.res_cap * residue_tile_bytes(RES_MOD)));
+      W.res_cap = P.res_cap;
+    } else {
+      W.exps_b = ws_take<int>(ws, rows);
+      W.nu = ws_take<float2>(ws, (size_t)P.max_pairs * g.np * g.np);
+    }
     W.eps_dd = ws_take<float2>(ws, (size_t)g.nh + g.nv);
     W.hp = ws_take<float2>(ws, (size_t)g.nh * g.np);
-    W.fused = fused_epilogue_enabled();
+    W.fused = !W.residue && fused_epilogue_enabled();
     if (W.fused) DSRG_TRY(reg_tables_device(&W.reg));
     if (want_d) {
       W.planes_s = ws_take<__nv_bfloat16>(ws, (size_t)ks * P.max_out * g.nv * W.kpad_v);
@@ -490,11 +533,11 @@ static int carve_pass(Workspace& ws, const Geometry& g, const Plan& P, bool want
     std::vector<int2> all, one;
     std::vector<int> slots(P.batches.size() * (size_t)g.nh * g.nh, -1);
     size_t bound = 0;
-    const int bn = pair_tile_n(pform.x, pform.y);
+    const int bm = pair_tile_rows(ks, pform), bn = pair_tile_cols(ks, pform);
     for (size_t bi = 0; bi < P.batches.size(); ++bi) {
       const Batch& b = P.batches[bi];
-      bound += (size_t)pair_tile_bound(bn, g, b.npairs);
-      DSRG_TRY(pair_tiles(bn, g, P.pairs.data() + b.pair_begin, b.npairs, !want_d, one));
+      bound += (size_t)pair_tile_bound(bm, bn, g, b.npairs);
+      DSRG_TRY(pair_tiles(bm, bn, g, P.pairs.data() + b.pair_begin, b.npairs, !want_d, one));
       W.tile_begin.push_back((long)all.size());
       W.tile_count.push_back((int)one.size());
       all.insert(all.end(), one.begin(), one.end());
@@ -545,7 +588,7 @@ static int energy_pass(const Geometry& g, int ks, int2 pform, const double* B, c
                        const double* lambda2, Workspace& ws, size_t base_off, size_t budget, double* e_out,
                        cudaStream_t st) {
   Plan P;
-  build_plan(g.nc, g.na, pair_cap_for_budget(g.nv, g.np, ks, budget), P);
+  make_plan(g, ks, pform, budget, P);
   ws.off = base_off;
   PassBuffers W{};
   size_t need = base_off + pass_bytes(g, P, false, 1, ks, pform);
@@ -559,7 +602,7 @@ static int energy_pass(const Geometry& g, int ks, int2 pform, const double* B, c
 
 static size_t energy_pass_bytes(const Geometry& g, int ks, int2 pform, size_t budget) {
   Plan P;
-  build_plan(g.nc, g.na, pair_cap_for_budget(g.nv, g.np, ks, budget), P);
+  make_plan(g, ks, pform, budget, P);
   return pass_bytes(g, P, false, 1, ks, pform);
 }
 
@@ -622,8 +665,9 @@ int impl_vv_opdm(Workspace& ws, size_t budget, const dsrg_fno_problem* prob, dou
   if (l3 && !is_device_ptr(l3)) return DSRG_FNO_ERR_ARG;
   const Geometry g = geometry_of(prob);
   const int ks = slices_of(prob);
+  const int2 pform = pair_form_of(prob, ks);
   Plan P;
-  build_plan(g.nc, g.na, pair_cap_for_budget(g.nv, g.np, ks, budget), P);
+  make_plan(g, ks, pform, budget, P);
   const int nsplit = nsplit_for(g.nv, P.max_out, ks ? syrk_slices(ks) : 0);
   const size_t small = small_terms_work_doubles(g.nc, g.na, g.nv);
   const int kmax = small_terms_kmax(g.nc, g.na);
@@ -632,7 +676,6 @@ int impl_vv_opdm(Workspace& ws, size_t budget, const dsrg_fno_problem* prob, dou
       small_fast ? ws_bytes(2 * (size_t)ks * g.nv * pad64(kmax), 2) + ws_bytes(2 * (size_t)g.nv, sizeof(int)) +
                        doubles((size_t)g.nv * g.nv) + ws_bytes(8, sizeof(int))
                  : 0;
-  const int2 pform = pair_form_of(prob, ks);
   size_t need = ws_bytes(8, sizeof(int)) + pass_bytes(g, P, true, nsplit, ks, pform) + doubles((size_t)g.nh * g.nv) +
                 doubles(small + 1) + small_fast_bytes;
   DSRG_TRY(ws_reserve(ws, need));

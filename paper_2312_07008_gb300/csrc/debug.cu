@@ -165,8 +165,8 @@ extern "C" int dsrg_fno_debug_pair_tiles(int32_t nslices, int32_t ncore, int32_t
     if (pr[k].x < 0 || pr[k].y < pr[k].x || pr[k].y >= g.nh) return DSRG_FNO_ERR_ARG;
   }
   const int bn = pair_tile_n(FORM_DIGITS, nslices);
-  DSRG_TRY(pair_tiles(bn, g, pr.data(), npairs, energy_only != 0, out));
-  if ((long)out.size() > max_tiles || (long)out.size() > pair_tile_bound(bn, g, npairs)) return DSRG_FNO_ERR_ARG;
+  DSRG_TRY(pair_tiles(PAIR_TILE_M, bn, g, pr.data(), npairs, energy_only != 0, out));
+  if ((long)out.size() > max_tiles || (long)out.size() > pair_tile_bound(PAIR_TILE_M, bn, g, npairs)) return DSRG_FNO_ERR_ARG;
   for (size_t t = 0; t < out.size(); ++t) {
     tiles[2 * t] = out[t].x;
     tiles[2 * t + 1] = out[t].y;

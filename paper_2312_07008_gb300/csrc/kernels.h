@@ -136,8 +136,10 @@ int slice_rows_dd(int KS, const float2* src, long R, int K, long rs, long ks, in
 enum { FORM_DIGITS = 0, FORM_BF16X3 = 1, FORM_TF32 = 2, FORM_DIGITS_T = 3 };
 // N of the 128 x N output tiles of a form (KS: digit planes or literal parts)
 int pair_tile_n(int form, int KS);
-int pair_tile_bound(int BN, const Geometry& g, int npairs);
-int pair_tiles(int BN, const Geometry& g, const int2* pairs, int npairs, bool energy_only, std::vector<int2>& out);
+// (BM x BN tiles; BM = PAIR_TILE_M in the digit and literal forms, RES_TILE in the residue form)
+constexpr int PAIR_TILE_M = 128;
+int pair_tile_bound(int BM, int BN, const Geometry& g, int npairs);
+int pair_tiles(int BM, int BN, const Geometry& g, const int2* pairs, int npairs, bool energy_only, std::vector<int2>& out);
 struct RegTables;
 // Eq. A7 epilogue fused into the pair contraction (see sliced.cu)
 struct PairEpilogue {
@@ -158,6 +160,28 @@ int sliced_pair_gemm(int KS, int form, const Geometry& g, const void* planes, co
 // float32 holding tf32 values for FORM_TF32), exps[R] = 0
 int stage_literal(int form, int KS, const double* src, long R, int K, long rs, long ks, int Kpad, void* planes,
                   int* exps, cudaStream_t st);
+// Residue form (residue.cu): the fast form's contractions modulo RES_MOD (or,
+// for the rotation of B, RES_MOD_X) coprime moduli on tcgen05, one product each.
+constexpr int RES_MOD = 10, RES_MOD_X = 12;
+constexpr int RES_TILE = 256;          // rows and columns of an output tile
+constexpr int RES_STAGE_BLOCKS = 608;  // four blocks per SM of a staging launch
+// bytes of the exponents of R staged rows and of the staging's scratch behind them
+size_t residue_exps_bytes(size_t R);
+// planes [nm][R][Kpad], exps [R] (residue_exps_bytes); arguments as slice_rows
+int residue_stage(int nm, const double* src, long R, int K, long rs, long ks, int Kpad, __nv_bfloat16* planes, int* exps,
+                  cudaStream_t st);
+size_t residue_tile_bytes(int nm);  // residues of one output tile
+// hp: hole_particle_dd; res: cap tiles of residues
+int residue_pair(const Geometry& g, const __nv_bfloat16* planes, const int* exps, int Kpad, const int2* tiles, int ntiles,
+                 const int* slot_of, const float2* hp, uint16_t* res, int cap, float2* tau, float2* kap, double* ts,
+                 int* err, cudaStream_t st);
+// Matrices [r0, r1) of a rank-K update that share their row scales; sign 0: all
+// of them, +-1: those of that sign.
+constexpr int RES_MAX_SEGMENTS = 64;
+struct ResSegment {
+  int r0, r1, sign, scale;  // scale: index of the range's row exponents
+};
+void* tensor_map_encoder();  // cuTensorMapEncodeTiled, or null
 // double-float elementwise stages (dd_stages.cu)
 int eps_to_dd(int n, const double* eps, float2* out, cudaStream_t st);
 int reg_tables_device(const RegTables** out);

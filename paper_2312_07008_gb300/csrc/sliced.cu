@@ -1,5 +1,7 @@
-// Fast form of the contractions: exact bfloat16 digit planes on the tcgen05
-// tensor cores (the planes are staged by stage.cu).
+// Contractions by exact bfloat16 digit planes on the tcgen05 tensor cores (the
+// planes are staged by stage.cu): the fast form with 3 or 4 planes, and the
+// literal forms of the precision study.  With 5 planes the residue form
+// (residue.cu) takes the pair contraction.
 //
 // Products.  For two rows a, b:  x_a . x_b = 2^-14 sum_L 2^-8L S_L with the
 // level sums S_L = sum_{s+t=L} sum_k d_s(a,k) d_t(b,k).  Only levels
@@ -31,7 +33,7 @@ namespace dsrg {
 
 namespace {
 
-constexpr int BM = 128;
+constexpr int BM = PAIR_TILE_M;
 constexpr int BKE = 64;            // k elements per block (128 bytes of bf16, 128-byte swizzle)
 constexpr int ROW_BYTES = 2 * BKE;
 constexpr int KCHUNK_BLOCKS = 320 / BKE;  // 320 k-values per exact sum of levels 0, 1, 2
@@ -683,6 +685,8 @@ int tile_n_for(int KS) { return KS == 6 ? 32 : (KS == 5 ? 48 : 64); }
 
 }  // namespace
 
+void* tensor_map_encoder() { return reinterpret_cast<void*>(encode_fn()); }
+
 // ------------------------------------------------------------ public (lib)
 // Output tiles of the pair contraction for one batch of hole pairs (i <= j).
 // The rows of all holes form one (nh np)-row operand, so tiles run across the
@@ -696,11 +700,11 @@ static constexpr int ROW_BAND = 8;
 
 int pair_tile_n(int form, int KS) { return form == FORM_DIGITS ? tile_n_for(KS) : 64; }
 
-int pair_tile_bound(int BN, const Geometry& g, int npairs) {
+int pair_tile_bound(int BM, int BN, const Geometry& g, int npairs) {
   return npairs * (ceil_div(g.np, BM) + 1) * (ceil_div(g.np, BN) + 1);
 }
 
-int pair_tiles(int BN, const Geometry& g, const int2* pairs, int npairs, bool energy_only, std::vector<int2>& out) {
+int pair_tiles(int BM, int BN, const Geometry& g, const int2* pairs, int npairs, bool energy_only, std::vector<int2>& out) {
   out.clear();
   if (npairs <= 0) return DSRG_FNO_OK;
   const long np = g.np, na = g.na;
