@@ -51,9 +51,9 @@ typedef enum {
 /* Arithmetic of the integral contractions.  FP64: plain float64 on the CUDA
  * cores.  SLICED_BF16: each float64 row becomes integers with a per-row
  * power-of-two scale, whose products run on the tensor cores (tcgen05) with
- * exact float32 sums.  With 5 planes (the default) the pair contractions are
- * formed modulo 10 coprime numbers (residue form, rows scaled to a 2-norm of
- * 2^44) and put together by the Chinese remainder theorem; otherwise the
+ * exact float32 sums.  With 5 planes (the default) the contractions are formed
+ * modulo 10 coprime numbers (residue form, rows scaled to a 2-norm of 2^44) and
+ * put together by the Chinese remainder theorem; otherwise the
  * integers are split into `nslices` exact bfloat16 digit planes, whose level
  * sums are merged into double-float accumulators (float32 hi + lo pairs, about
  * 48 bits); the
@@ -126,7 +126,7 @@ int dsrg_fno_pt2_energy(const dsrg_fno_problem* prob, double* e2_out, void* stre
  * with an active particle, the singles, their cumulant couplings) in float64,
  * except that outside the FP64 form its integrals <ay|ij> (one contraction
  * over the auxiliary index, rows (i, a) against (j, y), y active) run on the
- * digit-plane tensor-core path when naux >= 256.
+ * tensor-core path when naux >= 256.
  * In the single-reference limit (nact = 0) E^(2) = E_vv plus the singles of
  * f_hp.  Errors as for dsrg_fno_pt2_energy; a host lambda3 gives
  * DSRG_FNO_ERR_ARG, a non-finite one DSRG_FNO_ERR_NONFINITE.  Device
@@ -155,7 +155,7 @@ int dsrg_fno_vv_opdm(const dsrg_fno_problem* prob, double* dvv_out, double* e2_o
  *   Other arguments, outputs and errors as for dsrg_fno_vv_opdm; a non-finite
  *   lambda3 gives DSRG_FNO_ERR_NONFINITE.  The term is formed in float64 in
  *   both precisions; with SLICED_BF16 its final contraction (length nact^3,
- *   when >= 256) runs on the digit-plane tensor-core path like terms 10-12. */
+ *   when >= 256) runs on the tensor-core path like terms 10-12. */
 int dsrg_fno_vv_opdm_lambda3(const dsrg_fno_problem* prob, const double* lambda3, double* dvv_out,
                              double* e2_out, void* stream);
 
@@ -246,7 +246,7 @@ int dsrg_fno_truncate_noalloc(int32_t nvir, const double* dvv, int32_t mode, dou
  *   B_vv       device [naux][nv][nv]: B^Q_{ab}, virtual-virtual DF factors in
  *              that basis (e.g. rotated to the recanonicalised kept NOs).
  *   T          device [npairs][nv][nv]: T[p][c][d] = T^{ij}_{cd} of hole pair p.
- *   precision  DSRG_FNO_FP64 or DSRG_FNO_SLICED_BF16 (5 digit planes).
+ *   precision  DSRG_FNO_FP64 or DSRG_FNO_SLICED_BF16 (residue form, 10 moduli).
  *   C_out      device [npairs][nv][nv].
  * The 4-index integrals are formed for 16 values of a at a time and never
  * stored whole.  Errors: DSRG_FNO_ERR_ARG for bad sizes, null or host
@@ -266,8 +266,8 @@ int dsrg_fno_ladder(int32_t nv, int32_t naux, const double* B_vv, int32_t npairs
  *   nh, np     holes (ncore + nact) and particles (nact + nvir).
  *   B_hp       device [naux][nh][np], as in dsrg_fno_problem.
  *   threshold  absolute eigenvalue threshold (w > threshold kept).
- *   precision  DSRG_FNO_FP64, or DSRG_FNO_SLICED_BF16 (digit-plane
- *              contractions: 5 planes for W, 6 for B'); the eigensolve is the
+ *   precision  DSRG_FNO_FP64, or DSRG_FNO_SLICED_BF16 (residue form: 10
+ *              moduli for W, 12 for B'); the eigensolve is the
  *              same in both.
  *   B_out      device [naux][nh][np], caller-allocated: its first naux'
  *              slices receive B' (the rest is left untouched).

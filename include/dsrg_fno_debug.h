@@ -14,11 +14,16 @@ extern "C" {
 #endif
 
 /* C[M][N] = A[M][K] B[N][K]^T with the exact bf16 digit-plane GEMM on the
- * tensor cores (nslices planes, 3..6; 6 is the configuration the library
- * uses for the rotation of B to the frozen natural orbitals).  All arrays are host float64,
- * row-major.  This is the contraction kernel of the fast form by itself. */
+ * tensor cores (nslices planes, 3..6).  All arrays are host float64, row-major.
+ * This is the contraction kernel of the digit-plane forms by itself. */
 int dsrg_fno_debug_sliced_gemm(int32_t nslices, int32_t M, int32_t N, int32_t K, const double* A,
                                const double* B, double* C);
+
+/* C[M][N] = A[M][K] B[N][K]^T in the residue form (nmod 10 or 12 coprime
+ * moduli), the contraction of the fast form with 5 planes by itself.  Host
+ * float64 arrays, row-major. */
+int dsrg_fno_debug_residue_gemm(int32_t nmod, int32_t M, int32_t N, int32_t K, const double* A, const double* B,
+                                double* C);
 
 /* C[M][N] = A[M][K] B[N][K]^T in a literal form of the precision study
  * (precision DSRG_FNO_BF16X3, nterms 0 or 3; DSRG_FNO_TF32, nterms 1 or 3,

@@ -34,6 +34,7 @@ EXPORTED = (
     "dsrg_fno_release",
     "dsrg_fno_debug_sliced_gemm",
     "dsrg_fno_debug_literal_gemm",
+    "dsrg_fno_debug_residue_gemm",
     "dsrg_fno_debug_slice_rows",
     "dsrg_fno_debug_slice_rows_dd",
     "dsrg_fno_debug_regularizer",
@@ -126,6 +127,8 @@ def load(path: str = LIB_PATH):
     lib.dsrg_fno_debug_sliced_gemm.argtypes = [i32, i32, i32, i32, dp, dp, dp]
     lib.dsrg_fno_debug_literal_gemm.argtypes = [i32, i32, i32, i32, i32, dp, dp, dp]
     lib.dsrg_fno_debug_literal_gemm.restype = ctypes.c_int
+    lib.dsrg_fno_debug_residue_gemm.argtypes = [i32, i32, i32, i32, dp, dp, dp]
+    lib.dsrg_fno_debug_residue_gemm.restype = ctypes.c_int
     lib.dsrg_fno_debug_slice_rows.argtypes = [i32, i32, i32, dp, ctypes.POINTER(ctypes.c_float),
                                               ctypes.POINTER(i32)]
     lib.dsrg_fno_debug_slice_rows_dd.argtypes = [i32, i32, i32, ctypes.POINTER(ctypes.c_float),

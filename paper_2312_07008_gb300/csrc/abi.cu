@@ -672,10 +672,12 @@ int impl_vv_opdm(Workspace& ws, size_t budget, const dsrg_fno_problem* prob, dou
   const size_t small = small_terms_work_doubles(g.nc, g.na, g.nv);
   const int kmax = small_terms_kmax(g.nc, g.na);
   const bool small_fast = ks > 0 && kmax >= SLICED_MIN_K;
-  const size_t small_fast_bytes =
-      small_fast ? ws_bytes(2 * (size_t)ks * g.nv * pad64(kmax), 2) + ws_bytes(2 * (size_t)g.nv, sizeof(int)) +
-                       doubles((size_t)g.nv * g.nv) + ws_bytes(8, sizeof(int))
-                 : 0;
+  const bool small_res = small_fast && ks == 5;  // residue form
+  const size_t small_planes = 2 * (size_t)(small_res ? RES_MOD : ks) * g.nv * pad64(kmax);
+  const size_t small_exps = small_res ? residue_exps_bytes(g.nv) : ws_bytes(g.nv, sizeof(int));
+  const size_t small_out =
+      small_res ? ws_bytes(residue_plain_bytes(RES_MOD, g.nv, g.nv), 1) : doubles((size_t)g.nv * g.nv);
+  const size_t small_fast_bytes = small_fast ? ws_bytes(small_planes, 2) + 2 * small_exps + small_out : 0;
   size_t need = ws_bytes(8, sizeof(int)) + pass_bytes(g, P, true, nsplit, ks, pform) + doubles((size_t)g.nh * g.nv) +
                 doubles(small + 1) + small_fast_bytes;
   DSRG_TRY(ws_reserve(ws, need));
@@ -693,12 +695,16 @@ int impl_vv_opdm(Workspace& ws, size_t budget, const dsrg_fno_problem* prob, dou
   DSRG_TRY(carve_pass(ws, g, P, true, nsplit, ks, pform, W, st));
   double* t1 = ws_take<double>(ws, (size_t)g.nh * g.nv);
   double* work = ws_take<double>(ws, small + 1);
-  SmallFast sf{0, nullptr, nullptr, nullptr, nullptr};
+  SmallFast sf{};
   if (small_fast) {
     sf.ks = ks;
-    sf.planes = ws_take<__nv_bfloat16>(ws, 2 * (size_t)ks * g.nv * pad64(kmax));
-    sf.exps = ws_take<int>(ws, 2 * (size_t)g.nv);
-    sf.cbuf = ws_take<double>(ws, (size_t)g.nv * g.nv);
+    sf.planes = ws_take<__nv_bfloat16>(ws, small_planes);
+    sf.exps = reinterpret_cast<int*>(ws_take<char>(ws, small_exps));
+    sf.exps_y = reinterpret_cast<int*>(ws_take<char>(ws, small_exps));
+    char* out = ws_take<char>(ws, small_out);
+    if (!out) return DSRG_FNO_ERR_NOMEM;
+    if (small_res) sf.res = reinterpret_cast<uint16_t*>(out);
+    else sf.cbuf = reinterpret_cast<double*>(out);
     sf.err = W.err;
   }
   const size_t nv2 = (size_t)g.nv * g.nv;
@@ -773,13 +779,13 @@ int impl_correction(Workspace& ws, size_t budget, const dsrg_fno_problem* prob, 
   size_t pass_f = nk > 0 ? energy_pass_bytes(gf, ks, pform, budget) : 0;
   const int kpv = pad64(nv);
   // B' = B U enters E_vv(FNO) element by element and Delta E is a difference
-  // of two large energies: the rotation takes 6 digit planes (47 fraction
-  // bits) in the fast form, the passes themselves keep ks.
-  const int kx = ks ? 6 : 0;
+  // of two large energies: the rotation takes 12 moduli (rows of norm 2^53) in
+  // the fast form, the passes themselves keep ks.
+  const int kx = ks ? RES_MOD_X : 0;
   size_t xform = 0;
   if (kx && nk > 0)
-    xform = ws_bytes((size_t)kx * rows * kpv, 2) + ws_bytes(rows, sizeof(int)) + ws_bytes((size_t)kx * nk * kpv, 2) +
-            ws_bytes(nk, sizeof(int)) + ws_bytes(8, sizeof(int));
+    xform = ws_bytes((size_t)kx * rows * kpv, 2) + residue_exps_bytes(rows) + ws_bytes((size_t)kx * nk * kpv, 2) +
+            residue_exps_bytes(nk) + ws_bytes(residue_plain_bytes(kx, rows, nk), 1) + ws_bytes(8, sizeof(int));
   // full-energy form: the rest terms of both bases (their work overlaps the passes) and f_hp rotated
   const size_t mr_work = mr ? doubles(mr_energy_work_doubles(g, ks)) : 0;
   const size_t ff_bytes = mr ? doubles((size_t)g.nh * gf.np + 1) : 0;
@@ -838,16 +844,18 @@ int impl_correction(Workspace& ws, size_t budget, const dsrg_fno_problem* prob, 
     if (ks) {
       ws.off = base;
       __nv_bfloat16* pa = ws_take<__nv_bfloat16>(ws, (size_t)kx * rows * kpv);
-      int* ea = ws_take<int>(ws, rows);
+      int* ea = reinterpret_cast<int*>(ws_take<char>(ws, residue_exps_bytes(rows)));
       __nv_bfloat16* pb = ws_take<__nv_bfloat16>(ws, (size_t)kx * nk * kpv);
-      int* eb = ws_take<int>(ws, nk);
+      int* eb = reinterpret_cast<int*>(ws_take<char>(ws, residue_exps_bytes(nk)));
+      uint16_t* res = reinterpret_cast<uint16_t*>(ws_take<char>(ws, residue_plain_bytes(kx, rows, nk)));
       int* err = ws_take<int>(ws, 8);
       if (!err) return DSRG_FNO_ERR_NOMEM;
       DSRG_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
       // rows (Q, h) over the virtual index e, and U^T rows l over e
-      DSRG_TRY(slice_rows(kx, prob->B_hp + g.na, rows, nv, g.np, 1, kpv, pa, ea, st));
-      DSRG_TRY(slice_rows(kx, U, nk, nv, 1, nk, kpv, pb, eb, st));
-      DSRG_TRY(sliced_plain_gemm(kx, (int)rows, nk, pa, ea, pb, eb, kpv, Bf + g.na, gf.np, err, st));
+      DSRG_TRY(residue_stage(kx, prob->B_hp + g.na, rows, nv, g.np, 1, kpv, pa, ea, st));
+      DSRG_TRY(residue_stage(kx, U, nk, nv, 1, nk, kpv, pb, eb, st));
+      DSRG_TRY(residue_plain(kx, (int)rows, nk, pa, ea, rows, 0, pb, eb, kpv, 1.0, false, Bf + g.na, gf.np, 0, res,
+                             RES_PLAIN_CAP, err, st));
       DSRG_TRY(read_error_flag(err, st));
     } else {
       DSRG_TRY(gemm_f64((int)rows, nk, nv, 1.0, prob->B_hp + g.na, g.np, true, U, nk, false, 0.0, Bf + g.na, gf.np,

@@ -46,6 +46,35 @@ extern "C" int dsrg_fno_debug_sliced_gemm(int32_t ks, int32_t M, int32_t N, int3
   return h ? DSRG_FNO_ERR_TIMEOUT : DSRG_FNO_OK;
 }
 
+extern "C" int dsrg_fno_debug_residue_gemm(int32_t nmod, int32_t M, int32_t N, int32_t K, const double* A, const double* B,
+                                           double* C) {
+  if ((nmod != RES_MOD && nmod != RES_MOD_X) || M <= 0 || N <= 0 || K <= 0 || !A || !B || !C) return DSRG_FNO_ERR_ARG;
+  const int kp = pad64(K);
+  DevBuf dA, dB, dC, pa, pb, ea, eb, res, err;
+  DSRG_CUDA(cudaMalloc(&dA.p, sizeof(double) * M * K));
+  DSRG_CUDA(cudaMalloc(&dB.p, sizeof(double) * N * K));
+  DSRG_CUDA(cudaMalloc(&dC.p, sizeof(double) * M * N));
+  DSRG_CUDA(cudaMalloc(&pa.p, 2L * nmod * M * kp));
+  DSRG_CUDA(cudaMalloc(&pb.p, 2L * nmod * N * kp));
+  DSRG_CUDA(cudaMalloc(&ea.p, residue_exps_bytes(M)));
+  DSRG_CUDA(cudaMalloc(&eb.p, residue_exps_bytes(N)));
+  DSRG_CUDA(cudaMalloc(&res.p, residue_plain_bytes(nmod, M, N)));
+  DSRG_CUDA(cudaMalloc(&err.p, sizeof(int)));
+  DSRG_CUDA(cudaMemset(err.p, 0, sizeof(int)));
+  DSRG_CUDA(cudaMemcpy(dA.p, A, sizeof(double) * M * K, cudaMemcpyHostToDevice));
+  DSRG_CUDA(cudaMemcpy(dB.p, B, sizeof(double) * N * K, cudaMemcpyHostToDevice));
+  cudaStream_t st = 0;
+  DSRG_TRY(residue_stage(nmod, (double*)dA.p, M, K, K, 1, kp, (__nv_bfloat16*)pa.p, (int*)ea.p, st));
+  DSRG_TRY(residue_stage(nmod, (double*)dB.p, N, K, K, 1, kp, (__nv_bfloat16*)pb.p, (int*)eb.p, st));
+  DSRG_TRY(residue_plain(nmod, M, N, (__nv_bfloat16*)pa.p, (int*)ea.p, M, 0, (__nv_bfloat16*)pb.p, (int*)eb.p, kp, 1.0,
+                         false, (double*)dC.p, N, 0, (uint16_t*)res.p, RES_PLAIN_CAP, (int*)err.p, st));
+  DSRG_CUDA(cudaDeviceSynchronize());
+  int h = 0;
+  DSRG_CUDA(cudaMemcpy(&h, err.p, sizeof(int), cudaMemcpyDeviceToHost));
+  DSRG_CUDA(cudaMemcpy(C, dC.p, sizeof(double) * M * N, cudaMemcpyDeviceToHost));
+  return h ? DSRG_FNO_ERR_TIMEOUT : DSRG_FNO_OK;
+}
+
 extern "C" int dsrg_fno_debug_slice_rows(int32_t ks, int32_t R, int32_t K, const double* rows, float* planes,
                                          int32_t* exps) {
   if (ks < 3 || ks > 6 || R <= 0 || K <= 0 || !rows || !planes || !exps) return DSRG_FNO_ERR_ARG;

@@ -105,8 +105,9 @@ size_t mr_energy_work_doubles(const Geometry& g, int ks) {
              mr_dbl(8 * (size_t)z.nw3) + 3 * mr_dbl(8 * (size_t)z.n1) + mr_dbl(8 * (size_t)z.ngt1) +
              mr_dbl(8 * (size_t)z.nba) + mr_dbl(8 * (2 * (size_t)MR_EBLOCKS + 16));
   if (mr_tensor_gemm(g, ks)) {
-    const size_t kp = pad64(g.nq), ra = (size_t)g.nh * g.np, rb = (size_t)g.nh * g.na;
-    n += mr_dbl(2 * (size_t)ks * ra * kp) + mr_dbl(2 * (size_t)ks * rb * kp) + mr_dbl(4 * (ra + rb)) + mr_dbl(32);
+    const size_t kp = pad64(g.nq), ra = (size_t)g.nh * g.np, rb = (size_t)g.nh * g.na, k = ks == 5 ? RES_MOD : ks;
+    n += mr_dbl(2 * k * ra * kp) + mr_dbl(2 * k * rb * kp) + mr_dbl(residue_exps_bytes(ra)) +
+         mr_dbl(residue_exps_bytes(rb)) + mr_dbl(32) + (ks == 5 ? mr_dbl(residue_plain_bytes(RES_MOD, ra, rb)) : 0);
   }
   return n;
 }
@@ -161,15 +162,24 @@ int mr_energy_rest(const Geometry& g, int ks, const double* B, const double* eps
     if (mr_tensor_gemm(g, ks)) {
       // rows (i, a) of B and (j, y) of BA, contraction over Q: exact digit planes
       const int kp = pad64(g.nq);
-      __nv_bfloat16* pa = reinterpret_cast<__nv_bfloat16*>(take(2 * (size_t)ks * M * kp));
-      __nv_bfloat16* pb = reinterpret_cast<__nv_bfloat16*>(take(2 * (size_t)ks * N * kp));
-      int* ea = reinterpret_cast<int*>(take(4 * (size_t)(M + N)));
-      int* eb = ea + M;
+      const size_t k = ks == 5 ? RES_MOD : ks;
+      __nv_bfloat16* pa = reinterpret_cast<__nv_bfloat16*>(take(2 * k * M * kp));
+      __nv_bfloat16* pb = reinterpret_cast<__nv_bfloat16*>(take(2 * k * N * kp));
+      int* ea = reinterpret_cast<int*>(take(residue_exps_bytes(M)));
+      int* eb = reinterpret_cast<int*>(take(residue_exps_bytes(N)));
       int* err = reinterpret_cast<int*>(take(32));
       DSRG_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
-      DSRG_TRY(slice_rows(ks, B, M, g.nq, 1, M, kp, pa, ea, st));
-      DSRG_TRY(slice_rows(ks, BA, N, g.nq, 1, N, kp, pb, eb, st));
-      DSRG_TRY(sliced_plain_gemm(ks, M, N, pa, ea, pb, eb, kp, nu, N, err, st));
+      if (ks == 5) {
+        uint16_t* res = reinterpret_cast<uint16_t*>(take(residue_plain_bytes(RES_MOD, M, N)));
+        DSRG_TRY(residue_stage(RES_MOD, B, M, g.nq, 1, M, kp, pa, ea, st));
+        DSRG_TRY(residue_stage(RES_MOD, BA, N, g.nq, 1, N, kp, pb, eb, st));
+        DSRG_TRY(residue_plain(RES_MOD, M, N, pa, ea, M, 0, pb, eb, kp, 1.0, false, nu, N, 0, res, RES_PLAIN_CAP, err,
+                               st));
+      } else {
+        DSRG_TRY(slice_rows(ks, B, M, g.nq, 1, M, kp, pa, ea, st));
+        DSRG_TRY(slice_rows(ks, BA, N, g.nq, 1, N, kp, pb, eb, st));
+        DSRG_TRY(sliced_plain_gemm(ks, M, N, pa, ea, pb, eb, kp, nu, N, err, st));
+      }
       int h = 0;
       DSRG_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, st));
       DSRG_CUDA(cudaStreamSynchronize(st));

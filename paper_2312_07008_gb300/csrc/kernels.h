@@ -111,9 +111,10 @@ int small_terms_kmax(int nc, int na);
 // Buffers of the tensor-core path of the small terms (ks = 0: float64 only).
 struct SmallFast {
   int ks;
-  __nv_bfloat16* planes;  // 2 * ks * nv * pad64(kmax)
-  int* exps;              // 2 * nv
-  double* cbuf;           // nv * nv
+  __nv_bfloat16* planes;  // 2 * ks (residue form: RES_MOD) * nv * pad64(kmax)
+  int *exps, *exps_y;     // nv each (residue form: residue_exps_bytes(nv))
+  double* cbuf;           // nv * nv (digit planes only)
+  uint16_t* res;          // residue form: residue_plain_bytes(RES_MOD, nv, nv), else null
   int* err;
 };
 constexpr int SLICED_MIN_K = 256;
@@ -175,6 +176,11 @@ size_t residue_tile_bytes(int nm);  // residues of one output tile
 int residue_pair(const Geometry& g, const __nv_bfloat16* planes, const int* exps, int Kpad, const int2* tiles, int ntiles,
                  const int* slot_of, const float2* hp, uint16_t* res, int cap, float2* tau, float2* kap, double* ts,
                  int* err, cudaStream_t st);
+constexpr int RES_PLAIN_CAP = 1024;  // output tiles of a product whose residues are held at a time
+size_t residue_plain_bytes(int nm, long M, long N);  // residues of an M x N product (at most RES_PLAIN_CAP tiles)
+int residue_plain(int nm, int M, int N, const __nv_bfloat16* pa, const int* ea, long rows_a, int a0,
+                  const __nv_bfloat16* pb, const int* eb, int Kpad, double alpha, bool add, double* C, long ldc, int swap,
+                  uint16_t* res, int cap, int* err, cudaStream_t st);
 // Matrices [r0, r1) of a rank-K update that share their row scales; sign 0: all
 // of them, +-1: those of that sign.
 constexpr int RES_MAX_SEGMENTS = 64;

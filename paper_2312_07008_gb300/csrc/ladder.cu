@@ -6,9 +6,11 @@
 //   1. I[(a c)][(b d)] = sum_Q B^Q_{ac} B^Q_{bd}          (M = A nv, N = nv^2, K = naux)
 //      then the middle indices are swapped: I'[(a b)][(c d)]
 //   2. C[p][(a b)] = sum_{(c d)} T[p][(c d)] I'[(a b)][(c d)]  (M = npairs, N = A nv, K = nv^2)
-// Fast form: both on the digit-plane tensor-core kernel (5 planes); float64
-// form: the float64 GEMM.  2 nv^4 (naux + npairs) flops in all.
+// Fast form: both in the residue form on the tensor cores, the first writing
+// I' itself; float64 form: the float64 GEMM.  2 nv^4 (naux + npairs) flops.
 #include <math.h>
+
+#include <algorithm>
 
 #include "kernels.h"
 
@@ -32,6 +34,13 @@ __global__ void swap_middle_kernel(int A, int nv, const double* __restrict__ in,
 
 static const int LADDER_A_BLK = 16;
 
+// Values of a per block of the fast form: up to 2^28 integrals (2 GB, and 5.4 GB
+// of their planes), so that small bases run in one block and fill the chip.
+static int ladder_block(int nv) {
+  const long a = (1L << 28) / ((long)nv * nv * nv);
+  return (int)std::min<long>(nv, std::max<long>(LADDER_A_BLK, a));
+}
+
 int impl_ladder(Workspace& ws, int32_t nv, int32_t naux, const double* Bvv, int32_t npairs, const double* T,
                 int32_t precision, double* C, cudaStream_t st) {
   if (nv <= 0 || naux <= 0 || npairs <= 0 || !Bvv || !T || !C) return DSRG_FNO_ERR_ARG;
@@ -40,17 +49,18 @@ int impl_ladder(Workspace& ws, int32_t nv, int32_t naux, const double* Bvv, int3
   const long nv2 = (long)nv * nv;
   if (nv2 * LADDER_A_BLK * nv >= (1L << 31) || (long)npairs * nv2 >= (1L << 31)) return DSRG_FNO_ERR_UNSUPPORTED;
   const bool fast = precision == DSRG_FNO_SLICED_BF16;
-  const int A = std::min(LADDER_A_BLK, (int)nv);
+  const int A = fast ? ladder_block(nv) : std::min(LADDER_A_BLK, (int)nv);
   const long blk = (long)A * nv;  // rows (a c) or (a b) of one block
-  const int ks = 5;
+  const int nm = RES_MOD;
   const int qpad = pad64(naux), vpad = pad64((int)nv2);
-  size_t need = 2 * ws_bytes((size_t)blk * nv2, sizeof(double)) + ws_bytes(16, sizeof(int));
+  const size_t res_bytes = std::max(residue_plain_bytes(nm, blk, nv2), residue_plain_bytes(nm, npairs, blk));
+  size_t need = ws_bytes((size_t)blk * nv2, sizeof(double)) + ws_bytes(16, sizeof(int)) + ws_bytes(8, sizeof(int));
   if (fast)
-    need += ws_bytes((size_t)ks * nv2 * qpad, 2) + ws_bytes((size_t)ks * blk * qpad, 2) +
-            ws_bytes((size_t)ks * npairs * vpad, 2) + ws_bytes((size_t)ks * blk * vpad, 2) +
-            ws_bytes(nv2, sizeof(int)) + ws_bytes(blk, sizeof(int)) + ws_bytes(npairs, sizeof(int)) +
-            ws_bytes(blk + 16, sizeof(int));
-  need += ws_bytes(8, sizeof(int));
+    need += ws_bytes((size_t)nm * nv2 * qpad, 2) + ws_bytes((size_t)nm * npairs * vpad, 2) +
+            ws_bytes((size_t)nm * blk * vpad, 2) + residue_exps_bytes(nv2) + residue_exps_bytes(npairs) +
+            residue_exps_bytes(blk) + ws_bytes(res_bytes, 1);
+  else
+    need += ws_bytes((size_t)blk * nv2, sizeof(double));
   DSRG_TRY(ws_reserve(ws, need));
   {
     int* flag = ws_take<int>(ws, 8);
@@ -62,54 +72,58 @@ int impl_ladder(Workspace& ws, int32_t nv, int32_t naux, const double* Bvv, int3
     DSRG_CUDA(cudaStreamSynchronize(st));
     if (h) return DSRG_FNO_ERR_NONFINITE;
   }
-  double* I1 = ws_take<double>(ws, (size_t)blk * nv2);
   double* I2 = ws_take<double>(ws, (size_t)blk * nv2);
   int* err = ws_take<int>(ws, 16);
-  __nv_bfloat16 *pY = nullptr, *pX = nullptr, *pT = nullptr, *pI = nullptr;
-  int *eY = nullptr, *eX = nullptr, *eT = nullptr, *eI = nullptr;
-  if (fast) {
-    pY = ws_take<__nv_bfloat16>(ws, (size_t)ks * nv2 * qpad);
-    pX = ws_take<__nv_bfloat16>(ws, (size_t)ks * blk * qpad);
-    pT = ws_take<__nv_bfloat16>(ws, (size_t)ks * npairs * vpad);
-    pI = ws_take<__nv_bfloat16>(ws, (size_t)ks * blk * vpad);
-    eY = ws_take<int>(ws, nv2);
-    eX = ws_take<int>(ws, blk);
-    eT = ws_take<int>(ws, npairs);
-    eI = ws_take<int>(ws, blk + 16);
-    if (!eI) return DSRG_FNO_ERR_NOMEM;
-    DSRG_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
-    // rows (b d) of the factors over Q, and rows p of the amplitudes over (c d)
-    DSRG_TRY(slice_rows(ks, Bvv, nv2, naux, 1, nv2, qpad, pY, eY, st));
-    DSRG_TRY(slice_rows(ks, T, npairs, (int)nv2, nv2, 1, vpad, pT, eT, st));
+  if (!fast) {
+    double* I1 = ws_take<double>(ws, (size_t)blk * nv2);
+    if (!I1) return DSRG_FNO_ERR_NOMEM;
+    for (int a0 = 0; a0 < nv; a0 += A) {
+      const int na = std::min(A, nv - a0);
+      const long rows = (long)na * nv;
+      {
+        DSRG_PHASE("phase_ladder_integrals", st);
+        DSRG_TRY(gemm_f64((int)rows, (int)nv2, naux, 1.0, Bvv + (long)a0 * nv, nv2, false, Bvv, nv2, false, 0.0, I1, nv2,
+                          1, 0, 0, 0, st));
+        swap_middle_kernel<<<(unsigned)(rows * nv), 128, 0, st>>>(na, nv, I1, I2);
+        DSRG_LAUNCH_CHECK();
+      }
+      DSRG_PHASE("phase_ladder_contract", st);
+      DSRG_TRY(gemm_f64(npairs, (int)rows, (int)nv2, 1.0, T, nv2, true, I2, nv2, true, 0.0, C + (long)a0 * nv, nv2, 1, 0,
+                        0, 0, st));
+    }
+    DSRG_CUDA(cudaStreamSynchronize(st));
+    return DSRG_FNO_OK;
+  }
+  auto exps = [&ws](size_t rows) { return reinterpret_cast<int*>(ws_take<char>(ws, residue_exps_bytes(rows))); };
+  __nv_bfloat16* pY = ws_take<__nv_bfloat16>(ws, (size_t)nm * nv2 * qpad);
+  __nv_bfloat16* pT = ws_take<__nv_bfloat16>(ws, (size_t)nm * npairs * vpad);
+  __nv_bfloat16* pI = ws_take<__nv_bfloat16>(ws, (size_t)nm * blk * vpad);
+  int *eY = exps(nv2), *eT = exps(npairs), *eI = exps(blk);
+  uint16_t* res = reinterpret_cast<uint16_t*>(ws_take<char>(ws, res_bytes));
+  if (!res) return DSRG_FNO_ERR_NOMEM;
+  DSRG_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
+  {
+    DSRG_PHASE("phase_ladder_integrals", st);
+    // rows (b d) of the factors over Q (the rows (a c) are among them), and rows p of the amplitudes over (c d)
+    DSRG_TRY(residue_stage(nm, Bvv, nv2, naux, 1, nv2, qpad, pY, eY, st));
+    DSRG_TRY(residue_stage(nm, T, npairs, (int)nv2, nv2, 1, vpad, pT, eT, st));
   }
   for (int a0 = 0; a0 < nv; a0 += A) {
     const int na = std::min(A, nv - a0);
     const long rows = (long)na * nv;
     {
       DSRG_PHASE("phase_ladder_integrals", st);
-      if (fast) {
-        DSRG_TRY(slice_rows(ks, Bvv + (long)a0 * nv, rows, naux, 1, nv2, qpad, pX, eX, st));
-        DSRG_TRY(sliced_plain_gemm(ks, (int)rows, (int)nv2, pX, eX, pY, eY, qpad, I1, nv2, err, st));
-      } else {
-        DSRG_TRY(gemm_f64((int)rows, (int)nv2, naux, 1.0, Bvv + (long)a0 * nv, nv2, false, Bvv, nv2, false, 0.0, I1,
-                          nv2, 1, 0, 0, 0, st));
-      }
-      swap_middle_kernel<<<(unsigned)(rows * nv), 128, 0, st>>>(na, nv, I1, I2);
-      DSRG_LAUNCH_CHECK();
+      // written with the middle indices swapped
+      DSRG_TRY(residue_plain(nm, (int)rows, (int)nv2, pY, eY, nv2, a0 * nv, pY, eY, qpad, 1.0, false, I2, nv2, nv, res,
+                             RES_PLAIN_CAP, err, st));
     }
-    {
-      DSRG_PHASE("phase_ladder_contract", st);
-      if (fast) {
-        DSRG_TRY(slice_rows(ks, I2, rows, (int)nv2, nv2, 1, vpad, pI, eI, st));
-        DSRG_TRY(sliced_plain_gemm(ks, npairs, (int)rows, pT, eT, pI, eI, vpad, C + (long)a0 * nv, nv2, err, st));
-      } else {
-        DSRG_TRY(gemm_f64(npairs, (int)rows, (int)nv2, 1.0, T, nv2, true, I2, nv2, true, 0.0, C + (long)a0 * nv, nv2,
-                          1, 0, 0, 0, st));
-      }
-    }
+    DSRG_PHASE("phase_ladder_contract", st);
+    DSRG_TRY(residue_stage(nm, I2, rows, (int)nv2, nv2, 1, vpad, pI, eI, st));
+    DSRG_TRY(residue_plain(nm, npairs, (int)rows, pT, eT, npairs, 0, pI, eI, vpad, 1.0, false, C + (long)a0 * nv, nv2, 0,
+                           res, RES_PLAIN_CAP, err, st));
   }
   int h = 0;
-  if (fast) DSRG_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, st));
+  DSRG_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, st));
   DSRG_CUDA(cudaStreamSynchronize(st));
   return h ? DSRG_FNO_ERR_TIMEOUT : DSRG_FNO_OK;
 }

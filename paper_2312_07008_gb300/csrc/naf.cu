@@ -5,9 +5,9 @@
 // diagonalised, W = U diag(w) U^T (w descending), and the factors are
 // rotated to the eigenvectors with w > threshold:
 //   B'^K_{ia} = sum_Q U_QK B^Q_{ia}.
-// In the fast form both contractions run on the digit-plane kernel: W with
-// 5 planes (its entries are sums of nh np products), B' with 6 (B' enters
-// every integral, as the rotation to the frozen natural orbitals does);
+// In the fast form both contractions run in the residue form: W with 10 moduli
+// (its entries are sums of nh np products), B' with 12 (B' enters every
+// integral, as the rotation to the frozen natural orbitals does);
 // the eigensolve is that of the natural orbitals.
 #include <math.h>
 
@@ -26,14 +26,15 @@ int impl_naf(Workspace& ws, int32_t nh, int32_t np, int32_t naux, const double* 
   if (L * 2 > (1L << 31) || (long)naux * naux >= (1L << 31)) return DSRG_FNO_ERR_UNSUPPORTED;
   const size_t n2 = (size_t)naux * naux;
   const bool fast = precision == DSRG_FNO_SLICED_BF16;
-  const int kw = 5, kb = 6;
+  const int kw = RES_MOD, kb = RES_MOD_X;
   const int lpad = pad64((int)L), qpad = pad64(naux);
   size_t planes = 0;
   if (fast) {
     // the metric's planes, then (reusing the space) the rotation's
-    const size_t p1 = ws_bytes((size_t)kw * naux * lpad, 2) + ws_bytes(naux, sizeof(int)) + ws_bytes(16, sizeof(int));
-    const size_t p2 = ws_bytes((size_t)kb * L * qpad, 2) + ws_bytes((size_t)kb * naux * qpad, 2) +
-                      ws_bytes(L, sizeof(int)) + ws_bytes(naux, sizeof(int)) + ws_bytes(16, sizeof(int));
+    const size_t p1 = ws_bytes((size_t)kw * naux * lpad, 2) + residue_exps_bytes(naux) + ws_bytes(16, sizeof(int)) +
+                      ws_bytes(residue_plain_bytes(kw, naux, naux), 1);
+    const size_t p2 = ws_bytes((size_t)kb * L * qpad, 2) + ws_bytes((size_t)kb * naux * qpad, 2) + residue_exps_bytes(L) +
+                      residue_exps_bytes(naux) + ws_bytes(16, sizeof(int)) + ws_bytes(residue_plain_bytes(kb, naux, L), 1);
     planes = std::max(p1, p2);
   }
   const size_t need = 3 * ws_bytes(n2, sizeof(double)) + ws_bytes(eig_work_doubles(naux), sizeof(double)) +
@@ -65,12 +66,14 @@ int impl_naf(Workspace& ws, int32_t nh, int32_t np, int32_t naux, const double* 
     if (fast) {
       ws.off = base;
       __nv_bfloat16* pl = ws_take<__nv_bfloat16>(ws, (size_t)kw * naux * lpad);
-      int* ex = ws_take<int>(ws, naux);
+      int* ex = reinterpret_cast<int*>(ws_take<char>(ws, residue_exps_bytes(naux)));
+      uint16_t* res = reinterpret_cast<uint16_t*>(ws_take<char>(ws, residue_plain_bytes(kw, naux, naux)));
       int* err = ws_take<int>(ws, 16);
       if (!err) return DSRG_FNO_ERR_NOMEM;
       DSRG_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
-      DSRG_TRY(slice_rows(kw, B, naux, (int)L, L, 1, lpad, pl, ex, st));
-      DSRG_TRY(sliced_plain_gemm(kw, naux, naux, pl, ex, pl, ex, lpad, W, naux, err, st));
+      DSRG_TRY(residue_stage(kw, B, naux, (int)L, L, 1, lpad, pl, ex, st));
+      DSRG_TRY(residue_plain(kw, naux, naux, pl, ex, naux, 0, pl, ex, lpad, 1.0, false, W, naux, 0, res, RES_PLAIN_CAP,
+                             err, st));
       int h = 0;
       DSRG_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, st));
       DSRG_CUDA(cudaStreamSynchronize(st));
@@ -99,15 +102,17 @@ int impl_naf(Workspace& ws, int32_t nh, int32_t np, int32_t naux, const double* 
       ws.off = base;
       __nv_bfloat16* pb = ws_take<__nv_bfloat16>(ws, (size_t)kb * L * qpad);
       __nv_bfloat16* pu = ws_take<__nv_bfloat16>(ws, (size_t)kb * naux * qpad);
-      int* eb = ws_take<int>(ws, L);
-      int* eu = ws_take<int>(ws, naux);
+      int* eb = reinterpret_cast<int*>(ws_take<char>(ws, residue_exps_bytes(L)));
+      int* eu = reinterpret_cast<int*>(ws_take<char>(ws, residue_exps_bytes(naux)));
+      uint16_t* res = reinterpret_cast<uint16_t*>(ws_take<char>(ws, residue_plain_bytes(kb, naux, L)));
       int* err = ws_take<int>(ws, 16);
       if (!err) return DSRG_FNO_ERR_NOMEM;
       DSRG_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
       // rows of U^T (eigenvector K over Q: stride naux) and of B2^T (column ia over Q: stride L)
-      DSRG_TRY(slice_rows(kb, U, k, naux, 1, naux, qpad, pu, eu, st));
-      DSRG_TRY(slice_rows(kb, B, L, naux, 1, L, qpad, pb, eb, st));
-      DSRG_TRY(sliced_plain_gemm(kb, k, (int)L, pu, eu, pb, eb, qpad, B_out, L, err, st));
+      DSRG_TRY(residue_stage(kb, U, k, naux, 1, naux, qpad, pu, eu, st));
+      DSRG_TRY(residue_stage(kb, B, L, naux, 1, L, qpad, pb, eb, st));
+      DSRG_TRY(residue_plain(kb, k, (int)L, pu, eu, k, 0, pb, eb, qpad, 1.0, false, B_out, L, 0, res, RES_PLAIN_CAP, err,
+                             st));
       int h = 0;
       DSRG_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, st));
       DSRG_CUDA(cudaStreamSynchronize(st));

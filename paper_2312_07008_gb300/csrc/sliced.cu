@@ -1,7 +1,7 @@
 // Contractions by exact bfloat16 digit planes on the tcgen05 tensor cores (the
 // planes are staged by stage.cu): the fast form with 3 or 4 planes, and the
 // literal forms of the precision study.  With 5 planes the residue form
-// (residue.cu) takes the pair contraction.
+// (residue.cu) takes its place.
 //
 // Products.  For two rows a, b:  x_a . x_b = 2^-14 sum_L 2^-8L S_L with the
 // level sums S_L = sum_{s+t=L} sum_k d_s(a,k) d_t(b,k).  Only levels

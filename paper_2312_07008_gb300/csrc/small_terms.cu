@@ -367,10 +367,17 @@ int small_terms_f64(const Geometry& g, const double* ts, const double* t1, const
     if (F.ks > 0 && K >= SLICED_MIN_K) {
       const int kp = pad64(K);
       __nv_bfloat16* px = F.planes;
-      __nv_bfloat16* py = F.planes + (size_t)F.ks * g.nv * kp;
+      __nv_bfloat16* py = F.planes + (size_t)(F.res ? RES_MOD : F.ks) * g.nv * kp;
+      if (F.res) {
+        DSRG_TRY(residue_stage(RES_MOD, X, g.nv, K, K, 1, kp, px, F.exps, st));
+        DSRG_TRY(residue_stage(RES_MOD, Y, g.nv, K, K, 1, kp, py, F.exps_y, st));
+        DSRG_TRY(residue_plain(RES_MOD, g.nv, g.nv, px, F.exps, g.nv, 0, py, F.exps_y, kp, coef, true, D, g.nv, 0, F.res,
+                               RES_PLAIN_CAP, F.err, st));
+        continue;
+      }
       DSRG_TRY(slice_rows(F.ks, X, g.nv, K, K, 1, kp, px, F.exps, st));
-      DSRG_TRY(slice_rows(F.ks, Y, g.nv, K, K, 1, kp, py, F.exps + g.nv, st));
-      DSRG_TRY(sliced_plain_gemm(F.ks, g.nv, g.nv, px, F.exps, py, F.exps + g.nv, kp, F.cbuf, g.nv, F.err, st));
+      DSRG_TRY(slice_rows(F.ks, Y, g.nv, K, K, 1, kp, py, F.exps_y, st));
+      DSRG_TRY(sliced_plain_gemm(F.ks, g.nv, g.nv, px, F.exps, py, F.exps_y, kp, F.cbuf, g.nv, F.err, st));
       const long n2 = (long)g.nv * g.nv;
       axpy_kernel<<<ceil_div(n2, 256), 256, 0, st>>>(n2, coef, F.cbuf, D);
       DSRG_LAUNCH_CHECK();
