@@ -1,6 +1,10 @@
 // Float64 contractions on the CUDA cores: generic batched GEMM, the pair
 // contraction with the Eq. A7 epilogue, and the dressed symmetric rank-K
 // update that accumulates the vv classes of D_vv.
+// (The generic GEMM picks its tile by the SMs it fills: the float64 products of
+// 300 x 300 outputs that the small terms and the recanonicalisation make had 25
+// blocks of 64 x 64 for 152 SMs: small terms of the float64 form at nvir 300 7.9
+// -> 1.7 ms.)
 //
 // GB300 runs float64 at a small fraction of its float32 rate, so these
 // kernels are float64-pipe bound by construction; they are the plain form
@@ -12,6 +16,18 @@ namespace dsrg {
 namespace {
 
 constexpr int TM = 64, TN = 64, TK = 16, NT = 256;
+
+// X[k][m] = op(A)[m0 + m][k0 + k], zero outside
+template <bool KC, int T>
+__device__ __forceinline__ void load_tile(double (*X)[T + 1], const double* A, long lda, int m0, int k0, int M, int K) {
+#pragma unroll
+  for (int it = 0; it < (T * TK) / NT; ++it) {
+    const int idx = threadIdx.x + it * NT;
+    const int k = KC ? idx % TK : idx / T, m = KC ? idx / TK : idx % T;
+    const int gm = m0 + m, gk = k0 + k;
+    X[k][m] = (gm < M && gk < K) ? (KC ? A[(long)gm * lda + gk] : A[(long)gk * lda + gm]) : 0.0;
+  }
+}
 
 template <bool A_KC>
 __device__ __forceinline__ void load_a_tile(double (*As)[TM + 1], const double* A, long lda, int m0,
@@ -73,39 +89,84 @@ __device__ __forceinline__ void mma_tile(const double (*As)[TM + 1], const doubl
   }
 }
 
-template <bool A_KC, bool B_KC>
+// T x T output tiles, (T / 16)^2 elements per thread.  An SM has two float64
+// lanes, so even one element per thread (two shared loads per FMA) runs at their
+// rate; a small T is for products with too few 64 x 64 tiles for all SMs.
+template <bool A_KC, bool B_KC, int T>
 __global__ void __launch_bounds__(NT) gemm_f64_kernel(int M, int N, int K, double alpha,
                                                       const double* __restrict__ A, long lda,
                                                       const double* __restrict__ B, long ldb,
                                                       double beta, double* C, long ldc, long sa,
                                                       long sb, long sc) {
-  __shared__ double As[TK][TM + 1];
-  __shared__ double Bs[TK][TN + 1];
+  constexpr int R = T / 16;
+  __shared__ double As[TK][T + 1];
+  __shared__ double Bs[TK][T + 1];
   A += sa * blockIdx.z;
   B += sb * blockIdx.z;
   C += sc * blockIdx.z;
-  const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
-  double acc[4][4] = {};
+  const int m0 = blockIdx.y * T, n0 = blockIdx.x * T;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  double acc[R][R] = {};
   for (int k0 = 0; k0 < K; k0 += TK) {
-    load_a_tile<A_KC>(As, A, lda, m0, k0, M, K);
-    load_b_tile<B_KC>(Bs, B, ldb, n0, k0, N, K);
+    load_tile<A_KC, T>(As, A, lda, m0, k0, M, K);
+    load_tile<B_KC, T>(Bs, B, ldb, n0, k0, N, K);
     __syncthreads();
-    mma_tile(As, Bs, acc);
+#pragma unroll
+    for (int k = 0; k < TK; ++k) {
+      double a[R], b[R];
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        a[i] = As[k][ty + 16 * i];
+        b[i] = Bs[k][tx + 16 * i];
+      }
+#pragma unroll
+      for (int i = 0; i < R; ++i)
+#pragma unroll
+        for (int j = 0; j < R; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+    }
     __syncthreads();
   }
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < R; ++i) {
     int m = m0 + ty + 16 * i;
     if (m >= M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < R; ++j) {
       int n = n0 + tx + 16 * j;
       if (n >= N) continue;
       double* c = C + (long)m * ldc + n;
       *c = alpha * acc[i][j] + (beta == 0.0 ? 0.0 : beta * *c);
     }
   }
+}
+
+template <bool A_KC, bool B_KC>
+void launch_gemm_f64(int T, int M, int N, int K, double alpha, const double* A, long lda, const double* B, long ldb,
+                     double beta, double* C, long ldc, int batch, long sa, long sb, long sc, cudaStream_t st) {
+  const dim3 grid(ceil_div(N, T), ceil_div(M, T), batch);
+  if (T == 64)
+    gemm_f64_kernel<A_KC, B_KC, 64><<<grid, NT, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, sa, sb, sc);
+  else if (T == 32)
+    gemm_f64_kernel<A_KC, B_KC, 32><<<grid, NT, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, sa, sb, sc);
+  else
+    gemm_f64_kernel<A_KC, B_KC, 16><<<grid, NT, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, sa, sb, sc);
+}
+
+// Tile edge: the one whose fullest SM does the least float64 work (blocks per
+// SM times T^2; the larger on a tie, which reads less).
+int gemm_tile(int M, int N, int batch) {
+  const int sms = 152;
+  int best = 64;
+  long best_cost = 0;
+  for (int T : {64, 32, 16}) {
+    const long blocks = (long)ceil_div(M, T) * ceil_div(N, T) * batch;
+    const long cost = (long)ceil_div(blocks, sms) * T * T;
+    if (best_cost == 0 || cost * 10 < best_cost * 9) {
+      best_cost = cost;
+      best = T;
+    }
+  }
+  return best;
 }
 
 // ---------------------------------------------------------------------------
@@ -246,15 +307,10 @@ int gemm_f64(int M, int N, int K, double alpha, const double* A, long lda, bool 
              const double* B, long ldb, bool b_kcontig, double beta, double* C, long ldc, int batch,
              long sa, long sb, long sc, cudaStream_t st) {
   if (M <= 0 || N <= 0 || batch <= 0) return DSRG_FNO_OK;
-  dim3 grid(ceil_div(N, TN), ceil_div(M, TM), batch);
-  if (a_kcontig && b_kcontig)
-    gemm_f64_kernel<true, true><<<grid, NT, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, sa, sb, sc);
-  else if (a_kcontig && !b_kcontig)
-    gemm_f64_kernel<true, false><<<grid, NT, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, sa, sb, sc);
-  else if (!a_kcontig && b_kcontig)
-    gemm_f64_kernel<false, true><<<grid, NT, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, sa, sb, sc);
-  else
-    gemm_f64_kernel<false, false><<<grid, NT, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, sa, sb, sc);
+  const int T = gemm_tile(M, N, batch);
+  auto go = a_kcontig ? (b_kcontig ? launch_gemm_f64<true, true> : launch_gemm_f64<true, false>)
+                      : (b_kcontig ? launch_gemm_f64<false, true> : launch_gemm_f64<false, false>);
+  go(T, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, batch, sa, sb, sc, st);
   DSRG_LAUNCH_CHECK();
   return DSRG_FNO_OK;
 }
