@@ -51,6 +51,7 @@ struct Batch {
   int pair_begin, npairs, desc_begin, ndesc;
   int nout;  // dressed matrices written (a core-core pair writes two)
   int ncc;   // leading work items that are core-core groups
+  int ncc_out;  // their dressed matrices (weights 2 and 6: none negative)
 };
 
 struct Plan {
@@ -93,11 +94,11 @@ static void build_plan(int nc, int na, long cap_pairs, Plan& P) {
   long largest = 0;
   for (auto& G : groups) largest = std::max<long>(largest, (long)G.pairs.size());
   cap_pairs = std::max(cap_pairs, largest);
-  Batch cur{0, 0, 0, 0, 0, 0};
+  Batch cur{0, 0, 0, 0, 0, 0, 0};
   for (auto& G : groups) {
     if (cur.npairs > 0 && cur.npairs + (long)G.pairs.size() > cap_pairs) {
       P.batches.push_back(cur);
-      cur = Batch{(int)P.pairs.size(), 0, (int)P.desc.size(), 0, 0, 0};
+      cur = Batch{(int)P.pairs.size(), 0, (int)P.desc.size(), 0, 0, 0, 0};
     }
     for (int o0 = 0; o0 < G.nout; o0 += DRESS_OC) {
       DressDesc d{};
@@ -113,6 +114,7 @@ static void build_plan(int nc, int na, long cap_pairs, Plan& P) {
       if (G.kind == GROUP_CC_DIAG || G.kind == GROUP_CC_PAIR) ++cur.ncc;
     }
     cur.nout += G.nout;
+    if (G.kind == GROUP_CC_DIAG || G.kind == GROUP_CC_PAIR) cur.ncc_out += G.nout;
     for (auto p : G.pairs) P.pairs.push_back(p);
     cur.npairs += (int)G.pairs.size();
   }
@@ -197,6 +199,10 @@ struct PassBuffers {
   int kpad_q, kpad_v; // padded contraction lengths (naux, nvir)
   __nv_bfloat16 *planes_b, *planes_s;
   int *exps_b, *exps_s, *err;
+  bool syrk_residue;       // rank-K update in the residue form (where the digit form would take 5 planes)
+  float* rowpart;          // bound of each row's norm in each tile column of each dressed matrix
+  int* scale_of;           // scale group of each dressed matrix
+  uint16_t* res_s;         // residues of the update's output tiles
   float2* nu;        // double-float contraction tiles
   float2* eps_dd;    // orbital energies as double-float
   unsigned* rowmax;  // max |hi| per row of the dressed matrices (float bits)
@@ -270,7 +276,8 @@ static int pair_tile_cols(int ks, int2 pform) {
 static long pair_cap_for_budget(int nv, int np, int ks, bool residue, size_t budget) {
   // tau + kappa + two dressed matrices per pair (+ the dressed planes and, outside the residue form, nu in the fast form)
   double per_pair = 4.0 * (double)nv * nv * 8.0 + 1024.0;
-  if (ks) per_pair += (residue ? 0.0 : (double)np * np * 8.0) + 2.0 * ks * 2.0 * (double)nv * (nv + 64);
+  const int planes = ks == 5 ? RES_MOD_S : ks;
+  if (ks) per_pair += (residue ? 0.0 : (double)np * np * 8.0) + 2.0 * (planes * 2.0 + 0.25) * (double)nv * (nv + 64);
   long cap = (long)(budget / per_pair);
   return std::max<long>(cap, 1);
 }
@@ -375,10 +382,11 @@ static int run_pass(const Geometry& g, const double* B, const double* eps, const
     {
       DSRG_PHASE("phase_dress", st);
       if (W.ks) {
-        unsigned* rm = want_d ? W.rowmax : nullptr;
+        unsigned* rm = want_d && !W.syrk_residue ? W.rowmax : nullptr;
+        float* rp = want_d && W.syrk_residue ? W.rowpart : nullptr;
         if (rm) DSRG_CUDA(cudaMemsetAsync(rm, 0, sizeof(unsigned) * (size_t)b.nout * g.nv, st));
         DSRG_TRY(dress_dd(g, W.desc + b.desc_begin, b.ndesc, b.ncc, aux, as_dd(W.tau), as_dd(W.kap), as_dd(W.sig),
-                          W.sig_sign, W.e_part, want_d, rm, st));
+                          W.sig_sign, W.e_part, want_d, rm, rp, st));
       } else {
         DSRG_TRY(dress_f64(g, W.desc + b.desc_begin, b.ndesc, b.ncc, aux, W.tau, W.kap, W.sig, W.sig_sign,
                            W.e_part, want_d, st));
@@ -386,7 +394,10 @@ static int run_pass(const Geometry& g, const double* B, const double* eps, const
     }
     DSRG_TRY(ordered_sum(W.e_part, (long)b.ndesc * DRESS_TILE_BLOCKS, W.e_acc, bi > 0, st));
     if (want_d) {
-      if (W.ks) {
+      if (W.syrk_residue) {
+        DSRG_TRY(residue_syrk(g.nv, b.nout, b.ncc_out, as_dd(W.sig), W.rowpart, W.sig_sign, W.planes_s, W.exps_s,
+                              W.scale_of, W.kpad_v, W.res_s, D, W.err, st));
+      } else if (W.ks) {
         const long rows = (long)b.nout * g.nv;
         {
           DSRG_PHASE("phase_stage_sig", st);
@@ -461,8 +472,15 @@ static size_t pass_bytes(const Geometry& g, const Plan& P, bool want_d, int nspl
     b += rf ? ws_bytes(P.res_cap * residue_tile_bytes(RES_MOD), 1) : doubles((size_t)P.max_pairs * g.np * g.np);
     b += doubles((size_t)g.nh + g.nv);
     b += doubles((size_t)g.nh * g.np);
-    if (want_d)
-      b += ws_bytes((size_t)ks * P.max_out * g.nv * pad64(g.nv), 2) + 2 * ws_bytes((size_t)P.max_out * g.nv, sizeof(int));
+    if (want_d) {
+      if (syrk_slices(ks) == 5)
+        b += ws_bytes((size_t)RES_MOD_S * P.max_out * g.nv * pad64(g.nv), 2) +
+             ws_bytes((size_t)RES_MAX_SEGMENTS * g.nv, sizeof(int)) + ws_bytes((size_t)P.max_out * g.nv * ceil_div(g.nv, 16), sizeof(float)) +
+             ws_bytes(P.max_out, sizeof(int)) + ws_bytes(residue_syrk_res_bytes(g.nv), 1);
+      else
+        b += ws_bytes((size_t)ks * P.max_out * g.nv * pad64(g.nv), 2) +
+             2 * ws_bytes((size_t)P.max_out * g.nv, sizeof(int));
+    }
     b += ws_bytes(8, sizeof(int));
     size_t tiles = 0;
     const int bm = pair_tile_rows(ks, pform), bn = pair_tile_cols(ks, pform);
@@ -522,9 +540,18 @@ static int carve_pass(Workspace& ws, const Geometry& g, const Plan& P, bool want
     W.fused = !W.residue && fused_epilogue_enabled();
     if (W.fused) DSRG_TRY(reg_tables_device(&W.reg));
     if (want_d) {
-      W.planes_s = ws_take<__nv_bfloat16>(ws, (size_t)ks * P.max_out * g.nv * W.kpad_v);
-      W.exps_s = ws_take<int>(ws, (size_t)P.max_out * g.nv);
-      W.rowmax = ws_take<unsigned>(ws, (size_t)P.max_out * g.nv);
+      W.syrk_residue = W.ks_d == 5;
+      if (W.syrk_residue) {
+        W.planes_s = ws_take<__nv_bfloat16>(ws, (size_t)RES_MOD_S * P.max_out * g.nv * W.kpad_v);
+        W.exps_s = ws_take<int>(ws, (size_t)RES_MAX_SEGMENTS * g.nv);
+        W.rowpart = ws_take<float>(ws, (size_t)P.max_out * g.nv * ceil_div(g.nv, 16));
+        W.scale_of = ws_take<int>(ws, P.max_out);
+        W.res_s = reinterpret_cast<uint16_t*>(ws_take<char>(ws, residue_syrk_res_bytes(g.nv)));
+      } else {
+        W.planes_s = ws_take<__nv_bfloat16>(ws, (size_t)ks * P.max_out * g.nv * W.kpad_v);
+        W.exps_s = ws_take<int>(ws, (size_t)P.max_out * g.nv);
+        W.rowmax = ws_take<unsigned>(ws, (size_t)P.max_out * g.nv);
+      }
     }
     W.err = ws_take<int>(ws, 8);
     if (!W.err) return DSRG_FNO_ERR_NOMEM;

@@ -113,15 +113,178 @@ __device__ __forceinline__ dd dd_fma_acc(dd acc, dd c, dd s) {
   return quick_two_sum(t.hi, t.lo);
 }
 
+// What the staging of the dressed matrices needs of a row: the largest |hi| of
+// all its elements (digit planes: rowmax, atomics), or a bound of each tile's
+// norm (residues: rowpart[matrix][tile column][row], strides for tiles of GT).
+// Float64 atomics per row instead took more time than the dressing itself (the
+// SM has two float64 lanes; opdm pass of nvir 1200: 67 ms).
+__device__ __forceinline__ bool square_in_range(float s) { return s > 1e-30f && s < 1e38f; }
+
+// Norms of eight of a warp's rows of 32 elements each (v: this lane's |hi|; row
+// of value i: lane 4 i's result): the lanes halve the values before they halve
+// themselves (9 shuffles).  Where a square would leave float32's range, the
+// largest element times 32^1/2.
+__device__ __forceinline__ float row_norms8(const float (&v)[8]) {
+  const int lane = threadIdx.x & 31;
+  float x[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) x[i] = v[i] * v[i];
+#pragma unroll
+  for (int h = 4, o = 16; h > 0; h >>= 1, o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < h; ++i) x[i] = (up ? x[i + h] : x[i]) + __shfl_xor_sync(0xffffffffu, up ? x[i] : x[i + h], o);
+  }
+  x[0] += __shfl_xor_sync(0xffffffffu, x[0], 2);
+  x[0] += __shfl_xor_sync(0xffffffffu, x[0], 1);
+  float n = sqrtf(x[0]);
+  if (__any_sync(0xffffffffu, !square_in_range(x[0]))) {
+    const int mine = lane >> 2;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float m = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v[i])));
+      if (mine == i) n = m * 5.6568546f;  // above 32^1/2
+    }
+  }
+  return n;
+}
+
+// Core pairs.  With P = tau + tau^T and Q = tau - tau^T (and the same of kappa)
+// the pair (m, n) contributes E = <P, P_k> / 2 + 3 <Q, Q_k> / 2 and the dressed
+// matrices sqrt(lambda) sigma = P and sqrt(3) Q; the pair (m, m) E = <tau, kappa>
+// and sqrt(2) tau.  One pass over the upper 32 x 32 tiles, four elements and
+// their transposes per thread, no coefficients: the general kernel spent about
+// 200 instructions on an element (dressing of an opdm pass of nvir 1200: 54.3 ms,
+// now 48.5; nvir 300 with 6 active: 0.82, now 0.70).  Bound by memory: 16 bytes
+// read and 16 written per element.
+constexpr int CT = 32;
+__global__ void __launch_bounds__(256, 4) dress_core_dd_kernel(int nv, const DressDesc* __restrict__ desc,
+                                                               const float2* __restrict__ tau,
+                                                               const float2* __restrict__ kap, float2* __restrict__ sig,
+                                                               double* __restrict__ sig_sign, double* __restrict__ e_part,
+                                                               int want_sig, unsigned* __restrict__ rowmax,
+                                                               float* __restrict__ rowpart) {
+  __shared__ float2 sT[CT][CT + 1], sK[CT][CT + 1];
+  __shared__ double red[8];
+  const DressDesc D = desc[blockIdx.y];
+  const bool diag = D.kind == GROUP_CC_DIAG;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nt = (nv + CT - 1) / CT, nup = nt * (nt + 1) / 2;
+  const long nv2 = (long)nv * nv;
+  const float2* T = tau + (long)D.slot * nv2;
+  const float2* K = kap + (long)D.slot * nv2;
+  float2* S0 = want_sig ? sig + (long)D.out * nv2 : nullptr;
+  const dd root3 = dd_from_double(1.7320508075688772935), root2 = dd_from_double(1.4142135623730950488);
+  dd eP = dd_make(0.0f), eQ = dd_make(0.0f);
+  // rows R0 + warp + 8 r of both outputs, over tile column tcol
+  auto magnitudes = [&](const float (&mag)[8], int R0, int tcol) {
+    if (rowpart) {
+      const float n = row_norms8(mag);
+      const int i = lane >> 2, row = R0 + warp + 8 * (i & 3);
+      if ((lane & 3) == 0 && row < nv && !(diag && i >= 4))
+        rowpart[((long)(D.out + (i >> 2)) * ((nv + GT - 1) / GT) + tcol) * nv + row] = n;
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int row = R0 + warp + 8 * (i & 3);
+        const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(mag[i]));
+        if (lane == 0 && row < nv && !(diag && i >= 4)) atomicMax(rowmax + (long)(D.out + (i >> 2)) * nv + row, m);
+      }
+    }
+  };
+  int te = 0, base = 0;
+  for (int t = blockIdx.x; t < nup; t += gridDim.x) {
+    while (t >= base + (nt - te)) {
+      base += nt - te;
+      ++te;
+    }
+    const int tf = te + (t - base), E0 = te * CT, F0 = tf * CT;
+    const bool upper = te != tf;
+    const float w = upper ? 1.0f : 0.5f;
+    float2 a[4], b[4];
+    __syncthreads();  // the last tile's shared elements are read
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int e = E0 + warp + 8 * r, f = F0 + lane, fr = F0 + warp + 8 * r, ec = E0 + lane;
+      const bool in = e < nv && f < nv, ok = fr < nv && ec < nv;
+      a[r] = in ? T[(long)e * nv + f] : make_float2(0.f, 0.f);
+      b[r] = in ? K[(long)e * nv + f] : make_float2(0.f, 0.f);
+      sT[warp + 8 * r][lane] = ok ? T[(long)fr * nv + ec] : make_float2(0.f, 0.f);
+      sK[warp + 8 * r][lane] = ok ? K[(long)fr * nv + ec] : make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int er = warp + 8 * r;
+      const float2 xt = sT[lane][er], xk = sK[lane][er];
+      const dd ta = {a[r].x, a[r].y}, tb = {xt.x, xt.y}, ka = {b[r].x, b[r].y}, kb = {xk.x, xk.y};
+      dd p = dd_add_fast(ta, tb), q = dd_sub_fast(ta, tb);
+      const dd kp = dd_add_fast(ka, kb), kq = dd_sub_fast(ka, kb);
+      eP = dd_fma_acc(eP, dd{p.hi * w, p.lo * w}, kp);  // w = 1 or 1/2: exact
+      eQ = dd_fma_acc(eQ, dd{q.hi * w, q.lo * w}, kq);
+      if (want_sig) {
+        if (diag) p = dd_mul(root2, ta);
+        else q = dd_mul(root3, q);
+        // the transposed positions of this element: read by no other thread
+        a[r] = make_float2(p.hi, p.lo);
+        b[r] = make_float2(q.hi, q.lo);
+      }
+    }
+    if (!want_sig) continue;
+    float mag[8];
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int er = warp + 8 * r, e = E0 + er, f = F0 + lane;
+      const bool in = e < nv && f < nv;
+      if (in) {
+        S0[(long)e * nv + f] = a[r];
+        if (!diag) S0[nv2 + (long)e * nv + f] = b[r];
+      }
+      sT[er][lane] = a[r];
+      sK[er][lane] = b[r];
+      mag[r] = in ? fabsf(a[r].x) : 0.0f;
+      mag[4 + r] = in ? fabsf(b[r].x) : 0.0f;
+    }
+    magnitudes(mag, E0, tf);
+    if (!upper) continue;
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {  // rows f: S[f][e] = P, -Q
+      const int fr = warp + 8 * r, f = F0 + fr, e = E0 + lane;
+      const bool in = f < nv && e < nv;
+      const float2 p = sT[lane][fr], q = sK[lane][fr];
+      if (in) {
+        S0[(long)f * nv + e] = p;
+        if (!diag) S0[nv2 + (long)f * nv + e] = make_float2(-q.x, -q.y);
+      }
+      mag[r] = in ? fabsf(p.x) : 0.0f;
+      mag[4 + r] = in ? fabsf(q.x) : 0.0f;
+    }
+    magnitudes(mag, F0, te);
+  }
+  // over the upper tiles: <P, P_k> + 3 <Q, Q_k>; the pair (m, m) has <P, P_k> = 4 <tau, kappa>, half of it upper
+  double pd = diag ? 0.5 * dd_to_double(eP) : dd_to_double(eP) + 3.0 * dd_to_double(eQ);
+  for (int o = 16; o > 0; o >>= 1) pd += __shfl_down_sync(0xffffffffu, pd, o);
+  if (lane == 0) red[warp] = pd;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+    for (int v = 0; v < 8; ++v) s += red[v];
+    e_part[(long)blockIdx.y * gridDim.x + blockIdx.x] = s;
+  }
+  if (want_sig && blockIdx.x == 0 && threadIdx.x < (diag ? 1 : 2)) sig_sign[D.out + threadIdx.x] = 1.0;
+}
+
 // Double-float form of the group dressing (same structure as dress.cu).
 template <int OCT>
-__global__ void __launch_bounds__(GNT, (OCT == 2) ? 4 : 3)
+__global__ void __launch_bounds__(GNT, 3)
     dress_dd_kernel(int nv, int na, const DressDesc* __restrict__ desc, DressAux aux,
                     const float2* __restrict__ tau, const float2* __restrict__ kap, float2* __restrict__ sig,
                     double* __restrict__ sig_sign, double* __restrict__ e_part, int want_sig,
-                    unsigned* __restrict__ rowmax) {
+                    unsigned* __restrict__ rowmax, float* __restrict__ rowpart) {
   static_assert(OCT % 2 == 0, "coefficients are read two outputs at a time");
-  constexpr int NS = (OCT == 2) ? 1 : MAXSLOT;
+  constexpr int NS = MAXSLOT;
   // float64 coefficients, converted in place to double-float (same size)
   __shared__ __align__(16) union {
     double d[NS][OCT];
@@ -184,10 +347,26 @@ __global__ void __launch_bounds__(GNT, (OCT == 2) ? 4 : 3)
     nk_ = ok ? K[(long)fr * nv + ec] : make_float2(0.f, 0.f);
   };
   dd part = dd_make(0.0f);
-  // OCT = 2 (core pairs): sum_o lambda_o <sigma_o[tau], sigma_o[kappa]> is
-  // accumulated per output and weighted once at the end (two outputs' sums
-  // fit in registers; with 8 outputs they would lower the occupancy)
-  dd eacc[2] = {dd_make(0.0f), dd_make(0.0f)};
+  // one row's 16 elements of a tile (16 lanes share ty), as row_norms8
+  auto magnitude = [&](float v, long mat, int tcol, int row) {
+    if (rowpart) {
+      float x = v * v;
+#pragma unroll
+      for (int w = 8; w > 0; w >>= 1) x += __shfl_xor_sync(0xffffffffu, x, w);
+      float n = sqrtf(x);
+      if (__any_sync(0xffffffffu, !square_in_range(x))) {
+        n = v;
+#pragma unroll
+        for (int w = 8; w > 0; w >>= 1) n = fmaxf(n, __shfl_xor_sync(0xffffffffu, n, w));
+        n *= 4.0f;
+      }
+      if (tx == 0 && row < nv) rowpart[(mat * ((nv + GT - 1) / GT) + tcol) * nv + row] = n;
+    } else if (rowmax) {
+#pragma unroll
+      for (int w = 8; w > 0; w >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, w));
+      if (tx == 0 && row < nv) atomicMax(rowmax + mat * nv + row, __float_as_uint(v));
+    }
+  };
   int t = blockIdx.x, te = 0, tf = 0, buf = 0;
   if (t < nup) {
     decode(t, &te, &tf);
@@ -246,24 +425,13 @@ __global__ void __launch_bounds__(GNT, (OCT == 2) ? 4 : 3)
 #pragma unroll
     for (int o = 0; o < OCT; ++o) {
       if (o < oc) {
-        if constexpr (OCT == 2) {
-          // w = 1 or 2: the scaling of at is exact
-          if (inside) eacc[o] = dd_fma_acc(eacc[o], dd{at[o].hi * w, at[o].lo * w}, ak[o]);
-        } else {
-          if (inside) part = dd_add(part, dd_mul_f(dd_mul(lamw[o], dd_mul(at[o], ak[o])), w));
-        }
+        if (inside) part = dd_add(part, dd_mul_f(dd_mul(lamw[o], dd_mul(at[o], ak[o])), w));
         if (want_sig) {
           const dd v = dd_mul(sqd[o], at[o]);
           const long mat = D.out + D.o_begin + o;
           float2* S = sig + mat * nv2;
           if (inside) S[(long)e * nv + f] = make_float2(v.hi, v.lo);
-          if (rowmax) {
-            // max |hi| of row e over this tile (16 lanes share ty)
-            float m = inside ? fabsf(v.hi) : 0.0f;
-#pragma unroll
-            for (int w = 8; w > 0; w >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, w));
-            if (tx == 0 && e < nv) atomicMax(rowmax + mat * nv + e, __float_as_uint(m));
-          }
+          magnitude(inside ? fabsf(v.hi) : 0.0f, mat, tf, e);
           if (te != tf) {
             sA[ty][tx] = make_float2(v.hi, v.lo);
             __syncthreads();
@@ -271,12 +439,7 @@ __global__ void __launch_bounds__(GNT, (OCT == 2) ? 4 : 3)
             const float sg = sgnf[o];
             const bool ok = fr < nv && ec < nv;
             if (ok) S[(long)fr * nv + ec] = make_float2(sg * sA[tx][ty].x, sg * sA[tx][ty].y);
-            if (rowmax) {
-              float m = ok ? fabsf(sA[tx][ty].x) : 0.0f;
-#pragma unroll
-              for (int w = 8; w > 0; w >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, w));
-              if (tx == 0 && fr < nv) atomicMax(rowmax + mat * nv + fr, __float_as_uint(m));
-            }
+            magnitude(ok ? fabsf(sA[tx][ty].x) : 0.0f, mat, te, fr);
             __syncthreads();
           }
         }
@@ -285,11 +448,6 @@ __global__ void __launch_bounds__(GNT, (OCT == 2) ? 4 : 3)
     t = tn;
     te = ten;
     tf = tfn;
-  }
-  if constexpr (OCT == 2) {
-#pragma unroll
-    for (int o = 0; o < 2; ++o)
-      if (o < oc) part = dd_add(part, dd_mul(lamw[o], eacc[o]));
   }
   double pd = dd_to_double(part);
   for (int o = 16; o > 0; o >>= 1) pd += __shfl_down_sync(0xffffffffu, pd, o);
@@ -386,18 +544,18 @@ int pair_epilogue_dd(const Geometry& g, const double* eps, const float2* eps_dd,
 
 int dress_dd(const Geometry& g, const DressDesc* d_desc, int ndesc, int ncc, const DressAux& aux,
              const float2* tau, const float2* kap, float2* sig, double* sig_sign, double* e_part, bool want_sig,
-             unsigned* rowmax, cudaStream_t st) {
+             unsigned* rowmax, float* rowpart, cudaStream_t st) {
   if (ncc > 0) {
     dim3 grid(DRESS_TILE_BLOCKS, ncc);
-    dress_dd_kernel<2><<<grid, GNT, 0, st>>>(g.nv, g.na, d_desc, aux, tau, kap, sig, sig_sign, e_part,
-                                             want_sig ? 1 : 0, rowmax);
+    dress_core_dd_kernel<<<grid, 256, 0, st>>>(g.nv, d_desc, tau, kap, sig, sig_sign, e_part, want_sig ? 1 : 0, rowmax,
+                                               rowpart);
     DSRG_LAUNCH_CHECK();
   }
   if (ndesc > ncc) {
     dim3 grid(DRESS_TILE_BLOCKS, ndesc - ncc);
     dress_dd_kernel<DRESS_OC><<<grid, GNT, 0, st>>>(g.nv, g.na, d_desc + ncc, aux, tau, kap, sig, sig_sign,
                                                     e_part + (long)ncc * DRESS_TILE_BLOCKS, want_sig ? 1 : 0,
-                                                    rowmax);
+                                                    rowmax, rowpart);
     DSRG_LAUNCH_CHECK();
   }
   return DSRG_FNO_OK;

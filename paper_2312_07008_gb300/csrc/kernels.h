@@ -163,7 +163,10 @@ int stage_literal(int form, int KS, const double* src, long R, int K, long rs, l
                   int* exps, cudaStream_t st);
 // Residue form (residue.cu): the fast form's contractions modulo RES_MOD (or,
 // for the rotation of B, RES_MOD_X) coprime moduli on tcgen05, one product each.
-constexpr int RES_MOD = 10, RES_MOD_X = 12;
+// RES_MOD_S: the rank-K update of D_vv, whose sums run over whole segments of
+// dressed matrices: its errors average out over K = 10^4 and more (relative to
+// the rows' norms 2^-40 and less), the digit planes' were 2^-37.
+constexpr int RES_MOD = 10, RES_MOD_X = 12, RES_MOD_S = 9;
 constexpr int RES_TILE = 256;          // rows and columns of an output tile
 constexpr int RES_STAGE_BLOCKS = 608;  // four blocks per SM of a staging launch
 // bytes of the exponents of R staged rows and of the staging's scratch behind them
@@ -187,6 +190,10 @@ constexpr int RES_MAX_SEGMENTS = 64;
 struct ResSegment {
   int r0, r1, sign, scale;  // scale: index of the range's row exponents
 };
+size_t residue_syrk_res_bytes(int nv);
+int residue_syrk(int nv, int nr, int n_signed, const float2* sig, const float* rowpart, const double* sign,
+                 __nv_bfloat16* planes, int* exps, int* scale_of, int Kpad, uint16_t* res, double* D, int* err,
+                 cudaStream_t st);
 void* tensor_map_encoder();  // cuTensorMapEncodeTiled, or null
 // double-float elementwise stages (dd_stages.cu)
 int eps_to_dd(int n, const double* eps, float2* out, cudaStream_t st);
@@ -198,10 +205,12 @@ int hole_particle_dd(const Geometry& g, const double* eps, float2* out, cudaStre
 int pair_epilogue_dd(const Geometry& g, const double* eps, const float2* eps_dd, const int2* pairs, int npairs,
                      const float2* nu, float2* tau, float2* kap, double* ts, cudaStream_t st);
 // rowmax: NULL, or [nout][nv] zeroed words receiving max |hi| of each row of
-// the dressed matrices written (float bits, atomicMax)
+// the dressed matrices written (float bits, atomicMax); rowpart: NULL, or
+// [nout][ceil(nv / 16)][nv] words receiving a bound of each row's norm in each tile
+// column instead (tiles of 32 for the core pairs' matrices, else of 16)
 int dress_dd(const Geometry& g, const DressDesc* d_desc, int ndesc, int ncc, const DressAux& aux,
              const float2* tau, const float2* kap, float2* sig, double* sig_sign, double* e_part, bool want_sig,
-             unsigned* rowmax, cudaStream_t st);
+             unsigned* rowmax, float* rowpart, cudaStream_t st);
 int regularize_test(int n, const double* delta, double s, double* r1, double* y, cudaStream_t st);
 int sliced_syrk(int KS, int nv, int nr, const __nv_bfloat16* planes, const int* exps, int Kpad,
                 const double* sign, double* dpart, int nsplit, double* D, int* err, cudaStream_t st);

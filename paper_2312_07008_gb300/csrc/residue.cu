@@ -20,9 +20,28 @@ using namespace res;
 
 // ---------------------------------------------------------------- staging
 __device__ __forceinline__ double square_of(double v) { return v * v; }
+__device__ __forceinline__ double square_of(float2 v) {
+  const double x = (double)v.x + (double)v.y;
+  return x * x;
+}
 __device__ __forceinline__ double zero_like(double) { return 0.0; }
+__device__ __forceinline__ float2 zero_like(float2) { return make_float2(0.f, 0.f); }
 
 __device__ __forceinline__ long long integer_of(double v, int f) { return scaled_integer(v, f); }
+
+// hi + lo with the same rule, exactly in 64-bit fixed point with 16 guard bits
+__device__ __forceinline__ long long fixed_of(float v, int f) {
+  const int b = __float_as_int(v), E = (b >> 23) & 0xFF;
+  if (E == 0) return 0;
+  const long long m = (long long)((b & 0x7FFFFF) | 0x800000);
+  const int sh = E - 150 + f + 16;
+  const long long x = sh >= 0 ? (sh < 39 ? m << sh : 0) : (-sh < 63 ? m >> -sh : 0);
+  return b < 0 ? -x : x;
+}
+__device__ __forceinline__ long long integer_of(float2 v, int f) {
+  const long long x = fixed_of(v.x, f) + fixed_of(v.y, f);
+  return x >= 0 ? (x + 0x8000) >> 16 : -((-x + 0x8000) >> 16);
+}
 
 // Squared norms of the rows: part[split][row] over the split's share of k.
 // Source element (row, k) at src[row rs + k ks]; one of rs, ks is 1.
@@ -610,6 +629,100 @@ __global__ void __launch_bounds__(256) plain_residue_kernel(ResGemm P, PlainOut 
   }
 }
 
+// Rank-K update of D_vv, sums over all rows of all dressed matrices: bound by the
+// tensor cores.  opdm pass of nvir 1200 (10 active, K = 6.8e6): the products take
+// 65 ms (1.62 PFLOP/s) instead of the digit planes' 120; the staging 40 ms instead
+// of 28, for nine planes instead of five.  Row by row of D: sums over the
+// segments, in their order, of sign A_s[e] . A_s[f] (upper tiles, mirrored).
+__global__ void __launch_bounds__(256) syrk_residue_kernel(ResGemm P, const int* __restrict__ exps, int nv, double* D) {
+  constexpr int NM = RES_MOD_S;
+  int mt, nt;
+  rg_tile(P, blockIdx.y, &mt, &nt);
+  const int e = mt * GT_M + threadIdx.x;
+  if (e >= nv) return;
+  const int g = blockIdx.x, f0 = nt * GT_M + g * 8;
+  if (f0 >= nv || f0 + 7 < e) return;
+  double acc[8] = {};
+  for (int s = 0; s < P.nseg; ++s) {
+    const int* ex = exps + (long)P.seg[s].scale * nv;
+    uint32_t w[NM][4];
+    load_residues<NM>(P.res + (((long)s * P.ntiles + blockIdx.y) * NM) * GT_M * GT_M + threadIdx.x * 8, g, w);
+    const int ee = ex[e];
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+      if (f0 + c < nv) {
+        const double v = fraction_f64<NM>(recombine<NM>(w, c), ee + ex[f0 + c]);
+        acc[c] += P.seg[s].sign < 0 ? -v : v;
+      }
+  }
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const int f = f0 + c;
+    if (f >= nv || f < e) continue;
+    const double v = D[(long)e * nv + f] + acc[c];
+    D[(long)e * nv + f] = v;
+    if (f != e) D[(long)f * nv + e] += acc[c];
+  }
+}
+
+// -f of row e of scale group s, from its norm over the group's matrices: the
+// bounds of the tiles' rows (32 columns for the first n_core matrices, 16 for the
+// others).  Eight threads per row, each its share of the matrices in a fixed order.
+__global__ void __launch_bounds__(256) segment_shift_kernel(int nv, int n_core, ResGemm P, const float* __restrict__ rowpart,
+                                                            int* __restrict__ exps) {
+  __shared__ double red[8][32];
+  const int lane = threadIdx.x & 31, part = threadIdx.x >> 5, e = blockIdx.x * 32 + lane, s = blockIdx.y;
+  if (P.seg[s].sign < 0) return;  // the two signs of a range share its scales
+  constexpr double LIMIT = norm_limit(RES_MOD_S);
+  double x = 0.0;
+  const int stride = (nv + 15) / 16;
+  if (e < nv)
+    for (int r = P.seg[s].r0 + part; r < P.seg[s].r1; r += 8) {
+      const int w = r < n_core ? 32 : 16, nt = (nv + w - 1) / w;
+      const float* p = rowpart + (long)r * stride * nv + e;
+      double y = 0.0;
+      for (int t = 0; t < nt; ++t) {
+        const double m = p[(long)t * nv];
+        y = fma(m, m, y);
+      }
+      x += y;
+    }
+  red[part][lane] = x;
+  __syncthreads();
+  if (part != 0 || e >= nv) return;
+#pragma unroll
+  for (int q = 1; q < 8; ++q) x += red[q][lane];
+  // |hi + lo| <= |hi| (1 + 2^-23); float32 sums of up to 32 squares and their root
+  const int f = row_shift(x * (1.0 + 1e-5), (P.seg[s].r1 - P.seg[s].r0) * nv, LIMIT);
+  exps[(long)P.seg[s].scale * nv + e] = -f;
+}
+
+// Residue planes [RES_MOD_S][nr][nv][Kpad] of the dressed matrices (double-float
+// rows, contiguous), scaled by their segment's row exponents.  Bound by memory: 8
+// bytes read and 18 written per element.
+__global__ void __launch_bounds__(256) residue_dressed_kernel(const float2* __restrict__ src, int nv, int nr, int Kpad,
+                                                              const int* __restrict__ exps, const int* __restrict__ scale_of,
+                                                              __nv_bfloat16* __restrict__ planes) {
+  const long R = (long)nr * nv, row = (long)blockIdx.x * 32 + (threadIdx.x >> 3);
+  if (row >= R) return;
+  const int r = (int)(row / nv), e = (int)(row - (long)r * nv);
+  int f = -exps[(long)scale_of[r] * nv + e];
+  if (f == SHIFT_INVALID) f = 0;
+  for (int k0 = (threadIdx.x & 7) * 8; k0 < Kpad; k0 += 64) {
+    const float2* p = src + row * nv + k0;
+    Pieces<3> x[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) x[j] = pieces_of<3>(k0 + j < nv ? integer_of(p[j], f) : 0);
+#pragma unroll
+    for (int i = 0; i < RES_MOD_S; ++i) {
+      __nv_bfloat162 h[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) h[j] = __floats2bfloat162_rn(residue<RES_MOD_S>(x[2 * j], i), residue<RES_MOD_S>(x[2 * j + 1], i));
+      *reinterpret_cast<uint4*>(planes + ((long)i * R + row) * Kpad + k0) = *reinterpret_cast<uint4*>(h);
+    }
+  }
+}
+
 // ------------------------------------------------------- host side helpers
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -784,6 +897,79 @@ int residue_plain(int nm, int M, int N, const __nv_bfloat16* pa, const int* ea, 
     else plain_residue_kernel<RES_MOD_X><<<grid, 256, 0, st>>>(P, O);
     DSRG_LAUNCH_CHECK();
   }
+  return DSRG_FNO_OK;
+}
+
+// Segments of the rank-K update over nr matrices of which those from n_signed
+// on may carry a minus sign: every range of scales is one segment, or two (one
+// per sign).  Eight to 16 ranges bound the error (a range's rows share one
+// scale) and fill the pairs of SMs: their count is the one whose units leave
+// the least of the last round idle.
+int residue_segments(int nv, int nr, int n_signed, ResSegment* seg) {
+  const int nt = ceil_div(nv, GT_M), units = nt * (nt + 1) / 2 * RES_MOD_S, pairs = 76;
+  int best = 8;
+  double best_eff = 0.0;
+  for (int k = 8; k <= 16; ++k) {
+    const long u = (long)units * k;
+    const double eff = (double)u / ((double)ceil_div(u, pairs) * pairs);
+    if (eff > best_eff + 0.005) {
+      best_eff = eff;
+      best = k;
+    }
+  }
+  int n = 0, scale = 0;
+  auto add = [&](int b, int e, int count, bool both) {
+    count = std::max(1, std::min(count, e - b));
+    for (int k = 0; k < count; ++k) {
+      const int r0 = b + (int)((long)(e - b) * k / count), r1 = b + (int)((long)(e - b) * (k + 1) / count);
+      seg[n++] = ResSegment{r0, r1, both ? 1 : 0, scale};
+      if (both) seg[n++] = ResSegment{r0, r1, -1, scale};
+      ++scale;
+    }
+  };
+  // shares of the ranges in proportion to the matrices, at least one each
+  const int plain = std::min(n_signed, nr), sg = nr - plain;
+  if (plain > 0) add(0, plain, std::max(1, (int)((long)best * plain / nr)), false);
+  if (sg > 0) add(plain, nr, std::max(1, best - (plain > 0 ? std::max(1, (int)((long)best * plain / nr)) : 0)), true);
+  return n;
+}
+
+size_t residue_syrk_res_bytes(int nv) {
+  const int nt = ceil_div(nv, GT_M);
+  return (size_t)RES_MAX_SEGMENTS / 2 * (nt * (nt + 1) / 2) * residue_tile_bytes(RES_MOD_S);
+}
+
+// D += sum_r sign_r Sig_r Sig_r^T.  rowpart: as dress_dd writes it; exps: RES_MAX_SEGMENTS nv ints; scale_of: nr ints (host list, copied).
+int residue_syrk(int nv, int nr, int n_signed, const float2* sig, const float* rowpart, const double* sign,
+                 __nv_bfloat16* planes, int* exps, int* scale_of, int Kpad, uint16_t* res, double* D, int* err,
+                 cudaStream_t st) {
+  if (nr <= 0 || nv <= 0) return DSRG_FNO_OK;
+  ResGemm P{};
+  P.mode = RG_SYRK;
+  P.nm = RES_MOD_S;
+  P.ntm = P.ntn = ceil_div(nv, GT_M);
+  P.ntiles = P.ntm * (P.ntm + 1) / 2;
+  P.nseg = residue_segments(nv, nr, n_signed, P.seg);
+  P.nr = nr;
+  P.nunits = (long)P.nseg * P.nm * P.ntiles;
+  P.sign = sign;
+  P.res = res;
+  P.err = err;
+  std::vector<int> so(nr);
+  for (int s = 0; s < P.nseg; ++s)
+    for (int r = P.seg[s].r0; r < P.seg[s].r1; ++r) so[r] = P.seg[s].scale;
+  DSRG_CUDA(cudaMemcpyAsync(scale_of, so.data(), sizeof(int) * nr, cudaMemcpyHostToDevice, st));
+  {
+    DSRG_PHASE("phase_stage_sig", st);
+    segment_shift_kernel<<<dim3(ceil_div(nv, 32), P.nseg), 256, 0, st>>>(nv, n_signed, P, rowpart, exps);
+    DSRG_LAUNCH_CHECK();
+    residue_dressed_kernel<<<(unsigned)ceil_div((long)nr * nv, 32), 256, 0, st>>>(sig, nv, nr, Kpad, exps, scale_of,
+                                                                                  planes);
+    DSRG_LAUNCH_CHECK();
+  }
+  DSRG_TRY(launch_gemm(planes, nv, planes, nv, Kpad, P, st));
+  syrk_residue_kernel<<<dim3(32, P.ntiles), 256, 0, st>>>(P, exps, nv, D);
+  DSRG_LAUNCH_CHECK();
   return DSRG_FNO_OK;
 }
 
