@@ -10,8 +10,11 @@
 // SMs: 5.7e6 clocks of the whole chip for n = 1200.  The rest are the n grid
 // barriers of the reduction.  A Jacobi solve moves the whole matrix n - 1
 // times per sweep with a barrier each time and needs 4 to 10 sweeps.  Measured
-// (D_vv-like matrices): n = 1200 27 ms (column-pair Jacobi in double-float 97
-// ms), n = 203 3.1 (9.1), n = 90 1.5 (2.7), n = 3600 0.58 s (4.8 s).
+// (D_vv-like matrices): n = 1200 18.5 ms (column-pair Jacobi in double-float 97
+// ms), n = 203 1.95 (9.1), n = 90 0.92 (2.7), n = 3600 0.36 s (4.8 s).  Against
+// the first form of these kernels (27, 3.1, 1.5 ms): leaves of 8 rows instead of
+// 16, deflation by all threads of a block, reciprocals and roots by iteration
+// instead of the library's, scalar work by one warp.
 #include <algorithm>
 
 #include "eig_dc.cuh"
@@ -50,11 +53,13 @@ __device__ bool tri_barrier(const TriArgs& P, unsigned target) {
   if (threadIdx.x == 0) {
     __threadfence();
     atomicAdd(P.bar, 1u);
-    volatile unsigned* cnt = P.bar;
     volatile int* st = P.status + 1;
     long long it = 0;
     int ok = 1;
-    while ((int)(*cnt - target) < 0) {
+    unsigned cnt;
+    while (true) {
+      asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(cnt) : "l"(P.bar) : "memory");
+      if ((int)(cnt - target) >= 0) break;
       if (++it > P.spin_limit) {
         atomicExch(P.status + 1, 1);
         ok = 0;
@@ -65,18 +70,13 @@ __device__ bool tri_barrier(const TriArgs& P, unsigned target) {
         break;
       }
     }
-    __threadfence();
-    s_ok = ok && *st == 0;
+    s_ok = ok;
   }
   __syncthreads();
   return s_ok != 0;
 }
 
-__device__ __forceinline__ double warp_sum(double x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-  return x;
-}
+__device__ __forceinline__ double warp_sum(double x) { return WarpLane().sum(x); }
 
 // Step j: every block knows row j of the reduced matrix (r), forms the same
 // reflector from it, and in ONE pass over its own rows applies the rank-2
@@ -86,7 +86,9 @@ __device__ __forceinline__ double warp_sum(double x) {
 // The products p', their dot with v' and row j + 1 are published, and one grid
 // barrier later every block forms row j + 1 of the next matrix by itself: one
 // barrier per step, A read and written once per step, from shared memory as
-// long as a block's rows fit (SM).
+// long as a block's rows fit (SM).  (One cluster of 16 blocks for small n, its
+// hardware barrier and shared memory in place of the grid barrier and the
+// published arrays, took the same 6 us per step at n = 203.)
 template <bool SM>
 __global__ void __launch_bounds__(TNT) tridiag_kernel(TriArgs P) {
   extern __shared__ double smem[];
@@ -95,8 +97,15 @@ __global__ void __launch_bounds__(TNT) tridiag_kernel(TriArgs P) {
   double* v0 = pv + n;      // v of the previous step
   double* v1 = v0 + n;      // v of this step
   double* As = v1 + n;      // own rows (SM)
-  __shared__ double red[TNW];
+  __shared__ double part[TNT], sc[4];
   auto row_ptr = [&](int li) { return SM ? As + (long)li * n : P.A + (long)(b + li * G) * n; };
+  // sum of the threads' parts, by warp 0 (scalar work costs every warp that
+  // repeats it 16 clocks an instruction of the SM's float64 lanes)
+  auto total = [&]() {
+    static_assert(TNW == 8, "a tree of eight");
+    const double* x = part + lane;
+    return warp_sum(((x[0] + x[32]) + (x[64] + x[96])) + ((x[128] + x[160]) + (x[192] + x[224])));
+  };
   if (SM) {
     for (int li = warp; b + li * G < n; li += TNW) {
       const double* src = P.A + (long)(b + li * G) * n;
@@ -104,36 +113,41 @@ __global__ void __launch_bounds__(TNT) tridiag_kernel(TriArgs P) {
       for (int k = lane; k < n; k += 32) dst[k] = src[k];
     }
   }
-  double dj = P.A[0], alpha = P.A[1], s2 = 0.0;
+  double dj = P.A[0], alpha = P.A[1], s2 = 0.0;  // dj, alpha: warp 0's
   for (int k = 1 + tid; k < n; k += TNT) {
     const double r = P.A[k];
     v1[k] = r;
-    if (k > 1) s2 += r * r;
+    if (k > 1) s2 = fma(r, r, s2);
   }
   unsigned target = G;
   if (!tri_barrier(P, target)) return;  // every block has read its part of A
   double beta0 = 0.0, K2 = 0.0;         // of the previous step (none yet)
   for (int j = 0; j < n - 2; ++j) {
     // ---- reflector from row j (v1 holds A[j][k], k > j; s2 this thread's part of |r_{k > j + 1}|^2)
-    s2 = warp_sum(s2);
-    if (lane == 0) red[warp] = s2;
+    part[tid] = s2;
     __syncthreads();
-    double sig = 0.0;
-#pragma unroll
-    for (int w = 0; w < TNW; ++w) sig += red[w];
-    double ej = alpha, beta = 0.0;
-    if (sig > 0.0) {
-      const double nrm = sqrt(alpha * alpha + sig);
-      ej = alpha > 0.0 ? -nrm : nrm;
-      beta = 1.0 / (nrm * (nrm + fabs(alpha)));
-      if (tid == ((j + 1) % TNT)) v1[j + 1] = alpha - ej;
+    if (warp == 0) {
+      const double sig = total();
+      double ej = alpha, bt = 0.0, v = alpha;
+      if (sig > 0.0) {
+        // beta = 1 / (nrm (nrm + |alpha|))
+        const double q = fma(alpha, alpha, sig), r = dc_rsqrt(q), nrm = q * r;
+        ej = alpha > 0.0 ? -nrm : nrm;
+        bt = r * r * dc_rcp(fma(fabs(alpha), r, 1.0));
+        v = alpha - ej;
+      }
+      if (lane == 0) {
+        v1[j + 1] = v;
+        sc[0] = bt;
+        if (b == 0) {
+          P.d[j] = dj;
+          P.e[j] = ej;
+          P.beta[j] = bt;
+        }
+      }
     }
     __syncthreads();
-    if (b == 0 && tid == 0) {
-      P.d[j] = dj;
-      P.e[j] = ej;
-      P.beta[j] = beta;
-    }
+    const double beta = sc[0];
     if (b == j % G)
       for (int k = j + 1 + tid; k < n; k += TNT) P.A[(long)j * n + k] = v1[k];
     // ---- own rows: pending update and product with the new reflector
@@ -141,86 +155,87 @@ __global__ void __launch_bounds__(TNT) tridiag_kernel(TriArgs P) {
     double* pp = P.pub_p + (long)buf * n;
     double* pr = P.pub_row + (long)buf * n;
     double sw = 0.0;
-    int li0 = b > j ? 0 : (j - b) / G + 1;  // first own row above j
+    const int li0 = b > j ? 0 : (j - b) / G + 1;  // first own row above j
     const int kbeg = (j + 1) & ~31;
     for (int li = li0 + warp; b + li * G < n; li += TNW) {
       const int i = b + li * G;
       double* row = row_ptr(li);
-      const double c1 = beta0 * v0[i], c2 = beta0 * pv[i] - K2 * v0[i];
-      double acc = 0.0;
+      const double c1 = -beta0 * v0[i], c2 = fma(K2, v0[i], -beta0 * pv[i]);
+      // four partial sums: a chain of float64 FMAs waits for each of them
+      double acc[4] = {0.0, 0.0, 0.0, 0.0};
       const bool pub = i == j + 1;
-      if (j > 0) {
-#pragma unroll 4
-        for (int k = kbeg + lane; k < n; k += 32) {
-          if (k > j) {
-            const double a = row[k] - fma(c1, pv[k], c2 * v0[k]);
-            row[k] = a;
-            acc = fma(a, v1[k], acc);
-            if (pub) __stcg(pr + k, a);
-          }
-        }
-      } else {
-#pragma unroll 4
-        for (int k = kbeg + lane; k < n; k += 32) {
-          if (k > j) {
-            const double a = row[k];
-            acc = fma(a, v1[k], acc);
+      for (int k0 = kbeg + lane; k0 < n; k0 += 128) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int k = k0 + 32 * u;
+          if (k > j && k < n) {
+            double a = row[k];
+            if (j > 0) {
+              a = fma(c1, pv[k], fma(c2, v0[k], a));
+              row[k] = a;
+            }
+            acc[u] = fma(a, v1[k], acc[u]);
             if (pub) __stcg(pr + k, a);
           }
         }
       }
-      acc = warp_sum(acc);
-      if (lane == 0) {
-        __stcg(pp + i, acc);
-        sw = fma(acc, v1[i], sw);
-      }
+      double ps = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+      sw = fma(ps, v1[i], sw);  // p.v in lane parts
+      ps = warp_sum(ps);
+      if (lane == 0) __stcg(pp + i, ps);
       if (j == n - 3 && i == n - 1) {  // the last diagonal element (its lane wrote it)
         __syncwarp();
         if (lane == 0) __stcg(pr, row[n - 1]);
       }
     }
-    if (lane == 0) red[warp] = sw;
+    part[tid] = sw;
     __syncthreads();
-    if (tid == 0) {
-      double s = 0.0;
-#pragma unroll
-      for (int w = 0; w < TNW; ++w) s += red[w];
-      __stcg(P.pub_s + buf * EIG_MAX_BLOCKS + b, s);
+    if (warp == 0) {
+      const double s = total();
+      if (lane == 0) __stcg(P.pub_s + buf * EIG_MAX_BLOCKS + b, s);
     }
     target += G;
     if (!tri_barrier(P, target)) return;
     // ---- p, p.v and row j + 1 of the next matrix
-    double s = 0.0;
-    for (int g = tid; g < G; g += TNT) s += __ldcg(P.pub_s + buf * EIG_MAX_BLOCKS + g);
-    s = warp_sum(s);
-    if (lane == 0) red[warp] = s;
-    for (int k = j + 1 + tid; k < n; k += TNT) pv[k] = __ldcg(pp + k);
+    const int i = j + 1;
     double* vt = v0;
     v0 = v1;
     v1 = vt;
-    __syncthreads();
-    s = 0.0;
-#pragma unroll
-    for (int w = 0; w < TNW; ++w) s += red[w];
-    K2 = beta * beta * s;
+    for (int k = i + tid; k < n; k += TNT) {
+      pv[k] = __ldcg(pp + k);
+      v1[k] = __ldcg(pr + k);
+    }
     beta0 = beta;
-    const int i = j + 1;
-    const double c1 = beta0 * v0[i], c2 = beta0 * pv[i] - K2 * v0[i];
-    dj = __ldcg(pr + i) - fma(c1, pv[i], c2 * v0[i]);
-    alpha = __ldcg(pr + i + 1) - fma(c1, pv[i + 1], c2 * v0[i + 1]);
+    if (warp == 0) {
+      const double pi = __ldcg(pp + i), pi1 = __ldcg(pp + i + 1), ri = __ldcg(pr + i), ri1 = __ldcg(pr + i + 1);
+      double s = 0.0;
+      for (int g = lane; g < G; g += 32) s += __ldcg(P.pub_s + buf * EIG_MAX_BLOCKS + g);
+      s = warp_sum(s);
+      const double k2 = beta * (beta * s), vi = v0[i];  // beta^2 may overflow
+      const double c1 = -beta * vi, c2 = fma(k2, vi, -beta * pi);
+      dj = fma(c1, pi, fma(c2, vi, ri));
+      alpha = fma(c1, pi1, fma(c2, v0[i + 1], ri1));
+      if (lane == 0) {
+        sc[1] = k2;
+        sc[2] = c1;
+        sc[3] = c2;
+        if (j == n - 3 && b == 0) {
+          const double pl = __ldcg(pp + n - 1), vl = v0[n - 1];
+          P.d[n - 2] = dj;
+          P.e[n - 2] = alpha;
+          P.d[n - 1] = fma(-beta * vl, pl, fma(fma(k2, vl, -beta * pl), vl, __ldcg(pr)));
+        }
+      }
+    }
+    __syncthreads();
+    K2 = sc[1];
+    const double c1 = sc[2], c2 = sc[3];
     s2 = 0.0;
     for (int k = i + 1 + tid; k < n; k += TNT) {
-      const double r = __ldcg(pr + k) - fma(c1, pv[k], c2 * v0[k]);
+      const double r = fma(c1, pv[k], fma(c2, v0[k], v1[k]));
       v1[k] = r;
       if (k > i + 1) s2 = fma(r, r, s2);
     }
-    if (j == n - 3 && b == 0 && tid == 0) {
-      const double cl = beta0 * v0[n - 1], cm = beta0 * pv[n - 1] - K2 * v0[n - 1];
-      P.d[n - 2] = dj;
-      P.e[n - 2] = alpha;
-      P.d[n - 1] = __ldcg(pr) - fma(cl, pv[n - 1], cm * v0[n - 1]);
-    }
-    __syncthreads();  // red is reused
   }
 }
 
@@ -281,10 +296,8 @@ __global__ void __launch_bounds__(32) dc_leaf_kernel(DcArgs P) {
     Q[i][k] = i == k ? 1.0 : 0.0;
   }
   __syncwarp();
-  double big = 0.0;
-  for (int i = 0; i < m; ++i)
-    for (int k = max(0, i - 1); k <= min(m - 1, i + 1); ++k) big = fmax(big, fabs(A[i][k]));
-  const double floor_ = 0.125 * DC_EPS * big;
+  const double anorm = *P.anorm, floor_ = 4.0 * DC_EPS * anorm;  // the deflation's tolerance
+  const double unit = dc_rcp(anorm);                             // (unused when all entries are 0)
   for (int sweep = 0; sweep < 16 && m > 1; ++sweep) {
     bool any = false;
     for (int r = 0; r < me - 1; ++r) {
@@ -296,11 +309,13 @@ __global__ void __launch_bounds__(32) dc_leaf_kernel(DcArgs P) {
         if (q < m) {
           const double apq = A[p][q];
           if (fabs(apq) > floor_) {
-            const double th = (A[q][q] - A[p][p]) / (2.0 * apq);
-            const double t = (th >= 0.0 ? 1.0 : -1.0) / (fabs(th) + sqrt(1.0 + th * th));
-            c = 1.0 / sqrt(1.0 + t * t);
-            s = t * c;
-            any = true;
+            // tan in float32: any t gives an orthogonal rotation, and the next
+            // sweep takes off what this one leaves
+            const float th = (float)((A[q][q] - A[p][p]) * unit) / (2.0f * (float)(apq * unit));
+            const float t = copysignf(1.0f, th) / (fabsf(th) + sqrtf(fmaf(th, th, 1.0f)));
+            c = dc_rsqrt(fma((double)t, (double)t, 1.0));
+            s = (double)t * c;
+            any = any || t != 0.0f;
           }
         }
         pp[lane] = p;
@@ -356,10 +371,10 @@ __global__ void __launch_bounds__(256) dc_deflate_kernel(DcArgs P) {
   const int lo = dc_bound(n, l, t), hi = dc_bound(n, l, t + 1), mid = dc_bound(n, l + 1, 2 * t + 1), m = hi - lo;
   double* sd = sm;                                            // [m] sorted
   double* sz = sd + m;                                        // [m]
-  long long* key = reinterpret_cast<long long*>(sz + m);      // [m] unsorted keys; then the kept columns' types
+  long long* key = reinterpret_cast<long long*>(sz + m);      // [m] unsorted keys; then ci and kty
   int* ord = reinterpret_cast<int*>(key + m);                 // [m]
   unsigned char* ty = reinterpret_cast<unsigned char*>(ord + m);  // [m]
-  unsigned char* kty = reinterpret_cast<unsigned char*>(key);
+  unsigned char* fl = ty + m;                                     // [m]
   __shared__ int s_k, s_nr;
   const double ec = P.e[mid - 1], rho = 2.0 * fabs(ec);
   for (int i = threadIdx.x; i < m; i += 256) key[i] = dc_key(P.lam[lo + i]);
@@ -376,10 +391,51 @@ __global__ void __launch_bounds__(256) dc_deflate_kernel(DcArgs P) {
     ty[r] = top ? 1 : 3;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
+  const double tol = 4.0 * DC_EPS * *P.anorm;
+  int* ci = reinterpret_cast<int*>(key);                          // [m] ranks of the columns with a z to speak of
+  unsigned char* kty = reinterpret_cast<unsigned char*>(ci + m);  // [m]
+  __shared__ int s_cnt[256];
+  const int per = (m + 255) / 256, r0 = min(m, (int)threadIdx.x * per), r1 = min(m, r0 + per);
+  int cnt = 0;
+  for (int r = r0; r < r1; ++r) {
+    fl[r] = dc_flag(r, sd, sz, rho, tol);
+    cnt += !(fl[r] & 1);
+  }
+  s_cnt[threadIdx.x] = cnt;
+  __syncthreads();
+  for (int w = 1; w < 256; w <<= 1) {  // inclusive scan
+    const int x = (int)threadIdx.x >= w ? s_cnt[threadIdx.x - w] : 0;
+    __syncthreads();
+    s_cnt[threadIdx.x] += x;
+    __syncthreads();
+  }
+  int pos = s_cnt[threadIdx.x] - cnt;
+  const int kept = s_cnt[255];
+  for (int r = r0, q = pos; r < r1; ++r)
+    if (!(fl[r] & 1)) ci[q++] = r;
+  __syncthreads();
+  bool close = false;
+  for (int q = threadIdx.x + 1; q < kept; q += 256) close = close || dc_close(sd[ci[q - 1]], sz[ci[q - 1]], sd[ci[q]], sz[ci[q]], tol);
+  if (!__syncthreads_or(close)) {
+    // no pair to rotate (the usual case): the split by z is all of it
+    for (int r = r0; r < r1; ++r) {
+      if (!(fl[r] & 1)) {
+        P.kcol[lo + pos] = ord[r];
+        P.kd[lo + pos] = sd[r];
+        P.kz[lo + pos] = sz[r];
+        kty[pos++] = ty[r];
+      } else {
+        P.dcol[lo + r - pos] = ord[r];
+        P.dval[lo + r - pos] = sd[r];
+      }
+    }
+    if (threadIdx.x == 0) {
+      s_k = kept;
+      s_nr = 0;
+    }
+  } else if (threadIdx.x == 0) {
     int nr = 0;
-    const double tol = 4.0 * DC_EPS * *P.anorm;
-    s_k = dc_deflate(m, ord, sd, sz, ty, rho, tol, P.kcol + lo, P.kd + lo, P.kz + lo, kty, P.dcol + lo, P.dval + lo,
+    s_k = dc_deflate(m, ord, sd, sz, fl, ty, rho, tol, P.kcol + lo, P.kd + lo, P.kz + lo, kty, P.dcol + lo, P.dval + lo,
                      P.rot + lo, &nr);
     s_nr = nr;
   }
@@ -447,16 +503,16 @@ __device__ void dc_rotate_rows(const DcArgs& P, int row) {
 }
 
 // Blocks [0, rot_blocks): the rotations; the others: a warp per column, which
-// solves the secular equation of a kept one and hands on a deflated one's value.
-__global__ void __launch_bounds__(128) dc_secular_kernel(DcArgs P, int rot_blocks) {
+// solves the secular equation of a kept one and hands on a deflated one's value
+// (one warp per block: the warps spread over all SMs' float64 lanes).
+__global__ void __launch_bounds__(32) dc_secular_kernel(DcArgs P, int rot_blocks) {
   const int n = P.n;
   if ((int)blockIdx.x < rot_blocks) {
-    const int row = blockIdx.x * 128 + threadIdx.x;
+    const int row = blockIdx.x * 32 + threadIdx.x;
     if (row < n) dc_rotate_rows(P, row);
     return;
   }
-  const int i = ((int)blockIdx.x - rot_blocks) * 4 + (threadIdx.x >> 5);
-  if (i >= n) return;
+  const int i = (int)blockIdx.x - rot_blocks;
   const int t = dc_node_of(n, P.level, i), lo = dc_bound(n, P.level, t), mid = dc_bound(n, P.level + 1, 2 * t + 1);
   const int K = P.node[t].x, j = i - lo;
   const WarpLane L;
@@ -475,9 +531,8 @@ __global__ void __launch_bounds__(128) dc_secular_kernel(DcArgs P, int rot_block
   }
 }
 
-__global__ void __launch_bounds__(128) dc_zhat_kernel(DcArgs P) {
-  const int n = P.n, i = blockIdx.x * 4 + (threadIdx.x >> 5);
-  if (i >= n) return;
+__global__ void __launch_bounds__(32) dc_zhat_kernel(DcArgs P) {
+  const int n = P.n, i = blockIdx.x;
   const int t = dc_node_of(n, P.level, i), lo = dc_bound(n, P.level, t), K = P.node[t].x, k = i - lo;
   if (k >= K) return;
   const WarpLane L;
@@ -487,9 +542,8 @@ __global__ void __launch_bounds__(128) dc_zhat_kernel(DcArgs P) {
 
 // U row (lo + j): unit vector of root j over the node's kept columns, in the
 // grouped order; a deflated column's vector is copied to its place in Qout.
-__global__ void __launch_bounds__(128) dc_vectors_kernel(DcArgs P) {
-  const int n = P.n, i = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (i >= n) return;
+__global__ void __launch_bounds__(32) dc_vectors_kernel(DcArgs P) {
+  const int n = P.n, i = blockIdx.x, lane = threadIdx.x;
   const int l = P.level, t = dc_node_of(n, l, i), lo = dc_bound(n, l, t), hi = dc_bound(n, l, t + 1);
   const int K = P.node[t].x, j = i - lo;
   if (j >= K) {
@@ -502,7 +556,7 @@ __global__ void __launch_bounds__(128) dc_vectors_kernel(DcArgs P) {
   double* u = P.U + (long)i * n;
   double s = 0.0;
   for (int k = lane; k < K; k += 32) {
-    const double x = P.zhat[lo + k] / ((P.kd[lo + k] - db) - eta);
+    const double x = P.zhat[lo + k] * dc_rcp((P.kd[lo + k] - db) - eta);
     u[P.kpos[lo + k]] = x;
     s = fma(x, x, s);
   }
@@ -564,29 +618,111 @@ __global__ void __launch_bounds__(256) dc_gemm_kernel(DcArgs P) {
     }
 }
 
+// A group of BK consecutive reflectors, applied from the highest row down, takes
+// q to q + sum_t s_t v_t with s = W x, x_u = v_u . q and W lower triangular:
+// s_t = -beta_t (x_t + sum_{u < t} s_u v_u . v_t).  wy[group]: the ten entries of
+// W, row by row (one warp per group).
+constexpr int BK = 4, WY = 10;
+__device__ __forceinline__ int dc_group_row(int n, int g, int t) { return n - 3 - g * BK - t; }
+__global__ void __launch_bounds__(32) dc_wy_kernel(int n, const double* __restrict__ Vh, const double* __restrict__ beta,
+                                                   double* __restrict__ wy) {
+  const int g = blockIdx.x, lane = threadIdx.x;
+  double m[BK][BK] = {}, b[BK], w[BK][BK] = {};
+#pragma unroll
+  for (int t = 0; t < BK; ++t) {
+    const int jt = dc_group_row(n, g, t);
+    b[t] = jt < 0 ? 0.0 : beta[jt];
+#pragma unroll
+    for (int s = 0; s < t; ++s) {
+      const int js = dc_group_row(n, g, s);
+      double x = 0.0;
+      if (jt >= 0)
+        for (int k = js + 1 + lane; k < n; k += 32) x = fma(Vh[(long)js * n + k], Vh[(long)jt * n + k], x);
+      m[s][t] = warp_sum(x);
+    }
+  }
+#pragma unroll
+  for (int t = 0; t < BK; ++t) {
+    w[t][t] = -b[t];
+#pragma unroll
+    for (int u = 0; u < t; ++u) {
+      double x = 0.0;
+#pragma unroll
+      for (int s = u; s < t; ++s) x = fma(w[s][u], m[s][t], x);
+      w[t][u] = -b[t] * x;
+    }
+  }
+  if (lane == 0) {
+    int o = 0;
+#pragma unroll
+    for (int t = 0; t < BK; ++t)
+#pragma unroll
+      for (int u = 0; u <= t; ++u) wy[(long)g * WY + o++] = w[t][u];
+  }
+}
+
 // V[:, c] = H_0 H_1 ... H_{n-3} Q[:, c]: a warp per column, the column in shared
 // memory (each lane owns the rows equal to it modulo 32), no block barrier.
-__global__ void __launch_bounds__(256) dc_back_kernel(int n, const double* __restrict__ Vh, const double* __restrict__ beta,
-                                                      const double* __restrict__ Q, const double* __restrict__ lam,
-                                                      double* __restrict__ V, double* A, int* status) {
+// BK reflectors at a time: independent chains.
+__global__ void __launch_bounds__(256) dc_back_kernel(int n, const double* __restrict__ Vh, const double* __restrict__ wy,
+                                                      const double* __restrict__ Q,
+                                                      const double* __restrict__ lam, double* __restrict__ V, double* A,
+                                                      int* status) {
   extern __shared__ double sq[];
   const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5, c = blockIdx.x * wpb + (threadIdx.x >> 5);
   if (c >= n) return;
   double* q = sq + (long)(threadIdx.x >> 5) * n;
+  const WarpLane L;
   for (int k = lane; k < n; k += 32) q[k] = Q[(long)c * n + k];
-  for (int j = n - 3; j >= 0; --j) {
-    const double bj = beta[j];
-    if (bj == 0.0) continue;
-    const double* v = Vh + (long)j * n;
-    double s = 0.0;
-    const int kbeg = (j + 1) & ~31;
+  for (int g = 0; g * BK < n - 2; ++g) {
+    int j[BK];
+    double x[BK] = {0.0, 0.0, 0.0, 0.0}, w[WY];
+    const double* v[BK];
+#pragma unroll
+    for (int t = 0; t < BK; ++t) {
+      const int jt = dc_group_row(n, g, t);
+      j[t] = jt < 0 ? n : jt;                // beyond the last reflector: no rows
+      v[t] = Vh + (long)(jt < 0 ? 0 : jt) * n;
+    }
+#pragma unroll
+    for (int u = 0; u < WY; ++u) w[u] = wy[(long)g * WY + u];
+    const int top = dc_group_row(n, g, 0), low = top - BK + 1 < 0 ? 0 : top - BK + 1;
+    int k = ((low + 1) & ~31) + lane;
+    // rows up to the highest reflector's first one: masked
+    if (k <= top) {
+#pragma unroll
+      for (int t = 0; t < BK; ++t)
+        if (k < n && k > j[t]) x[t] = v[t][k] * q[k];
+      k += 32;
+      if (k <= top) {
+#pragma unroll
+        for (int t = 0; t < BK; ++t)
+          if (k < n && k > j[t]) x[t] = fma(v[t][k], q[k], x[t]);
+        k += 32;
+      }
+    }
 #pragma unroll 4
-    for (int k = kbeg + lane; k < n; k += 32)
-      if (k > j) s = fma(v[k], q[k], s);
-    s = -bj * warp_sum(s);
+    for (int kk = k; kk < n; kk += 32) {
+      const double y = q[kk];
+#pragma unroll
+      for (int t = 0; t < BK; ++t)
+        x[t] = fma(v[t][kk], y, x[t]);
+    }
+    L.sum4(x[0], x[1], x[2], x[3]);
+    const double s[BK] = {w[0] * x[0], fma(w[1], x[0], w[2] * x[1]), fma(w[3], x[0], w[4] * x[1]) + w[5] * x[2],
+                          fma(w[6], x[0], w[7] * x[1]) + fma(w[8], x[2], w[9] * x[3])};
+    for (int kk = ((low + 1) & ~31) + lane; kk < k && kk < n; kk += 32) {
+      double y = q[kk];
+#pragma unroll
+      for (int t = 0; t < BK; ++t)
+        if (kk > j[t]) y = fma(s[t], v[t][kk], y);
+      q[kk] = y;
+    }
 #pragma unroll 4
-    for (int k = kbeg + lane; k < n; k += 32)
-      if (k > j) q[k] = fma(s, v[k], q[k]);
+    for (int kk = k; kk < n; kk += 32) {
+      const double y0 = fma(s[1], v[1][kk], fma(s[0], v[0][kk], q[kk]));  // (a missing reflector's s is 0)
+      q[kk] = y0 + fma(s[3], v[3][kk], s[2] * v[2][kk]);
+    }
   }
   for (int k = lane; k < n; k += 32) V[(long)k * n + c] = q[k];
   if (lane == 0) {
@@ -643,6 +779,7 @@ int eig_dc(int n, double* A, double* V, double* work, unsigned* bar, int* status
   D.dcol = D.kpos + n;
   D.base = D.dcol + n;
   D.colpos = D.base + n;
+  double* wy = take(3);  // WY per group of BK reflectors
   D.anorm = red;
   D.U = U;
   int dev = 0, sms = 0;
@@ -669,21 +806,21 @@ int eig_dc(int n, double* A, double* V, double* work, unsigned* bar, int* status
   D.Qout = Q0;
   dc_leaf_kernel<<<1 << D.levels, 32, 0, st>>>(D);
   DSRG_LAUNCH_CHECK();
-  DSRG_CUDA(cudaFuncSetAttribute(dc_deflate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 29 * EIG_DC_MAX_N));
+  DSRG_CUDA(cudaFuncSetAttribute(dc_deflate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 30 * EIG_DC_MAX_N));
   for (int l = D.levels - 1; l >= 0; --l) {
     std::swap(Q0, Q1);
     D.level = l;
     D.Qin = Q1;
     D.Qout = Q0;
     const int nodes = 1 << l, mmax = ceil_div(n, nodes) + 1, hmax = ceil_div(mmax, 2) + 1;
-    dc_deflate_kernel<<<nodes, 256, 29 * (size_t)mmax, st>>>(D);
+    dc_deflate_kernel<<<nodes, 256, 30 * (size_t)mmax, st>>>(D);
     DSRG_LAUNCH_CHECK();
-    const int rb = ceil_div(n, 128), cb = ceil_div(n, 4);
-    dc_secular_kernel<<<rb + cb, 128, 0, st>>>(D, rb);
+    const int rb = ceil_div(n, 32);
+    dc_secular_kernel<<<rb + n, 32, 0, st>>>(D, rb);
     DSRG_LAUNCH_CHECK();
-    dc_zhat_kernel<<<cb, 128, 0, st>>>(D);
+    dc_zhat_kernel<<<n, 32, 0, st>>>(D);
     DSRG_LAUNCH_CHECK();
-    dc_vectors_kernel<<<cb, 128, 0, st>>>(D);
+    dc_vectors_kernel<<<n, 32, 0, st>>>(D);
     DSRG_LAUNCH_CHECK();
     if (mmax <= 512) dc_gemm_kernel<16><<<dim3(ceil_div(hmax, 16), ceil_div(mmax, 16), 2 * nodes), 256, 0, st>>>(D);
     else dc_gemm_kernel<32><<<dim3(ceil_div(hmax, 32), ceil_div(mmax, 32), 2 * nodes), 256, 0, st>>>(D);
@@ -693,8 +830,9 @@ int eig_dc(int n, double* A, double* V, double* work, unsigned* bar, int* status
   const int wfit = (int)(TRI_SMEM / (sizeof(double) * (size_t)n));
   const int wpb = std::max(1, std::min(std::min(8, wfit), ceil_div(n, sms)));
   DSRG_CUDA(cudaFuncSetAttribute(dc_back_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TRI_SMEM));
-  dc_back_kernel<<<ceil_div(n, wpb), 32 * wpb, sizeof(double) * (size_t)n * wpb, st>>>(n, A, T.beta, Q0, D.lam, V, A,
-                                                                                      status_dev);
+  dc_wy_kernel<<<ceil_div(n - 2, BK), 32, 0, st>>>(n, A, T.beta, wy);
+  DSRG_LAUNCH_CHECK();
+  dc_back_kernel<<<ceil_div(n, wpb), 32 * wpb, sizeof(double) * (size_t)n * wpb, st>>>(n, A, wy, Q0, D.lam, V, A, status_dev);
   DSRG_LAUNCH_CHECK();
   return DSRG_FNO_OK;
 }

@@ -70,12 +70,12 @@ int syrk_dressed_f64(int nv, int nr, const double* sig, const double* sig_sign, 
 
 // Symmetric-eigen helpers (eig.cu)
 constexpr int EIG_MAX_BLOCKS = 1024;  // grid bound of the eigensolver (reduction scratch)
-constexpr int EIG_DC_VECTORS = 22;    // vectors of n doubles that the divide-and-conquer solver keeps
+constexpr int EIG_DC_VECTORS = 26;    // vectors of n doubles that the divide-and-conquer solver keeps
 constexpr size_t eig_work_doubles(int n) {
   return 3 * (size_t)n * n + 2 * EIG_MAX_BLOCKS + 16 + EIG_DC_VECTORS * (size_t)n + 16;
 }
 // Householder reduction and divide and conquer (eig_dc.cu), EIG_DC_MIN_N <= n <= EIG_DC_MAX_N
-constexpr int EIG_DC_MIN_N = 33, EIG_DC_MAX_N = 7800;
+constexpr int EIG_DC_MIN_N = 33, EIG_DC_MAX_N = 7700;
 int eig_dc(int n, double* A, double* V, double* work, unsigned* bar, int* status_dev, long long spin_limit, bool shared,
            cudaStream_t st);
 int eig_set_barrier_limit(long long spins);

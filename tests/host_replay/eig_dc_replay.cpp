@@ -84,8 +84,10 @@ extern "C" void eig_dc_replay(int n, const double* d0, const double* e, double* 
         ty[r] = c < mid ? 1 : 3;
         sz[r] = (c < mid ? Q[c * ld + mid - 1] : (ec < 0 ? -1 : 1) * Q[c * ld + mid]) * sqrt(0.5);
       }
+      vector<unsigned char> fl(m);
+      for (int r = 0; r < m; ++r) fl[r] = dc_flag(r, sd.data(), sz.data(), rho, tol);
       int nr = 0;
-      const int K = dc_deflate(m, ord.data(), sd.data(), sz.data(), ty.data(), rho, tol, kcol.data(), kd.data(), kz.data(),
+      const int K = dc_deflate(m, ord.data(), sd.data(), sz.data(), fl.data(), ty.data(), rho, tol, kcol.data(), kd.data(), kz.data(),
                                kty.data(), dcol.data(), dval.data(), rot.data(), &nr);
       counts[0] += m - K;
       counts[1] += nr;
