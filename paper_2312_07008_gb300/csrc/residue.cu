@@ -631,38 +631,40 @@ __global__ void __launch_bounds__(256) plain_residue_kernel(ResGemm P, PlainOut 
 
 // Rank-K update of D_vv, sums over all rows of all dressed matrices: bound by the
 // tensor cores.  opdm pass of nvir 1200 (10 active, K = 6.8e6): the products take
-// 65 ms (1.62 PFLOP/s) instead of the digit planes' 120; the staging 40 ms instead
-// of 28, for nine planes instead of five.  Row by row of D: sums over the
-// segments, in their order, of sign A_s[e] . A_s[f] (upper tiles, mirrored).
-__global__ void __launch_bounds__(256) syrk_residue_kernel(ResGemm P, const int* __restrict__ exps, int nv, double* D) {
+// 69 ms (1.52 PFLOP/s) instead of the digit planes' 120; the staging 40 ms instead
+// of 28, for nine planes instead of five.  D[e][f] += the sum over the segments,
+// in a fixed order, of sign A_s[e] . A_s[f] (upper tiles, mirrored).
+__global__ void __launch_bounds__(256) syrk_residue_kernel(const __grid_constant__ ResGemm P, const int* __restrict__ exps,
+                                                           int nv, double* D) {
   constexpr int NM = RES_MOD_S;
+  __shared__ double part[8][32][9];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int mt, nt;
   rg_tile(P, blockIdx.y, &mt, &nt);
-  const int e = mt * GT_M + threadIdx.x;
-  if (e >= nv) return;
-  const int g = blockIdx.x, f0 = nt * GT_M + g * 8;
-  if (f0 >= nv || f0 + 7 < e) return;
+  const int g = blockIdx.x, e0 = mt * GT_M + blockIdx.z * 32, f0 = nt * GT_M + g * 8, e = e0 + lane;
+  if (e0 >= nv || f0 >= nv || f0 + 7 < e0) return;
   double acc[8] = {};
-  for (int s = 0; s < P.nseg; ++s) {
+  for (int s = warp; s < P.nseg; s += 8) {  // a warp per segment, eight columns of 32 rows
     const int* ex = exps + (long)P.seg[s].scale * nv;
     uint32_t w[NM][4];
-    load_residues<NM>(P.res + (((long)s * P.ntiles + blockIdx.y) * NM) * GT_M * GT_M + threadIdx.x * 8, g, w);
-    const int ee = ex[e];
+    load_residues<NM>(P.res + (((long)s * P.ntiles + blockIdx.y) * NM) * GT_M * GT_M + (blockIdx.z * 32 + lane) * 8, g, w);
+    const int ee = ex[min(e, nv - 1)];
 #pragma unroll
-    for (int c = 0; c < 8; ++c)
-      if (f0 + c < nv) {
-        const double v = fraction_f64<NM>(recombine<NM>(w, c), ee + ex[f0 + c]);
-        acc[c] += P.seg[s].sign < 0 ? -v : v;
-      }
+    for (int c = 0; c < 8; ++c) {
+      const double v = fraction_f64<NM>(recombine<NM>(w, c), ee + ex[min(f0 + c, nv - 1)]);
+      acc[c] += P.seg[s].sign < 0 ? -v : v;
+    }
   }
 #pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const int f = f0 + c;
-    if (f >= nv || f < e) continue;
-    const double v = D[(long)e * nv + f] + acc[c];
-    D[(long)e * nv + f] = v;
-    if (f != e) D[(long)f * nv + e] += acc[c];
-  }
+  for (int c = 0; c < 8; ++c) part[warp][lane][c] = acc[c];
+  __syncthreads();
+  const int r = threadIdx.x >> 3, c = threadIdx.x & 7, er = e0 + r, f = f0 + c;
+  if (er >= nv || f >= nv || f < er) return;
+  double v = part[0][r][c];
+#pragma unroll
+  for (int q = 1; q < 8; ++q) v += part[q][r][c];
+  D[(long)er * nv + f] += v;
+  if (f != er) D[(long)f * nv + er] += v;
 }
 
 // -f of row e of scale group s, from its norm over the group's matrices: the
@@ -902,14 +904,22 @@ int residue_plain(int nm, int M, int N, const __nv_bfloat16* pa, const int* ea, 
 
 // Segments of the rank-K update over nr matrices of which those from n_signed
 // on may carry a minus sign: every range of scales is one segment, or two (one
-// per sign).  Eight to 16 ranges bound the error (a range's rows share one
-// scale) and fill the pairs of SMs: their count is the one whose units leave
-// the least of the last round idle.
+// per sign).  A range's rows share one scale, whose roundings average out over
+// the ranges: with 32 or more the errors of D_vv stay below those of five digit
+// planes at every size tried (nvir 20 to 420; with 8 to 16 up to 1.3 times them
+// at the smallest).  Their residues are written and read once (nvir 1200: 0.57 GB
+// for 32 ranges; where 64 would take more than 4 GB, fewer).  Of the counts
+// allowed the one whose units leave the least of the last round of SM pairs idle.
+static int residue_max_segments(int nv) {
+  const int nt = ceil_div(nv, GT_M);
+  const size_t per = (size_t)(nt * (nt + 1) / 2) * residue_tile_bytes(RES_MOD_S);
+  return (int)std::max<size_t>(16, std::min<size_t>(RES_MAX_SEGMENTS, ((size_t)4 << 30) / per));
+}
 int residue_segments(int nv, int nr, int n_signed, ResSegment* seg) {
-  const int nt = ceil_div(nv, GT_M), units = nt * (nt + 1) / 2 * RES_MOD_S, pairs = 76;
-  int best = 8;
+  const int nt = ceil_div(nv, GT_M), units = nt * (nt + 1) / 2 * RES_MOD_S, pairs = 76, most = residue_max_segments(nv);
+  int best = most / 2;
   double best_eff = 0.0;
-  for (int k = 8; k <= 16; ++k) {
+  for (int k = most / 2; k <= most; ++k) {
     const long u = (long)units * k;
     const double eff = (double)u / ((double)ceil_div(u, pairs) * pairs);
     if (eff > best_eff + 0.005) {
@@ -927,16 +937,17 @@ int residue_segments(int nv, int nr, int n_signed, ResSegment* seg) {
       ++scale;
     }
   };
-  // shares of the ranges in proportion to the matrices, at least one each
+  // shares of the segments in proportion to the matrices, at least one range each
   const int plain = std::min(n_signed, nr), sg = nr - plain;
-  if (plain > 0) add(0, plain, std::max(1, (int)((long)best * plain / nr)), false);
-  if (sg > 0) add(plain, nr, std::max(1, best - (plain > 0 ? std::max(1, (int)((long)best * plain / nr)) : 0)), true);
+  const int np = plain > 0 ? std::max(1, (int)((long)best * plain / nr)) : 0;
+  if (plain > 0) add(0, plain, sg > 0 ? std::min(np, best - 2) : np, false);
+  if (sg > 0) add(plain, nr, std::max(1, (best - np) / 2), true);
   return n;
 }
 
 size_t residue_syrk_res_bytes(int nv) {
   const int nt = ceil_div(nv, GT_M);
-  return (size_t)RES_MAX_SEGMENTS / 2 * (nt * (nt + 1) / 2) * residue_tile_bytes(RES_MOD_S);
+  return (size_t)residue_max_segments(nv) * (nt * (nt + 1) / 2) * residue_tile_bytes(RES_MOD_S);
 }
 
 // D += sum_r sign_r Sig_r Sig_r^T.  rowpart: as dress_dd writes it; exps: RES_MAX_SEGMENTS nv ints; scale_of: nr ints (host list, copied).
@@ -968,7 +979,7 @@ int residue_syrk(int nv, int nr, int n_signed, const float2* sig, const float* r
     DSRG_LAUNCH_CHECK();
   }
   DSRG_TRY(launch_gemm(planes, nv, planes, nv, Kpad, P, st));
-  syrk_residue_kernel<<<dim3(32, P.ntiles), 256, 0, st>>>(P, exps, nv, D);
+  syrk_residue_kernel<<<dim3(GT_M / 8, P.ntiles, GT_M / 32), 256, 0, st>>>(P, exps, nv, D);
   DSRG_LAUNCH_CHECK();
   return DSRG_FNO_OK;
 }
