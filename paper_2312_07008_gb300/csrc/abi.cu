@@ -100,14 +100,15 @@ static void build_plan(int nc, int na, long cap_pairs, Plan& P) {
       P.batches.push_back(cur);
       cur = Batch{(int)P.pairs.size(), 0, (int)P.desc.size(), 0, 0, 0, 0};
     }
-    for (int o0 = 0; o0 < G.nout; o0 += DRESS_OC) {
+    const int o_step = ceil_div(G.nout, ceil_div(G.nout, DRESS_OC));
+    for (int o0 = 0; o0 < G.nout; o0 += o_step) {
       DressDesc d{};
       d.kind = G.kind;
       d.slot = cur.npairs;
       d.nslots = (int)G.pairs.size();
       d.out = cur.nout;
       d.o_begin = o0;
-      d.o_count = std::min(DRESS_OC, G.nout - o0);
+      d.o_count = std::min(o_step, G.nout - o0);
       d.m = G.pairs[0].x;
       P.desc.push_back(d);
       ++cur.ndesc;

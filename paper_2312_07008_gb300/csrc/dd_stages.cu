@@ -24,9 +24,6 @@ __global__ void reg_tables_fill_kernel() {
     g_reg.C[j] = dd_from_double(-expm1(-j * 0.69314718055994530942 / 64.0));
   }
   if (threadIdx.x == 0) {
-    g_reg.log2e = dd_from_double(1.44269504088896340736);
-    g_reg.ln2 = dd_from_double(0.69314718055994530942);
-    g_reg.sixth = dd_from_double(1.0 / 6.0);
   }
 }
 
@@ -103,14 +100,19 @@ __device__ __forceinline__ dd ld(const float2* p, long i) {
   return {v.x, v.y};
 }
 
-// acc + c s: the product's high part is added error-free (TwoSum), its low
-// parts and the accumulator's low word in float32; one renormalisation.
+// acc + c s without renormalisation: the product's high part is added error-free
+// (TwoSum), its low parts and both errors to the low word in float32.  nh = -s.hi.
+template <class T>
+__device__ __forceinline__ void dd_fma_into(ddt<T>& acc, ddt<T> c, ddt<T> s, T nh) {
+  const T p = fl_mul(c.hi, s.hi);
+  const T ne = fl_fma(c.hi, nh, p);  // minus the product's error
+  const ddt<T> t = two_sum(acc.hi, p);
+  acc.lo = fl_sub(fl_add(fl_fma(c.lo, s.hi, fl_fma(c.hi, s.lo, acc.lo)), t.lo), ne);
+  acc.hi = t.hi;
+}
 __device__ __forceinline__ dd dd_fma_acc(dd acc, dd c, dd s) {
-  const dd p = two_prod(c.hi, s.hi);
-  const float e = __fmaf_rn(c.hi, s.lo, __fmaf_rn(c.lo, s.hi, p.lo));
-  dd t = two_sum(acc.hi, p.hi);
-  t.lo = __fadd_rn(t.lo, __fadd_rn(acc.lo, e));
-  return quick_two_sum(t.hi, t.lo);
+  dd_fma_into(acc, c, s, -s.hi);
+  return quick_two_sum(acc.hi, acc.lo);
 }
 
 // What the staging of the dressed matrices needs of a row: the largest |hi| of
@@ -276,20 +278,21 @@ __global__ void __launch_bounds__(256, 4) dress_core_dd_kernel(int nv, const Dre
   if (want_sig && blockIdx.x == 0 && threadIdx.x < (diag ? 1 : 2)) sig_sign[D.out + threadIdx.x] = 1.0;
 }
 
-// Double-float form of the group dressing (same structure as dress.cu).
+// Double-float form of the group dressing (same structure as dress.cu).  Bound
+// by the float32 pipe and the latency of its chains: 12 operations per slot and
+// output for each of tau and kappa, which share the coefficient and go through
+// packed pairs.  nvir 600, 40 core and 10 active orbitals, with the core pairs'
+// kernel: 7.48 -> 6.98 ms (a third block per SM: 7.24 with two, 7.73 with four).
 template <int OCT>
 __global__ void __launch_bounds__(GNT, 3)
     dress_dd_kernel(int nv, int na, const DressDesc* __restrict__ desc, DressAux aux,
                     const float2* __restrict__ tau, const float2* __restrict__ kap, float2* __restrict__ sig,
                     double* __restrict__ sig_sign, double* __restrict__ e_part, int want_sig,
                     unsigned* __restrict__ rowmax, float* __restrict__ rowpart) {
-  static_assert(OCT % 2 == 0, "coefficients are read two outputs at a time");
   constexpr int NS = MAXSLOT;
-  // float64 coefficients, converted in place to double-float (same size)
-  __shared__ __align__(16) union {
-    double d[NS][OCT];
-    dd f[NS][OCT];
-  } cf;
+  // double-float coefficients, every word twice: {hi, hi, lo, lo} multiplies a
+  // (tau, kappa) pair
+  __shared__ float4 cf2[NS * OCT];
   __shared__ double lam[OCT], sgn[OCT], dg[NS];
   __shared__ dd lamw[OCT], sqd[OCT];
   __shared__ float sgnf[OCT], dgf[NS];  // float copies: no float64 op in the loops
@@ -297,12 +300,17 @@ __global__ void __launch_bounds__(GNT, 3)
   __shared__ float2 tT[2][GT][GT + 1], tK[2][GT][GT + 1], sA[GT][GT + 1];
   __shared__ double red[GNT / 32];
   const DressDesc D = desc[blockIdx.y];
-  group_coefficients<OCT>(D, aux, na, cf.d, lam, sgn, dg);
+  // the float64 coefficients fill the lower half; each thread's, from the back
+  double(*cd)[OCT] = reinterpret_cast<double(*)[OCT]>(cf2);
+  group_coefficients<OCT>(D, aux, na, cd, lam, sgn, dg);
   const int oc = D.o_count;
-  for (int idx = threadIdx.x; idx < D.nslots * OCT; idx += blockDim.x) {
-    const int u = idx / OCT, o = idx % OCT;
-    const double v = cf.d[u][o];
-    cf.f[u][o] = dd_from_double(v);
+  for (int base = (D.nslots * OCT - 1) / GNT * GNT; base >= 0; base -= GNT) {
+    const int idx = base + threadIdx.x;
+    const bool in = idx < D.nslots * OCT;
+    const dd v = in ? dd_from_double(cd[idx / OCT][idx % OCT]) : dd_make(0.0f);
+    __syncthreads();  // read before the places of this pass, which start at 2 base, are written
+    if (in) cf2[idx] = make_float4(v.hi, v.hi, v.lo, v.lo);
+    __syncthreads();
   }
   for (int o = threadIdx.x; o < oc; o += blockDim.x) {
     lamw[o] = dd_from_double(0.5 * lam[o]);
@@ -380,16 +388,13 @@ __global__ void __launch_bounds__(GNT, 3)
     const int e = E0 + ty, f = F0 + tx;
     const bool inside = e < nv && f < nv;
     const float w = (te == tf) ? 1.0f : 2.0f;
-    dd at[OCT], ak[OCT];
+    dd2 acc[OCT];  // outputs of tau and of kappa, packed: half the instructions
 #pragma unroll
-    for (int o = 0; o < OCT; ++o) {
-      at[o] = dd_make(0.0f);
-      ak[o] = dd_make(0.0f);
-    }
+    for (int o = 0; o < OCT; ++o) acc[o] = {f2_set(0.f, 0.f), f2_set(0.f, 0.f)};
     for (int u = 0; u < ns; ++u) {
       tT[buf][ty][tx] = nt_;
       tK[buf][ty][tx] = nk_;
-      const dd a = {na_.x, na_.y}, b = {nb_.x, nb_.y};
+      const dd2 a = {f2_set(na_.x, nb_.x), f2_set(na_.y, nb_.y)};
       // the next slot's (or the next tile's first slot's) loads fly during
       // this slot's arithmetic
       if (u + 1 < ns) fetch(te, tf, u + 1);
@@ -399,25 +404,17 @@ __global__ void __launch_bounds__(GNT, 3)
       // the two signed combinations are formed once per slot
       const float du = dgf[u];
       const float2 xt = tT[buf][tx][ty], xk = tK[buf][tx][ty];
-      const dd att = {du * xt.x, du * xt.y}, btt = {du * xk.x, du * xk.y};
-      const dd tp = dd_add_fast(a, att), tm = dd_sub_fast(a, att);
-      const dd kp = dd_add_fast(b, btt), km = dd_sub_fast(b, btt);
-      // the slot's coefficients, two outputs per 16-byte shared load
-      const float4* cu = reinterpret_cast<const float4*>(&cf.f[u][0]);
+      const f32x2 du2 = f2_set(du, du);
+      const dd2 at = {f2_mul(du2, f2_set(xt.x, xk.x)), f2_mul(du2, f2_set(xt.y, xk.y))};
+      const dd2 sp = dd_add_fast(a, at), sm = dd_sub_fast(a, at);
+      const f32x2 np = fl_neg(sp.hi), nm = fl_neg(sm.hi);
+      const float4* cu = cf2 + u * OCT;
 #pragma unroll
-      for (int o2 = 0; o2 < OCT; o2 += 2) {
-        if (o2 < oc) {
-          const float4 c2 = cu[o2 >> 1];
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int o = o2 + h;
-            if (o < oc) {
-              const dd c = h ? dd{c2.z, c2.w} : dd{c2.x, c2.y};
-              const bool pos = (posmask >> o) & 1u;
-              at[o] = dd_fma_acc(at[o], c, pos ? tp : tm);
-              ak[o] = dd_fma_acc(ak[o], c, pos ? kp : km);
-            }
-          }
+      for (int o = 0; o < OCT; ++o) {
+        if (o < oc) {
+          const float4 c = cu[o];
+          const bool pos = (posmask >> o) & 1u;
+          dd_fma_into(acc[o], dd2{f2_set(c.x, c.y), f2_set(c.z, c.w)}, pos ? sp : sm, pos ? np : nm);
         }
       }
       buf ^= 1;
@@ -425,9 +422,13 @@ __global__ void __launch_bounds__(GNT, 3)
 #pragma unroll
     for (int o = 0; o < OCT; ++o) {
       if (o < oc) {
-        if (inside) part = dd_add(part, dd_mul_f(dd_mul(lamw[o], dd_mul(at[o], ak[o])), w));
+        dd at, ak;
+        acc[o] = quick_two_sum(acc[o].hi, acc[o].lo);
+        f2_get(acc[o].hi, &at.hi, &ak.hi);
+        f2_get(acc[o].lo, &at.lo, &ak.lo);
+        if (inside) part = dd_add(part, dd_mul_f(dd_mul(lamw[o], dd_mul(at, ak)), w));
         if (want_sig) {
-          const dd v = dd_mul(sqd[o], at[o]);
+          const dd v = dd_mul(sqd[o], at);
           const long mat = D.out + D.o_begin + o;
           float2* S = sig + mat * nv2;
           if (inside) S[(long)e * nv + f] = make_float2(v.hi, v.lo);
@@ -468,8 +469,16 @@ __global__ void regularize_test_kernel(int n, const double* delta, double s, dou
   reg_tables_load(R);
   __syncthreads();
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+    // this value beside another one of the list, as the pairs of the epilogue
+    const dd p = dd_from_double(delta[k]), q = dd_from_double(delta[n - 1 - k]);
+    dd2 r, z;
+    regularize(dd2{f2_set(p.hi, q.hi), f2_set(p.lo, q.lo)}, dd_from_double(s), R, &r, &z);
     dd a, b;
-    regularize(dd_from_double(delta[k]), dd_from_double(s), R, &a, &b);
+    float other;
+    f2_get(r.hi, &a.hi, &other);
+    f2_get(r.lo, &a.lo, &other);
+    f2_get(z.hi, &b.hi, &other);
+    f2_get(z.lo, &b.lo, &other);
     r1[k] = dd_to_double(a);
     y[k] = dd_to_double(b);
   }

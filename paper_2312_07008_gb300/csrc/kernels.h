@@ -39,9 +39,11 @@ enum DressKind {
   GROUP_AA = 3        // all active pairs: eigenvectors of the two swap blocks of the aa hole 2-RDM
 };
 
-// outputs per work item; blocks per work item (they stride over upper tiles)
+// outputs per work item at most (a group's are split evenly: its slots are read
+// and combined with their transposes once per item; with 8, 12 and 16 slower by 4,
+// 1 and 14 %); blocks per work item (they stride over upper tiles)
 #ifndef DRESS_OUTPUTS
-#define DRESS_OUTPUTS 8
+#define DRESS_OUTPUTS 10
 #endif
 #ifndef DRESS_BLOCKS
 #define DRESS_BLOCKS 48

@@ -20,28 +20,9 @@ using namespace res;
 
 // ---------------------------------------------------------------- staging
 __device__ __forceinline__ double square_of(double v) { return v * v; }
-__device__ __forceinline__ double square_of(float2 v) {
-  const double x = (double)v.x + (double)v.y;
-  return x * x;
-}
 __device__ __forceinline__ double zero_like(double) { return 0.0; }
-__device__ __forceinline__ float2 zero_like(float2) { return make_float2(0.f, 0.f); }
 
 __device__ __forceinline__ long long integer_of(double v, int f) { return scaled_integer(v, f); }
-
-// hi + lo with the same rule, exactly in 64-bit fixed point with 16 guard bits
-__device__ __forceinline__ long long fixed_of(float v, int f) {
-  const int b = __float_as_int(v), E = (b >> 23) & 0xFF;
-  if (E == 0) return 0;
-  const long long m = (long long)((b & 0x7FFFFF) | 0x800000);
-  const int sh = E - 150 + f + 16;
-  const long long x = sh >= 0 ? (sh < 39 ? m << sh : 0) : (-sh < 63 ? m >> -sh : 0);
-  return b < 0 ? -x : x;
-}
-__device__ __forceinline__ long long integer_of(float2 v, int f) {
-  const long long x = fixed_of(v.x, f) + fixed_of(v.y, f);
-  return x >= 0 ? (x + 0x8000) >> 16 : -((-x + 0x8000) >> 16);
-}
 
 // Squared norms of the rows: part[split][row] over the split's share of k.
 // Source element (row, k) at src[row rs + k ks]; one of rs, ks is 1.
@@ -446,8 +427,10 @@ __device__ __forceinline__ dd fraction_dd(uint64_t u) {
 // the regulariser's code is there once.  (Written from the 8-element threads, 8
 // bytes to 32 rows at once, an opdm pass of nvir 1200 spent 96 ms here; with the
 // regulariser unrolled for 8 elements 57 ms, waiting for instructions.)
-// Delta = hp[row] + hp[column].  Bound by instruction issue: about 100 for the
-// residues of an element beside some 250 for its regulariser.
+// Delta = hp[row] + hp[column].  Bound by the float32 pipe (72 %) and instruction
+// issue (68 %): about 100 instructions for the residues of an element beside some
+// 100 for its regulariser, two rows packed (250 one by one; nvir 443 with 5 active
+// orbitals 2.13 -> 1.74 ms).
 struct PairResidues {
   const int2* tiles;
   const uint16_t* res;
@@ -520,30 +503,45 @@ __global__ void __launch_bounds__(256, 4) pair_epilogue_residue_kernel(PairResid
       const float2 hc = P.hp[C];
       const float fc = pow2_float(P.exps[C] + EX - EX / 2);
 #pragma unroll 1
-      for (int u = 0; u < 4; ++u) {
-        const int rr = warp * 4 + u, a = s_a[rr], i = s_i[rr];
-        if (a < 0) break;
-        const bool av = a >= na;
-        // vv -> tau, kappa; va -> ts[i][j]; av -> ts[j][i], written by the va element of (i, i) itself
-        if (!((av && bv) || (P.ts != nullptr && (av || (bv && i != j))))) continue;
-        const int slot = P.slot_of[(long)i * P.nh + j];
-        if (slot < 0) continue;
-        const float2 f = sN[rr][q * 32 + lane], hr = s_hp[rr];
-        const float fr = s_fr[rr];
-        dd n = dd_mul(dd{f.x, f.y}, mu);
-        n = {n.hi * fr * fc, n.lo * fr * fc};
-        dd r1, y;
-        regularize(dd_add(dd{hr.x, hr.y}, dd{hc.x, hc.y}), s, R, &r1, &y);
-        const dd x = dd_mul(n, r1);
-        if (av && bv) {
-          const dd k = dd_mul(n, dd_add_f(y, 1.0f));
-          const long o = ((long)slot * nv + (a - na)) * nv + (b - na);
-          P.tau[o] = make_float2(x.hi, x.lo);
-          P.kap[o] = make_float2(k.hi, k.lo);
-        } else if (av) {
-          P.ts[(((long)i * P.nh + j) * nv + (a - na)) * na + b] = dd_to_double(x);
-        } else {
-          P.ts[(((long)j * P.nh + i) * nv + (b - na)) * na + a] = dd_to_double(x);
+      for (int u = 0; u < 4; u += 2) {  // two rows at a time, packed
+        const int rr = warp * 4 + u;
+        int slot[2], a[2], i[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          a[k] = s_a[rr + k];
+          i[k] = s_i[rr + k];
+          const bool av = a[k] >= na;
+          // vv -> tau, kappa; va -> ts[i][j]; av -> ts[j][i], written by the va element of (i, i) itself
+          const bool use = a[k] >= 0 && ((av && bv) || (P.ts != nullptr && (av || (bv && i[k] != j))));
+          slot[k] = use ? P.slot_of[(long)i[k] * P.nh + j] : -1;
+        }
+        if (slot[0] < 0 && slot[1] < 0) continue;
+        const float2 f0 = sN[rr][q * 32 + lane], f1 = sN[rr + 1][q * 32 + lane], h0 = s_hp[rr], h1 = s_hp[rr + 1];
+        const f32x2 fr = f2_set(s_fr[rr], s_fr[rr + 1]), fc2 = f2_set(fc, fc);
+        dd2 n = dd_mul(dd2{f2_set(f0.x, f1.x), f2_set(f0.y, f1.y)}, dd_splat<f32x2>(mu));
+        n = {f2_mul(f2_mul(n.hi, fr), fc2), f2_mul(f2_mul(n.lo, fr), fc2)};
+        dd2 r1, y;
+        regularize(dd_add(dd2{f2_set(h0.x, h1.x), f2_set(h0.y, h1.y)}, dd_splat<f32x2>(dd{hc.x, hc.y})), s, R, &r1, &y);
+        const dd2 x = dd_mul(n, r1);
+        const dd2 k2 = dd_mul(n, dd_add_ordered(dd_splat<f32x2>(dd_make(1.0f)), y));
+        float xh[2], xl[2], kh[2], kl[2];
+        fl_get(x.hi, xh);
+        fl_get(x.lo, xl);
+        fl_get(k2.hi, kh);
+        fl_get(k2.lo, kl);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          if (slot[k] < 0) continue;
+          const bool av = a[k] >= na;
+          if (av && bv) {
+            const long o = ((long)slot[k] * nv + (a[k] - na)) * nv + (b - na);
+            P.tau[o] = make_float2(xh[k], xl[k]);
+            P.kap[o] = make_float2(kh[k], kl[k]);
+          } else if (av) {
+            P.ts[(((long)i[k] * P.nh + j) * nv + (a[k] - na)) * na + b] = dd_to_double(dd{xh[k], xl[k]});
+          } else {
+            P.ts[(((long)j * P.nh + i[k]) * nv + (b - na)) * na + a[k]] = dd_to_double(dd{xh[k], xl[k]});
+          }
         }
       }
     }
@@ -720,27 +718,80 @@ __global__ void __launch_bounds__(256) segment_shift_kernel(int nv, int n_core, 
   exps[(long)P.seg[s].scale * nv + e] = -f;
 }
 
+// Two dressed elements times 2^(fa + fb), rounded, in the pieces of pieces_of<3>:
+// X < 2^40, so hi leaves pieces of 2^30 and 2^15, lo (below 2^16) of 2^15, and
+// what is left of both (below 2^15, rounded to 2^-9 and then to an integer).
+struct Pieces2 {
+  f32x2 x[3];
+};
+__device__ __forceinline__ f32x2 f2_rint(f32x2 v) {
+  return f2_sub(f2_add(v, f2_set(ROUND_MAGIC, ROUND_MAGIC)), f2_set(ROUND_MAGIC, ROUND_MAGIC));
+}
+__device__ __forceinline__ Pieces2 pieces2_of(float4 v, float fa, float fb) {
+  const f32x2 sa = f2_set(fa, fa), sb = f2_set(fb, fb);
+  f32x2 h = f2_mul(f2_mul(f2_set(v.x, v.z), sa), sb), l = f2_mul(f2_mul(f2_set(v.y, v.w), sa), sb);
+  const f32x2 up15 = f2_set(-32768.0f, -32768.0f), dn15 = f2_set(1.0f / 32768.0f, 1.0f / 32768.0f);
+  Pieces2 p;
+  p.x[2] = f2_rint(f2_mul(h, f2_set(1.0f / 1073741824.0f, 1.0f / 1073741824.0f)));
+  h = f2_fma(p.x[2], f2_set(-1073741824.0f, -1073741824.0f), h);
+  const f32x2 h1 = f2_rint(f2_mul(h, dn15)), l1 = f2_rint(f2_mul(l, dn15));
+  p.x[1] = f2_add(h1, l1);
+  p.x[0] = f2_rint(f2_add(f2_fma(h1, up15, h), f2_fma(l1, up15, l)));
+  return p;
+}
+
 // Residue planes [RES_MOD_S][nr][nv][Kpad] of the dressed matrices (double-float
 // rows, contiguous), scaled by their segment's row exponents.  Bound by memory: 8
-// bytes read and 18 written per element.
-__global__ void __launch_bounds__(256) residue_dressed_kernel(const float2* __restrict__ src, int nv, int nr, int Kpad,
+// bytes read and 18 written per element; float32 arithmetic in packed pairs, about
+// 50 instructions per element (165 with 64-bit integers; nvir 600 with 40 core and
+// 10 active orbitals 4.99 -> 3.96 ms, 6.5 TB/s).  Exponents beyond +-126 need two
+// factors.
+__global__ void __launch_bounds__(256, 3) residue_dressed_kernel(const float2* __restrict__ src, int nv, int nr, int Kpad,
                                                               const int* __restrict__ exps, const int* __restrict__ scale_of,
                                                               __nv_bfloat16* __restrict__ planes) {
+  constexpr Tables<RES_MOD_S> T{};
   const long R = (long)nr * nv, row = (long)blockIdx.x * 32 + (threadIdx.x >> 3);
   if (row >= R) return;
   const int r = (int)(row / nv), e = (int)(row - (long)r * nv);
-  int f = -exps[(long)scale_of[r] * nv + e];
-  if (f == SHIFT_INVALID) f = 0;
+  const int ex = exps[(long)scale_of[r] * nv + e];
+  const int f = ex == -SHIFT_INVALID ? 0 : min(max(-ex, -252), 252);
+  const float fa = pow2_float(f / 2), fb = pow2_float(f - f / 2);
+  const bool wide = nv % 2 == 0;  // rows start on 16 bytes
   for (int k0 = (threadIdx.x & 7) * 8; k0 < Kpad; k0 += 64) {
     const float2* p = src + row * nv + k0;
-    Pieces<3> x[8];
+    Pieces2 x[4];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) x[j] = pieces_of<3>(k0 + j < nv ? integer_of(p[j], f) : 0);
+    for (int j = 0; j < 4; ++j) {
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (wide) {
+        if (k0 + 2 * j < nv) v = reinterpret_cast<const float4*>(p)[j];
+      } else {
+        if (k0 + 2 * j < nv) {
+          const float2 q = p[2 * j];
+          v.x = q.x;
+          v.y = q.y;
+        }
+        if (k0 + 2 * j + 1 < nv) {
+          const float2 q = p[2 * j + 1];
+          v.z = q.x;
+          v.w = q.y;
+        }
+      }
+      x[j] = pieces2_of(v, fa, fb);
+    }
 #pragma unroll
     for (int i = 0; i < RES_MOD_S; ++i) {
+      const f32x2 c15 = f2_set(T.c15[i], T.c15[i]), c30 = f2_set(T.c30[i], T.c30[i]), inv = f2_set(T.inv[i], T.inv[i]),
+                  np = f2_set(-T.p[i], -T.p[i]), magic = f2_set(ROUND_MAGIC, ROUND_MAGIC);
       __nv_bfloat162 h[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) h[j] = __floats2bfloat162_rn(residue<RES_MOD_S>(x[2 * j], i), residue<RES_MOD_S>(x[2 * j + 1], i));
+      for (int j = 0; j < 4; ++j) {
+        f32x2 t = f2_fma(x[j].x[2], c30, f2_fma(x[j].x[1], c15, x[j].x[0]));
+        t = f2_fma(f2_sub(f2_fma(t, inv, magic), magic), np, t);
+        float a, b;
+        f2_get(t, &a, &b);
+        h[j] = __floats2bfloat162_rn(a, b);
+      }
       *reinterpret_cast<uint4*>(planes + ((long)i * R + row) * Kpad + k0) = *reinterpret_cast<uint4*>(h);
     }
   }

@@ -4,6 +4,8 @@
 #include <cuda.h>
 #include <stdint.h>
 
+#include "f32x2.cuh"
+
 namespace dsrg {
 namespace tc {
 
@@ -197,28 +199,12 @@ __device__ __forceinline__ void mma2_commit(uint64_t* bar) {
                : "memory");
 }
 
-// ------------------------------------------------ packed float32 pairs (f32x2)
-struct f32x2 {
-  unsigned long long v;
-};
-__device__ __forceinline__ f32x2 f2_set(float a, float b) {
-  f32x2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ void f2_get(f32x2 x, float* a, float* b) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(*a), "=f"(*b) : "l"(x.v));
-}
-__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
-  return r;
-}
-__device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-  return r;
-}
+// packed float32 pairs
+using dsrg::f2_add;
+using dsrg::f2_fma;
+using dsrg::f2_get;
+using dsrg::f2_set;
+using dsrg::f32x2;
 
 // 32 lanes x 16 columns of 32-bit from TMEM (thread t <- lane base+t).
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
