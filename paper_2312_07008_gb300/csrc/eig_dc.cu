@@ -10,11 +10,11 @@
 // SMs: 5.7e6 clocks of the whole chip for n = 1200.  The rest are the n grid
 // barriers of the reduction.  A Jacobi solve moves the whole matrix n - 1
 // times per sweep with a barrier each time and needs 4 to 10 sweeps.  Measured
-// (D_vv-like matrices): n = 1200 18.5 ms (column-pair Jacobi in double-float 97
-// ms), n = 203 1.95 (9.1), n = 90 0.92 (2.7), n = 3600 0.36 s (4.8 s).  Against
+// (D_vv-like matrices): n = 1200 16.8 ms (column-pair Jacobi in double-float 97
+// ms), n = 203 1.6 (9.1), n = 90 0.80 (2.7), n = 3600 0.37 s (4.8 s).  Against
 // the first form of these kernels (27, 3.1, 1.5 ms): leaves of 8 rows instead of
 // 16, deflation by all threads of a block, reciprocals and roots by iteration
-// instead of the library's, scalar work by one warp.
+// instead of the library's, scalar work by one warp beside the rows.
 #include <algorithm>
 
 #include "eig_dc.cuh"
@@ -36,9 +36,7 @@ struct TriArgs {
   int n, rows;      // rows held per block (cyclic: block b has rows b, b + G, ...)
   double* A;        // [n][n]; on return row j holds reflector v_j at k > j
   double *d, *e, *beta;
-  double* pub_p;    // [2][n]
-  double* pub_row;  // [2][n]
-  double* pub_s;    // [2][EIG_MAX_BLOCKS]
+  double* pub;      // [2][2][n]: p and row j + 1 of even and odd steps
   unsigned* bar;    // arrivals, zero at launch
   int* status;      // [1] = 1: a barrier wait expired
   long long spin_limit;
@@ -83,12 +81,13 @@ __device__ __forceinline__ double warp_sum(double x) { return WarpLane().sum(x);
 // update left from step j - 1 and multiplies by the new reflector:
 //   A -= v w^T + w v^T with w = beta p - K v, K = beta^2 (p.v) / 2, so
 //   A_ik -= (beta v_i) p_k + (beta p_i - 2 K v_i) v_k,   p'_i = sum_k A_ik v'_k.
-// The products p', their dot with v' and row j + 1 are published, and one grid
-// barrier later every block forms row j + 1 of the next matrix by itself: one
-// barrier per step, A read and written once per step, from shared memory as
-// long as a block's rows fit (SM).  (One cluster of 16 blocks for small n, its
-// hardware barrier and shared memory in place of the grid barrier and the
-// published arrays, took the same 6 us per step at n = 203.)
+// The products p' and row j + 1 are published, and every block forms p'.v' and
+// row j + 1 of the next matrix by itself.  A is read and written once per step,
+// from shared memory as long as a block's rows fit (SM).  A step is a chain of
+// two block sums, the rows and one grid barrier: n = 203 1.95 -> 1.59 ms for the
+// whole solve, n = 1200 18.5 -> 16.8, against a reflector formed before the rows.
+// (Words tagged with the step's number and polled for in place of the barrier: n =
+// 90 0.80 -> 0.75, n = 203 1.57, n = 300 2.30 -> 2.39, twice the bytes.)
 template <bool SM>
 __global__ void __launch_bounds__(TNT) tridiag_kernel(TriArgs P) {
   extern __shared__ double smem[];
@@ -96,8 +95,9 @@ __global__ void __launch_bounds__(TNT) tridiag_kernel(TriArgs P) {
   double* pv = smem;        // p of the previous step
   double* v0 = pv + n;      // v of the previous step
   double* v1 = v0 + n;      // v of this step
-  double* As = v1 + n;      // own rows (SM)
-  __shared__ double part[TNT], sc[4];
+  double* rp = v1 + n;      // products of the own rows
+  double* As = rp + P.rows; // own rows (SM)
+  __shared__ double part[TNT], sc[5];
   auto row_ptr = [&](int li) { return SM ? As + (long)li * n : P.A + (long)(b + li * G) * n; };
   // sum of the threads' parts, by warp 0 (scalar work costs every warp that
   // repeats it 16 clocks an instruction of the SM's float64 lanes)
@@ -124,8 +124,15 @@ __global__ void __launch_bounds__(TNT) tridiag_kernel(TriArgs P) {
   double beta0 = 0.0, K2 = 0.0;         // of the previous step (none yet)
   for (int j = 0; j < n - 2; ++j) {
     // ---- reflector from row j (v1 holds A[j][k], k > j; s2 this thread's part of |r_{k > j + 1}|^2)
+    // The rows need v_j only in their products, and there only element j + 1 is
+    // not yet known: warp 0 forms the reflector while the others update the rows
+    // and multiply by the elements beyond.
     part[tid] = s2;
     __syncthreads();
+    double* pp = P.pub + (long)(j & 1) * 2 * n;
+    double* pr = pp + n;
+    const int li0 = b > j ? 0 : (j - b) / G + 1;  // first own row above j
+    const int kbeg = (j + 1) & ~31;
     if (warp == 0) {
       const double sig = total();
       double ej = alpha, bt = 0.0, v = alpha;
@@ -137,99 +144,91 @@ __global__ void __launch_bounds__(TNT) tridiag_kernel(TriArgs P) {
         v = alpha - ej;
       }
       if (lane == 0) {
-        v1[j + 1] = v;
         sc[0] = bt;
-        if (b == 0) {
+        sc[1] = v;
+        if (b == (j + 1) % G) {
           P.d[j] = dj;
           P.e[j] = ej;
           P.beta[j] = bt;
         }
       }
     }
-    __syncthreads();
-    const double beta = sc[0];
-    if (b == j % G)
-      for (int k = j + 1 + tid; k < n; k += TNT) P.A[(long)j * n + k] = v1[k];
-    // ---- own rows: pending update and product with the new reflector
-    const int buf = j & 1;
-    double* pp = P.pub_p + (long)buf * n;
-    double* pr = P.pub_row + (long)buf * n;
-    double sw = 0.0;
-    const int li0 = b > j ? 0 : (j - b) / G + 1;  // first own row above j
-    const int kbeg = (j + 1) & ~31;
-    for (int li = li0 + warp; b + li * G < n; li += TNW) {
-      const int i = b + li * G;
-      double* row = row_ptr(li);
-      const double c1 = -beta0 * v0[i], c2 = fma(K2, v0[i], -beta0 * pv[i]);
-      // four partial sums: a chain of float64 FMAs waits for each of them
-      double acc[4] = {0.0, 0.0, 0.0, 0.0};
-      const bool pub = i == j + 1;
-      for (int k0 = kbeg + lane; k0 < n; k0 += 128) {
+    if (!SM || warp > 0) {  // rows in global memory: warp 0 takes its share of them as well
+      for (int li = li0 + (SM ? warp - 1 : warp); b + li * G < n; li += SM ? TNW - 1 : TNW) {
+        const int i = b + li * G;
+        double* row = row_ptr(li);
+        const double c1 = -beta0 * v0[i], c2 = fma(K2, v0[i], -beta0 * pv[i]);
+        // four partial sums: a chain of float64 FMAs waits for each of them
+        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+        const bool pub = i == j + 1;
+        for (int k0 = kbeg + lane; k0 < n; k0 += 128) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int k = k0 + 32 * u;
-          if (k > j && k < n) {
-            double a = row[k];
-            if (j > 0) {
-              a = fma(c1, pv[k], fma(c2, v0[k], a));
-              row[k] = a;
+          for (int u = 0; u < 4; ++u) {
+            const int k = k0 + 32 * u;
+            if (k > j && k < n) {
+              double a = row[k];
+              if (j > 0) {
+                a = fma(c1, pv[k], fma(c2, v0[k], a));
+                row[k] = a;
+              }
+              if (k > j + 1) acc[u] = fma(a, v1[k], acc[u]);
+              if (pub) __stcg(pr + k, a);
             }
-            acc[u] = fma(a, v1[k], acc[u]);
-            if (pub) __stcg(pr + k, a);
           }
         }
-      }
-      double ps = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-      sw = fma(ps, v1[i], sw);  // p.v in lane parts
-      ps = warp_sum(ps);
-      if (lane == 0) __stcg(pp + i, ps);
-      if (j == n - 3 && i == n - 1) {  // the last diagonal element (its lane wrote it)
-        __syncwarp();
-        if (lane == 0) __stcg(pr, row[n - 1]);
+        const double ps = warp_sum((acc[0] + acc[1]) + (acc[2] + acc[3]));
+        if (lane == 0) rp[li] = ps;
       }
     }
-    part[tid] = sw;
     __syncthreads();
-    if (warp == 0) {
-      const double s = total();
-      if (lane == 0) __stcg(P.pub_s + buf * EIG_MAX_BLOCKS + b, s);
+    const double beta = sc[0];
+    for (int li = li0 + tid; b + li * G < n; li += TNT) {
+      const int i = b + li * G;
+      const double p = fma(row_ptr(li)[j + 1], sc[1], rp[li]);
+      __stcg(pp + i, p);
     }
-    target += G;
-    if (!tri_barrier(P, target)) return;
+    if (tid == TNT - 1) v1[j + 1] = sc[1];
+    if (b == (j + 1) % G)
+      for (int k = j + 1 + tid; k < n; k += TNT) P.A[(long)j * n + k] = k == j + 1 ? sc[1] : v1[k];
     // ---- p, p.v and row j + 1 of the next matrix
     const int i = j + 1;
+    target += G;
+    if (!tri_barrier(P, target)) return;
     double* vt = v0;
     v0 = v1;
     v1 = vt;
+    double dot = 0.0;
     for (int k = i + tid; k < n; k += TNT) {
       pv[k] = __ldcg(pp + k);
       v1[k] = __ldcg(pr + k);
+      dot = fma(pv[k], v0[k], dot);
     }
+    part[tid] = dot;
+    __syncthreads();
     beta0 = beta;
     if (warp == 0) {
-      const double pi = __ldcg(pp + i), pi1 = __ldcg(pp + i + 1), ri = __ldcg(pr + i), ri1 = __ldcg(pr + i + 1);
-      double s = 0.0;
-      for (int g = lane; g < G; g += 32) s += __ldcg(P.pub_s + buf * EIG_MAX_BLOCKS + g);
-      s = warp_sum(s);
-      const double k2 = beta * (beta * s), vi = v0[i];  // beta^2 may overflow
+      const double s = total();
+      const double k2 = beta * (beta * s), vi = v0[i], pi = pv[i];  // beta^2 may overflow
       const double c1 = -beta * vi, c2 = fma(k2, vi, -beta * pi);
-      dj = fma(c1, pi, fma(c2, vi, ri));
-      alpha = fma(c1, pi1, fma(c2, v0[i + 1], ri1));
+      dj = fma(c1, pi, fma(c2, vi, v1[i]));
+      alpha = fma(c1, pv[i + 1], fma(c2, v0[i + 1], v1[i + 1]));
       if (lane == 0) {
-        sc[1] = k2;
-        sc[2] = c1;
-        sc[3] = c2;
-        if (j == n - 3 && b == 0) {
-          const double pl = __ldcg(pp + n - 1), vl = v0[n - 1];
+        sc[2] = k2;
+        sc[3] = c1;
+        sc[4] = c2;
+      }
+      if (j == n - 3 && b == (n - 1) % G) {  // the last 2 x 2, by the owner of row n - 1
+        const double pl = pv[n - 1], vl = v0[n - 1];
+        if (lane == 0) {
           P.d[n - 2] = dj;
           P.e[n - 2] = alpha;
-          P.d[n - 1] = fma(-beta * vl, pl, fma(fma(k2, vl, -beta * pl), vl, __ldcg(pr)));
+          P.d[n - 1] = fma(-beta * vl, pl, fma(fma(k2, vl, -beta * pl), vl, row_ptr((n - 1) / G)[n - 1]));
         }
       }
     }
     __syncthreads();
-    K2 = sc[1];
-    const double c1 = sc[2], c2 = sc[3];
+    K2 = sc[2];
+    const double c1 = sc[3], c2 = sc[4];
     s2 = 0.0;
     for (int k = i + 1 + tid; k < n; k += TNT) {
       const double r = fma(c1, pv[k], fma(c2, v0[k], v1[k]));
@@ -755,9 +754,7 @@ int eig_dc(int n, double* A, double* V, double* work, unsigned* bar, int* status
   T.d = take(1);
   T.e = take(1);
   T.beta = take(1);
-  T.pub_p = take(2);
-  T.pub_row = take(2);
-  T.pub_s = red;
+  T.pub = take(4);
   T.bar = bar;
   T.status = status_dev;
   T.spin_limit = spin_limit;
@@ -790,7 +787,7 @@ int eig_dc(int n, double* A, double* V, double* work, unsigned* bar, int* status
   const int per = shared ? 8 : 4;
   const int G = std::max(1, std::min(std::min(shared ? sms / 2 : sms, EIG_MAX_BLOCKS), ceil_div(n, per)));
   T.rows = ceil_div(n, G);
-  const size_t vec = 3 * sizeof(double) * (size_t)n, own = sizeof(double) * (size_t)n * T.rows;
+  const size_t vec = sizeof(double) * (3 * (size_t)n + T.rows), own = sizeof(double) * (size_t)n * T.rows;
   const bool in_smem = vec + own <= TRI_SMEM;
   const size_t smem = vec + (in_smem ? own : 0);
   if (smem > TRI_SMEM) return DSRG_FNO_ERR_UNSUPPORTED;
