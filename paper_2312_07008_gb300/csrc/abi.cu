@@ -300,13 +300,24 @@ static size_t plan_budget(const Workspace& ws) { return device_budget(ws.cap); }
 
 // Batches of pairs that fit the budget.  The residues of 4096 output tiles (5.4
 // GB, 54 rounds of units on 76 pairs of SMs) lose nothing to the launches' last
-// rounds; a small budget holds an eighth of itself, at least 64 tiles.
-static void make_plan(const Geometry& g, int ks, int2 pform, size_t budget, Plan& P) {
+// rounds; a small budget holds an eighth of itself, at least 64 tiles.  What the
+// residue form holds beside the batches and five digit planes would not (ten
+// planes of B and of the small terms' operands, the update's residues) comes off
+// the budget, so that a pass's workspace is no larger than theirs: several batch
+// workers' passes stand beside each other and the inputs.
+static void make_plan(const Geometry& g, int ks, int2 pform, size_t budget, bool want_d, Plan& P) {
   const bool rf = residue_form(ks, pform);
   const size_t tile = residue_tile_bytes(RES_MOD);
   if (rf) P.res_cap = (int)std::max<size_t>(64, std::min<size_t>(4096, budget / 8 / tile));
   const size_t held = rf ? std::min(budget / 8, (size_t)P.res_cap * tile) : 0;
-  build_plan(g.nc, g.na, pair_cap_for_budget(g.nv, g.np, ks, rf, budget - held), P);
+  size_t avail = budget - held;
+  if (rf) {
+    size_t more = (size_t)(RES_MOD - 5) * 2 * g.nh * g.np * pad64(g.nq);
+    if (want_d)
+      more += residue_syrk_res_bytes(g.nv) + (size_t)(RES_MOD - 5) * 2 * 2 * g.nv * pad64(small_terms_kmax(g.nc, g.na));
+    avail = std::max(avail / 4, avail > more ? avail - more : 0);
+  }
+  build_plan(g.nc, g.na, pair_cap_for_budget(g.nv, g.np, ks, rf, avail), P);
   if (rf) {
     int most = 1;
     for (const Batch& b : P.batches) most = std::max(most, pair_tile_bound(RES_TILE, RES_TILE, g, b.npairs));
@@ -616,7 +627,7 @@ static int energy_pass(const Geometry& g, int ks, int2 pform, const double* B, c
                        const double* lambda2, Workspace& ws, size_t base_off, size_t budget, double* e_out,
                        cudaStream_t st) {
   Plan P;
-  make_plan(g, ks, pform, budget, P);
+  make_plan(g, ks, pform, budget, false, P);
   ws.off = base_off;
   PassBuffers W{};
   size_t need = base_off + pass_bytes(g, P, false, 1, ks, pform);
@@ -630,7 +641,7 @@ static int energy_pass(const Geometry& g, int ks, int2 pform, const double* B, c
 
 static size_t energy_pass_bytes(const Geometry& g, int ks, int2 pform, size_t budget) {
   Plan P;
-  make_plan(g, ks, pform, budget, P);
+  make_plan(g, ks, pform, budget, false, P);
   return pass_bytes(g, P, false, 1, ks, pform);
 }
 
@@ -695,7 +706,7 @@ int impl_vv_opdm(Workspace& ws, size_t budget, const dsrg_fno_problem* prob, dou
   const int ks = slices_of(prob);
   const int2 pform = pair_form_of(prob, ks);
   Plan P;
-  make_plan(g, ks, pform, budget, P);
+  make_plan(g, ks, pform, budget, true, P);
   const int nsplit = nsplit_for(g.nv, P.max_out, ks ? syrk_slices(ks) : 0);
   const size_t small = small_terms_work_doubles(g.nc, g.na, g.nv);
   const int kmax = small_terms_kmax(g.nc, g.na);

@@ -34,6 +34,7 @@ struct Worker {
   Workspace ws;
   cudaStream_t stream = nullptr;
   cudaEvent_t done = nullptr;
+  size_t planned = 0;  // largest share of the memory its workspace was planned with
 };
 
 struct DevicePool {
@@ -141,6 +142,17 @@ extern "C" int dsrg_fno_batch_run(dsrg_fno_batch_item* items, int32_t n, int32_t
   size_t have = 0;
   for (int k = 0; k < workers; ++k) have += pool.w[k].ws.cap;
   const size_t share = device_budget(have) / (size_t)workers;
+  // workspaces planned for fewer workers with larger shares go back first: beside
+  // them the shares of all workers need not fit
+  for (Worker& w : pool.w) {
+    if (w.ws.base && w.planned > share + share / 2) {
+      DSRG_CUDA(cudaStreamSynchronize(w.stream));
+      DSRG_CUDA(cudaFree(w.ws.base));
+      w.ws = Workspace{};
+      w.planned = 0;
+    }
+  }
+  for (int k = 0; k < workers; ++k) pool.w[k].planned = std::max(pool.w[k].planned, share);
 
   const auto t0 = std::chrono::steady_clock::now();
   std::atomic<int> next{0};
@@ -194,6 +206,7 @@ void release_batch_pools() {
     for (int k = 0; k < MAX_WORKERS; ++k) {
       Worker& w = pool.w[k];
       if (w.ws.base) cudaFree(w.ws.base);
+      w.planned = 0;
       w.ws = Workspace{};
       if (w.stream) cudaStreamDestroy(w.stream);
       if (w.done) cudaEventDestroy(w.done);

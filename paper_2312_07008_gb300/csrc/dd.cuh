@@ -142,17 +142,6 @@ __device__ __forceinline__ ddt<T> dd_mul_f(ddt<T> a, T b) {
   return quick_two_sum(p.hi, p.lo);
 }
 
-// a / b: float reciprocal estimate, one dd correction step
-__device__ __forceinline__ dd dd_div(dd a, dd b) {
-  const float q1 = __fdiv_rn(a.hi, b.hi);
-  const dd r = dd_sub(a, dd_mul_f(b, q1));
-  const float q2 = __fdiv_rn(r.hi, b.hi);
-  const dd r2 = dd_sub(r, dd_mul_f(b, q2));
-  const float q3 = __fdiv_rn(r2.hi, b.hi);
-  dd q = quick_two_sum(q1, q2);
-  return dd_add_f(q, q3);
-}
-
 // 1 / b by Newton's iteration r + r (1 - b r) with fused multiply-adds (Markstein,
 // IBM J. Res. Dev. 34, 1990): from the hardware's approximation to float32, where
 // 1 - b.hi r is exact, and from there to double-float: relative error about 2^-46.
@@ -174,8 +163,6 @@ __device__ __forceinline__ ddt<T> dd_recip(ddt<T> b) {
   const T e = fl_sub(fl_fma(nh, r, one), fl_mul(b.lo, r));
   return quick_two_sum(r, fl_mul(r, e));
 }
-
-__device__ __forceinline__ dd dd_ldexp(dd a, int e) { return {ldexpf(a.hi, e), ldexpf(a.lo, e)}; }
 
 __device__ __forceinline__ dd dd_from_double(double x) {
   const float h = __double2float_rn(x);
