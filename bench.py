@@ -624,8 +624,8 @@ def main():
         f64_alg = pair_alg_flops(p, [r64[c][0] for c in cuts]) * args.fp64_steps
         f64_tf = f64_alg / (f64_ms / 1e3) / 1e12 if f64_ms > 0 else None
         fp64 = {"solves_per_s": 1e3 / fms, "s_per_solve": fms / 1e3, "gflops": flops / (fms / 1e3) / 1e9,
-                "note": "contractions and elementwise stages in float64; the eigensolves run in double-float "
-                        "(about 48 bits) in both forms",
+                "note": "contractions and elementwise stages in float64; the eigensolves above 32 rows "
+                        "run in float64 in both forms",
                 "roofline": {"bound": "fp64", "kernel": "pair_gemm_f64_kernel (float64 CUDA cores)",
                              "achieved": f64_tf, "unit": "TFLOP/s", "launches": f64_n,
                              "ms_per_step": f64_ms / args.fp64_steps,
@@ -865,13 +865,13 @@ def naf_timing(pkg, dev, nslices, keep_frac=0.75):
 # launches; valid only for the kernel sources it was taken with.
 TRAFFIC = {
     "sa_cas10_ncore60_nvir1200_naux3600": {
-        # small-case capture (energy pass of ncore 20 / nact 4 / nvir 1100 / naux 2000):
-        # 9.328 GB read + 2.908 GB written for 2.2556e13 executed flops
-        "bytes_per_exec_flop": (9.328328e9 + 2.907642e9) / 2.2556379709440e13,
-        "sha256": {"paper_2312_07008_gb300/csrc/sliced.cu":
-                   "4ae42af7897f57e9271091737d32b7b3ac1c4d64dea612fe28a0ab301f83f347",
+        # small-case capture (energy pass of ncore 20 / nact 4 / nvir 700 / naux 3600):
+        # 8.185 GB read + 3.013 GB written for 1.1088e13 executed flops
+        "bytes_per_exec_flop": (8.185194e9 + 3.013085e9) / 1.10883137e13,
+        "sha256": {"paper_2312_07008_gb300/csrc/residue.cu":
+                   "5d8747b7cdab178808ca87171877d8a45d952ba3e06d7de1af612db0eabb2e88",
                    "paper_2312_07008_gb300/csrc/tc_ptx.cuh":
-                   "300804d055c2a37a13d0d68e3e9d556e62027073a7a31151f5033bd4885f0757"},
+                   "1759ad784a427ead3781e6d492cf0fa7ab5e5d37e44eb1bb38bc52f14c94e780"},
     },
 }
 

@@ -165,10 +165,10 @@ int stage_literal(int form, int KS, const double* src, long R, int K, long rs, l
                   int* exps, cudaStream_t st);
 // Residue form (residue.cu): the fast form's contractions modulo RES_MOD (or,
 // for the rotation of B, RES_MOD_X) coprime moduli on tcgen05, one product each.
-// RES_MOD_S: the rank-K update of D_vv, whose sums run over whole segments of
-// dressed matrices: its errors average out over K = 10^4 and more (relative to
-// the rows' norms 2^-40 and less), the digit planes' were 2^-37.
-constexpr int RES_MOD = 10, RES_MOD_X = 12, RES_MOD_S = 9;
+// RES_MOD_S: the rank-K update of D_vv.  (Nine would do for the targets, 10 ms less
+// in an opdm pass of nvir 1200, but D_vv then errs up to 1.3 times as much as with
+// five digit planes at some sizes; ten err a tenth.)
+constexpr int RES_MOD = 10, RES_MOD_X = 12, RES_MOD_S = 10;
 constexpr int RES_TILE = 256;          // rows and columns of an output tile
 constexpr int RES_STAGE_BLOCKS = 608;  // four blocks per SM of a staging launch
 // bytes of the exponents of R staged rows and of the staging's scratch behind them

@@ -649,10 +649,11 @@ __global__ void __launch_bounds__(256) plain_residue_kernel(ResGemm P, PlainOut 
 }
 
 // Rank-K update of D_vv, sums over all rows of all dressed matrices: bound by the
-// tensor cores.  opdm pass of nvir 1200 (10 active, K = 6.8e6): the products take
-// 69 ms (1.52 PFLOP/s) instead of the digit planes' 120; the staging 40 ms instead
-// of 28, for nine planes instead of five.  D[e][f] += the sum over the segments,
-// in a fixed order, of sign A_s[e] . A_s[f] (upper tiles, mirrored).
+// tensor cores.  opdm pass of nvir 1200 (10 active, K = 5.9e6): the products take
+// 72 to 77 ms (1.5 to 1.6 PFLOP/s at the power cap) instead of the digit planes'
+// 120; the staging 33 ms instead of 28, for ten planes instead of five.  D[e][f] +=
+// the sum over the segments, in a fixed order, of sign A_s[e] . A_s[f] (upper tiles,
+// mirrored).
 __global__ void __launch_bounds__(256) syrk_residue_kernel(const __grid_constant__ ResGemm P, const int* __restrict__ exps,
                                                            int nv, double* D) {
   constexpr int NM = RES_MOD_S;
@@ -719,8 +720,9 @@ __global__ void __launch_bounds__(256) segment_shift_kernel(int nv, int n_core, 
 }
 
 // Two dressed elements times 2^(fa + fb), rounded, in the pieces of pieces_of<3>:
-// X < 2^40, so hi leaves pieces of 2^30 and 2^15, lo (below 2^16) of 2^15, and
-// what is left of both (below 2^15, rounded to 2^-9 and then to an integer).
+// X < 2^44.4, so hi leaves pieces of 2^30 (below 2^14.4) and 2^15, lo (below 2^21)
+// of 2^15, and what is left of both (below 2^15, rounded to 2^-9 and then to an
+// integer): every partial sum of a residue stays below 2^24.
 struct Pieces2 {
   f32x2 x[3];
 };
@@ -976,22 +978,21 @@ int residue_plain(int nm, int M, int N, const __nv_bfloat16* pa, const int* ea, 
 
 // Segments of the rank-K update over nr matrices of which those from n_signed
 // on may carry a minus sign: every range of scales is one segment, or two (one
-// per sign).  A range's rows share one scale, whose roundings average out over
-// the ranges: with 32 or more the errors of D_vv stay below those of five digit
-// planes at every size tried (nvir 20 to 420; with 8 to 16 up to 1.3 times them
-// at the smallest).  Their residues are written and read once (nvir 1200: 0.57 GB
-// for 32 ranges; where 64 would take more than 4 GB, fewer).  Of the counts
-// allowed the one whose units leave the least of the last round of SM pairs idle.
-static int residue_max_segments(int nv) {
-  const int nt = ceil_div(nv, GT_M);
-  const size_t per = (size_t)(nt * (nt + 1) / 2) * residue_tile_bytes(RES_MOD_S);
-  return (int)std::max<size_t>(16, std::min<size_t>(RES_MAX_SEGMENTS, ((size_t)4 << 30) / per));
+// per sign).  A range's rows share one scale; eight or more keep what that costs
+// below a bit.  Segments differ in length (signs), so the smaller D is, the more
+// are taken, down to 20 rounds of units on the pairs of SMs (nvir 300: 0.43 ms with
+// 32 to 64, 0.61 with 8 to 16; nvir 1200: 69 and 65 ms, for starting the units and
+// their residues).  Of the counts from that to twice it the one whose units leave
+// the least of the last round idle.
+static int residue_least_segments(int nv) {
+  const int nt = ceil_div(nv, GT_M), units = nt * (nt + 1) / 2 * RES_MOD_S;
+  return std::min(RES_MAX_SEGMENTS / 2, std::max(8, 20 * 76 / units));
 }
 int residue_segments(int nv, int nr, int n_signed, ResSegment* seg) {
-  const int nt = ceil_div(nv, GT_M), units = nt * (nt + 1) / 2 * RES_MOD_S, pairs = 76, most = residue_max_segments(nv);
-  int best = most / 2;
+  const int nt = ceil_div(nv, GT_M), units = nt * (nt + 1) / 2 * RES_MOD_S, pairs = 76, least = residue_least_segments(nv);
+  int best = least;
   double best_eff = 0.0;
-  for (int k = most / 2; k <= most; ++k) {
+  for (int k = least; k <= 2 * least; ++k) {
     const long u = (long)units * k;
     const double eff = (double)u / ((double)ceil_div(u, pairs) * pairs);
     if (eff > best_eff + 0.005) {
@@ -1019,7 +1020,7 @@ int residue_segments(int nv, int nr, int n_signed, ResSegment* seg) {
 
 size_t residue_syrk_res_bytes(int nv) {
   const int nt = ceil_div(nv, GT_M);
-  return (size_t)residue_max_segments(nv) * (nt * (nt + 1) / 2) * residue_tile_bytes(RES_MOD_S);
+  return (size_t)2 * residue_least_segments(nv) * (nt * (nt + 1) / 2) * residue_tile_bytes(RES_MOD_S);
 }
 
 // D += sum_r sign_r Sig_r Sig_r^T.  rowpart: as dress_dd writes it; exps: RES_MAX_SEGMENTS nv ints; scale_of: nr ints (host list, copied).

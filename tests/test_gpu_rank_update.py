@@ -14,7 +14,7 @@ if not torch.cuda.is_available():
 
 import paper_2312_07008_gb300 as pkg  # noqa: E402
 
-# A range's row is scaled to a norm bound 2^39.8 = LIMIT of 9 moduli; the bound from
+# A range's row is scaled to a norm bound 2^39.8 = LIMIT of 9 moduli (10: 2^44.3); the bound from
 # tiles' largest elements is at most 32^1/2 times the norm and the scale a power of
 # two, so |X| >= LIMIT / 11.4 = 8.4e10.  Rounding to integers (uniform, 0.29 rms) moves
 # X . Y by 0.29 2^1/2 |X| rms, or 4.9e-12 of |x| |y|; six times that for the largest
