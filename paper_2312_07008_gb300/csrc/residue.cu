@@ -159,7 +159,7 @@ struct ResGemm {
   int* err;
 };
 
-__constant__ float c_mod[NMAX], c_inv[NMAX];
+__constant__ ModulusTable c_moduli = ModulusTable();
 
 // unit -> tile, modulus and matrices [r0, r1); the moduli of a segment run one
 // after another over all its tiles, so that a modulus's planes stay in L2
@@ -333,7 +333,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(G_THREADS, 1)
     bool failed = false;
     for (long u = cluster; u < P.nunits && !failed; u += nclusters) {
       const ResUnit x = rg_decode(P, u);
-      const float p = c_mod[x.mod], inv = c_inv[x.mod];
+      const float p = c_moduli.p[x.mod], inv = c_moduli.inv[x.mod];
       int nk = 0;
       for (int r = x.r0 + lane; r < x.r1; r += 32) nk += rg_takes(P, x, r) ? P.nkb : 0;
       nk = __reduce_add_sync(0xffffffffu, nk);
@@ -817,32 +817,10 @@ int plane_map(CUtensorMap* map, const void* planes, int nm, long nr, long rows, 
   return r == CUDA_SUCCESS ? DSRG_FNO_OK : DSRG_FNO_ERR_CUDA;
 }
 
-// the moduli of the contraction kernel, copied to the current device once
-int moduli_ready() {
-  static std::mutex mu;
-  static bool ready[64] = {};
-  int dev = 0;
-  DSRG_CUDA(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= 64) return DSRG_FNO_ERR_UNSUPPORTED;
-  std::lock_guard<std::mutex> lk(mu);
-  if (!ready[dev]) {
-    float m[NMAX], inv[NMAX];
-    for (int i = 0; i < NMAX; ++i) {
-      m[i] = (float)modulus(i);
-      inv[i] = 1.0f / (float)modulus(i);
-    }
-    DSRG_CUDA(cudaMemcpyToSymbol(c_mod, m, sizeof(m)));
-    DSRG_CUDA(cudaMemcpyToSymbol(c_inv, inv, sizeof(inv)));
-    ready[dev] = true;
-  }
-  return DSRG_FNO_OK;
-}
-
 int launch_gemm(const void* pa, long rows_a, const void* pb, long rows_b, int Kpad, ResGemm P, cudaStream_t st) {
   if (P.nunits <= 0) return DSRG_FNO_OK;
   if (Kpad % 64 != 0) return DSRG_FNO_ERR_ARG;
   P.nkb = Kpad / 64;
-  DSRG_TRY(moduli_ready());
   CUtensorMap ma, mb;
   DSRG_TRY(plane_map(&ma, pa, P.nm, P.nr, rows_a, Kpad));
   DSRG_TRY(plane_map(&mb, pb, P.nm, P.nr, rows_b, Kpad));

@@ -63,6 +63,18 @@ struct Tables {
   }
 };
 
+// p and 1 / p of every modulus: the contraction kernel's constant memory, initialised
+// with the module, so that no launch on any stream can precede it.
+struct ModulusTable {
+  float p[NMAX], inv[NMAX];
+  constexpr ModulusTable() : p{}, inv{} {
+    for (int i = 0; i < NMAX; ++i) {
+      p[i] = (float)modulus(i);
+      inv[i] = 1.0f / (float)modulus(i);
+    }
+  }
+};
+
 // M / 2 = mantissa 2^exponent, mantissa in [1, 2)
 constexpr double crt_half_mantissa(int nm) {
   double m = 0.5;
