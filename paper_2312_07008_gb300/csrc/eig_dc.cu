@@ -29,6 +29,9 @@ using namespace dc;
 constexpr int TNT = 256;                   // threads per block of the reduction
 constexpr int TNW = TNT / 32;
 constexpr size_t TRI_SMEM = 200 * 1024;
+// the deflation of the largest matrix beside its 1040 bytes of static shared memory
+constexpr int DC_DEFLATE_SMEM = DC_DEFLATE_ROW_BYTES * EIG_DC_MAX_N;
+static_assert(DC_DEFLATE_SMEM + 1040 <= 232448, "shared memory per block");
 constexpr double RSQRT2 = 0.70710678118654752440;
 
 // ------------------------------------------------------------- reduction
@@ -803,14 +806,14 @@ int eig_dc(int n, double* A, double* V, double* work, unsigned* bar, int* status
   D.Qout = Q0;
   dc_leaf_kernel<<<1 << D.levels, 32, 0, st>>>(D);
   DSRG_LAUNCH_CHECK();
-  DSRG_CUDA(cudaFuncSetAttribute(dc_deflate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 30 * EIG_DC_MAX_N));
+  DSRG_CUDA(cudaFuncSetAttribute(dc_deflate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DC_DEFLATE_SMEM));
   for (int l = D.levels - 1; l >= 0; --l) {
     std::swap(Q0, Q1);
     D.level = l;
     D.Qin = Q1;
     D.Qout = Q0;
-    const int nodes = 1 << l, mmax = ceil_div(n, nodes) + 1, hmax = ceil_div(mmax, 2) + 1;
-    dc_deflate_kernel<<<nodes, 256, 30 * (size_t)mmax, st>>>(D);
+    const int nodes = 1 << l, mmax = dc_node_rows(n, l), hmax = dc_node_rows(n, l + 1);
+    dc_deflate_kernel<<<nodes, 256, dc_deflate_bytes(n, l), st>>>(D);
     DSRG_LAUNCH_CHECK();
     const int rb = ceil_div(n, 32);
     dc_secular_kernel<<<rb + n, 32, 0, st>>>(D, rb);
@@ -819,7 +822,7 @@ int eig_dc(int n, double* A, double* V, double* work, unsigned* bar, int* status
     DSRG_LAUNCH_CHECK();
     dc_vectors_kernel<<<n, 32, 0, st>>>(D);
     DSRG_LAUNCH_CHECK();
-    if (mmax <= 512) dc_gemm_kernel<16><<<dim3(ceil_div(hmax, 16), ceil_div(mmax, 16), 2 * nodes), 256, 0, st>>>(D);
+    if (mmax < 512) dc_gemm_kernel<16><<<dim3(ceil_div(hmax, 16), ceil_div(mmax, 16), 2 * nodes), 256, 0, st>>>(D);
     else dc_gemm_kernel<32><<<dim3(ceil_div(hmax, 32), ceil_div(mmax, 32), 2 * nodes), 256, 0, st>>>(D);
     DSRG_LAUNCH_CHECK();
   }

@@ -32,6 +32,13 @@ DC_HD int dc_levels(int n) {
 // first row of node t on level l (the nodes of level l + 1 halve them)
 DC_HD int dc_bound(int n, int l, int t) { return (int)(((long)t * n) >> l); }
 
+// rows of the largest node of level l (a node is at most one row longer than another)
+DC_HD int dc_node_rows(int n, int l) { return (n + (1 << l) - 1) >> l; }
+// shared memory of the deflation on level l: sorted d and z, keys, order, type and
+// flag of every row of a node
+constexpr int DC_DEFLATE_ROW_BYTES = 8 + 8 + 8 + 4 + 1 + 1;
+DC_HD int dc_deflate_bytes(int n, int l) { return DC_DEFLATE_ROW_BYTES * dc_node_rows(n, l); }
+
 // 1 / x, 1 / sqrt(x) and sqrt(x) from a float32 estimate and one step of third
 // order (relative error of a few 2^-53): chains of 3 to 5 float64 instructions
 // where the library's take 15 to 30; an SM has two float64 lanes, and a chain of
