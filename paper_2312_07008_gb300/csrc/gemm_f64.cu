@@ -9,6 +9,7 @@
 // GB300 runs float64 at a small fraction of its float32 rate, so these
 // kernels are float64-pipe bound by construction; they are the plain form
 // the sliced tensor-core form is measured against.
+#include "gemm_tile.h"
 #include "kernels.h"
 
 namespace dsrg {
@@ -152,23 +153,6 @@ void launch_gemm_f64(int T, int M, int N, int K, double alpha, const double* A, 
     gemm_f64_kernel<A_KC, B_KC, 16><<<grid, NT, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, sa, sb, sc);
 }
 
-// Tile edge: the one whose fullest SM does the least float64 work (blocks per
-// SM times T^2; the larger on a tie, which reads less).
-int gemm_tile(int M, int N, int batch) {
-  const int sms = 152;
-  int best = 64;
-  long best_cost = 0;
-  for (int T : {64, 32, 16}) {
-    const long blocks = (long)ceil_div(M, T) * ceil_div(N, T) * batch;
-    const long cost = (long)ceil_div(blocks, sms) * T * T;
-    if (best_cost == 0 || cost * 10 < best_cost * 9) {
-      best_cost = cost;
-      best = T;
-    }
-  }
-  return best;
-}
-
 // ---------------------------------------------------------------------------
 // Pair contraction with the regulariser epilogue.
 // Rows a and columns b run over the particles (active first).  The operands
@@ -307,7 +291,7 @@ int gemm_f64(int M, int N, int K, double alpha, const double* A, long lda, bool 
              const double* B, long ldb, bool b_kcontig, double beta, double* C, long ldc, int batch,
              long sa, long sb, long sc, cudaStream_t st) {
   if (M <= 0 || N <= 0 || batch <= 0) return DSRG_FNO_OK;
-  const int T = gemm_tile(M, N, batch);
+  const int T = gemm_f64_tile(M, N, batch);
   auto go = a_kcontig ? (b_kcontig ? launch_gemm_f64<true, true> : launch_gemm_f64<true, false>)
                       : (b_kcontig ? launch_gemm_f64<false, true> : launch_gemm_f64<false, false>);
   go(T, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, batch, sa, sb, sc, st);
