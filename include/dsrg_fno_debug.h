@@ -103,6 +103,10 @@ int dsrg_fno_debug_eig_batch(int32_t count, const int32_t* n, double* const* A, 
  * Host only: reads the library's bookkeeping, launches nothing. */
 int64_t dsrg_fno_debug_workspace_bytes(void);
 
+/* Device allocations of workspaces that this process has made so far, those of
+ * the batch workers among them.  Host only. */
+int64_t dsrg_fno_debug_workspace_allocations(void);
+
 #ifdef __cplusplus
 }
 #endif

@@ -40,6 +40,7 @@ EXPORTED = (
     "dsrg_fno_debug_regularizer",
     "dsrg_fno_debug_mma_schedule",
     "dsrg_fno_debug_workspace_bytes",
+    "dsrg_fno_debug_workspace_allocations",
     "dsrg_fno_debug_eig_batch",
     "dsrg_fno_debug_pair_tiles",
     "dsrg_fno_debug_set_barrier_limit",
@@ -150,6 +151,8 @@ def load(path: str = LIB_PATH):
     lib.dsrg_fno_debug_eig_batch.argtypes = [i32, ctypes.POINTER(i32), ctypes.POINTER(ctypes.POINTER(d)),
                                              ctypes.POINTER(ctypes.POINTER(d))]
     lib.dsrg_fno_debug_eig_batch.restype = ctypes.c_int
+    lib.dsrg_fno_debug_workspace_allocations.argtypes = []
+    lib.dsrg_fno_debug_workspace_allocations.restype = ctypes.c_int64
     lib.dsrg_fno_debug_workspace_bytes.argtypes = []
     lib.dsrg_fno_debug_workspace_bytes.restype = ctypes.c_int64
     lib.dsrg_fno_set_log_callback.argtypes = [LOG_FN, vp]

@@ -26,9 +26,13 @@ Workspace& workspace_for_current_device() {
   return g_ws[dev];
 }
 
+static std::atomic<int64_t> g_ws_allocs{0};
+int64_t ws_allocations() { return g_ws_allocs.load(); }
+
 int ws_reserve(Workspace& ws, size_t bytes) {
   ws.off = 0;
   if (bytes <= ws.cap) return DSRG_FNO_OK;
+  g_ws_allocs.fetch_add(1);
   if (ws.base) {
     DSRG_CUDA(cudaDeviceSynchronize());
     DSRG_CUDA(cudaFree(ws.base));

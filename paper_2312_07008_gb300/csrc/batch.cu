@@ -142,10 +142,12 @@ extern "C" int dsrg_fno_batch_run(dsrg_fno_batch_item* items, int32_t n, int32_t
   size_t have = 0;
   for (int k = 0; k < workers; ++k) have += pool.w[k].ws.cap;
   const size_t share = device_budget(have) / (size_t)workers;
-  // workspaces planned for fewer workers with larger shares go back first: beside
-  // them the shares of all workers need not fit
+  // workspaces that a larger share (fewer workers) let grow beyond the present one
+  // go back first: beside them the shares of all workers need not fit.  One that
+  // fits the present share stays, whatever it was planned with: calls with few and
+  // with many workers in turn would otherwise free and allocate on every call.
   for (Worker& w : pool.w) {
-    if (w.ws.base && w.planned > share + share / 2) {
+    if (w.planned > share + share / 2 && w.ws.cap > share + share / 2) {
       DSRG_CUDA(cudaStreamSynchronize(w.stream));
       DSRG_CUDA(cudaFree(w.ws.base));
       w.ws = Workspace{};

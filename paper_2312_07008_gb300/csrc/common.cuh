@@ -76,6 +76,7 @@ std::mutex& workspace_mutex();
 
 // Makes sure at least `bytes` are available; may synchronise the device.
 int ws_reserve(Workspace& ws, size_t bytes);
+int64_t ws_allocations();  // allocations of workspaces so far (all of the process)
 
 template <typename T>
 T* ws_take(Workspace& ws, size_t count) {

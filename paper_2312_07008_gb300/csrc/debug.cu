@@ -176,6 +176,8 @@ extern "C" int64_t dsrg_fno_debug_workspace_bytes(void) {
   return (int64_t)workspace_for_current_device().cap;
 }
 
+extern "C" int64_t dsrg_fno_debug_workspace_allocations(void) { return ws_allocations(); }
+
 extern "C" int dsrg_fno_debug_pair_tiles(int32_t nslices, int32_t ncore, int32_t nact, int32_t nvir,
                                          const int32_t* pairs, int32_t npairs, int32_t energy_only,
                                          int32_t* tiles, int32_t max_tiles) {
