@@ -24,7 +24,9 @@ __device__ __forceinline__ double zero_like(double) { return 0.0; }
 
 __device__ __forceinline__ long long integer_of(double v, int f) { return scaled_integer(v, f); }
 
-// Squared norms of the rows: part[split][row] over the split's share of k.
+__device__ __forceinline__ uint32_t high_word(double v) { return (uint32_t)__double2hiint(v) & 0x7fffffffu; }
+
+// Norms of the rows: part[split][row] (row_part) over the split's share of k.
 // Source element (row, k) at src[row rs + k ks]; one of rs, ks is 1.
 template <typename T>
 __global__ void __launch_bounds__(256) row_norm_kernel(const T* __restrict__ src, long R, int K, long rs, long ks,
@@ -33,27 +35,44 @@ __global__ void __launch_bounds__(256) row_norm_kernel(const T* __restrict__ src
   const int k0 = blockIdx.y * per, k1 = min(K, k0 + per);
   const long row0 = (long)blockIdx.x * 32;
   double s = 0.0;
+  uint32_t hi = 0;
   if (ks == 1) {  // 8 threads per row
     const long row = row0 + (threadIdx.x >> 3);
     if (row < R)
-      for (int k = k0 + (threadIdx.x & 7); k < k1; k += 8) s += square_of(src[row * rs + k]);
+      for (int k = k0 + (threadIdx.x & 7); k < k1; k += 8) {
+        const T v = src[row * rs + k];
+        s += square_of(v);
+        hi = max(hi, high_word(v));
+      }
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (row < R && (threadIdx.x & 7) == 0) part[blockIdx.y * R + row] = s;
+    for (int o = 4; o > 0; o >>= 1) {
+      s += __shfl_xor_sync(0xffffffffu, s, o);
+      hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    }
+    if (row < R && (threadIdx.x & 7) == 0) part[blockIdx.y * R + row] = row_part(s, hi);
     return;
   }
   // a lane per row, 8 warps over k
   __shared__ double red[8][32];
+  __shared__ uint32_t red_hi[8][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const long row = row0 + lane;
   if (row < R)
-    for (int k = k0 + w; k < k1; k += 8) s += square_of(src[row * rs + (long)k * ks]);
+    for (int k = k0 + w; k < k1; k += 8) {
+      const T v = src[row * rs + (long)k * ks];
+      s += square_of(v);
+      hi = max(hi, high_word(v));
+    }
   red[w][lane] = s;
+  red_hi[w][lane] = hi;
   __syncthreads();
   if (w == 0 && row < R) {
 #pragma unroll
-    for (int q = 1; q < 8; ++q) s += red[q][lane];
-    part[blockIdx.y * R + row] = s;
+    for (int q = 1; q < 8; ++q) {
+      s += red[q][lane];
+      hi = max(hi, red_hi[q][lane]);
+    }
+    part[blockIdx.y * R + row] = row_part(s, hi);
   }
 }
 
@@ -73,8 +92,8 @@ __global__ void __launch_bounds__(256) residue_rows_kernel(const T* __restrict__
   constexpr double LIMIT = norm_limit(NM);
   int f = 0;
   if (row < R) {
-    double s = 0.0;
-    for (int q = 0; q < nsplit; ++q) s += part[q * R + row];
+    RowNorm s{0.0, 0};
+    for (int q = 0; q < nsplit; ++q) add_part(s, part[q * R + row]);
     f = row_shift(s, K, LIMIT);
     if (seg == 0 && blockIdx.y == 0) exps[row] = -f;
     if (f == SHIFT_INVALID) f = 0;

@@ -183,6 +183,33 @@ __host__ __device__ __forceinline__ int row_shift(double sumsq, int K, double li
   return e - 1 < 1000 ? e - 1 : 1000;
 }
 
+// A row's norm from its parts.  A part is the sum of its elements' squares or, where the
+// largest element lies beyond 2^+-480 and its square near the ends of float64's range,
+// minus that element's biased exponent; hi: the largest high word of |v|.
+__host__ __device__ __forceinline__ double row_part(double sumsq, uint32_t hi) {
+  const int E = (int)(hi >> 20);
+  if (E == 0) return 0.0;  // elements below 2^-1022 are staged as zeros
+  return (E >= 543 && E <= 1503) || E == 2047 ? sumsq : -(double)E;
+}
+struct RowNorm {
+  double sumsq;
+  int e;  // largest exponent of the parts that are one, 0: none
+};
+__host__ __device__ __forceinline__ void add_part(RowNorm& r, double part) {
+  if (part < 0.0) r.e = r.e > (int)-part ? r.e : (int)-part;
+  else r.sumsq += part;
+}
+// As above; a part by exponent counts as K elements of 2^(e - 1022), above all of its
+// own: the row keeps half of log2 K bits less than by its norm, as many as by its
+// largest element.
+__host__ __device__ __forceinline__ int row_shift(const RowNorm& r, int K, double limit) {
+  if (r.e == 0 || !(r.sumsq <= 1.7e308)) return row_shift(r.sumsq, K, limit);
+  if (r.e < 1023 && r.sumsq > 0.0) return row_shift(r.sumsq + K * ldexp(1.0, 2 * (r.e - 1022)), K, limit);
+  int e;
+  frexp((limit - 0.5 * sqrt((double)K) - 1.0) / sqrt((double)K), &e);
+  return e - 1 - (r.e - 1022);
+}
+
 // The contraction: u = sum_i r_i C_i mod 2^64 as a signed fraction of M, i.e.
 // value = u 2^-63 (M / 2) 2^(e_a + e_b) for row exponents e = -f.
 template <int NM>
