@@ -63,7 +63,8 @@ struct Plan {
   std::vector<DressDesc> desc;
   std::vector<Batch> batches;
   int max_pairs = 0, max_desc = 0, max_out = 0;
-  int res_cap = 0;  // residue form: output tiles whose residues are held at a time
+  bool residue = false;  // B.B contraction in the residue form
+  int res_cap = 0;       // residue form: output tiles whose residues are held at a time
 };
 
 static void build_plan(int nc, int na, long cap_pairs, Plan& P) {
@@ -271,12 +272,11 @@ static int2 pair_form_of(const dsrg_fno_problem* p, int ks) {
 static size_t doubles(size_t n) { return ws_bytes(n, sizeof(double)); }
 
 // The B.B contraction of five planes runs in the residue form (10 products
-// instead of 15 and no dropped ones); 3 and 4 planes stay digit planes.
+// instead of 15 and no dropped ones) unless its ten planes do not fit the device
+// (make_plan); 3 and 4 planes stay digit planes.
 static bool residue_form(int ks, int2 pform) { return ks == 5 && pform.x == FORM_DIGITS; }
-static int pair_tile_rows(int ks, int2 pform) { return residue_form(ks, pform) ? RES_TILE : PAIR_TILE_M; }
-static int pair_tile_cols(int ks, int2 pform) {
-  return residue_form(ks, pform) ? RES_TILE : pair_tile_n(pform.x, pform.y);
-}
+static int pair_tile_rows(const Plan& P) { return P.residue ? RES_TILE : PAIR_TILE_M; }
+static int pair_tile_cols(const Plan& P, int2 pform) { return P.residue ? RES_TILE : pair_tile_n(pform.x, pform.y); }
 
 static long pair_cap_for_budget(int nv, int np, int ks, bool residue, size_t budget) {
   // tau + kappa + two dressed matrices per pair (+ the dressed planes and, outside the residue form, nu in the fast form)
@@ -301,33 +301,6 @@ size_t device_budget(size_t held) {
 }
 
 static size_t plan_budget(const Workspace& ws) { return device_budget(ws.cap); }
-
-// Batches of pairs that fit the budget.  The residues of 4096 output tiles (5.4
-// GB, 54 rounds of units on 76 pairs of SMs) lose nothing to the launches' last
-// rounds; a small budget holds an eighth of itself, at least 64 tiles.  What the
-// residue form holds beside the batches and five digit planes would not (ten
-// planes of B and of the small terms' operands, the update's residues) comes off
-// the budget, so that a pass's workspace is no larger than theirs: several batch
-// workers' passes stand beside each other and the inputs.
-static void make_plan(const Geometry& g, int ks, int2 pform, size_t budget, bool want_d, Plan& P) {
-  const bool rf = residue_form(ks, pform);
-  const size_t tile = residue_tile_bytes(RES_MOD);
-  if (rf) P.res_cap = (int)std::max<size_t>(64, std::min<size_t>(4096, budget / 8 / tile));
-  const size_t held = rf ? std::min(budget / 8, (size_t)P.res_cap * tile) : 0;
-  size_t avail = budget - held;
-  if (rf) {
-    size_t more = (size_t)(RES_MOD - 5) * 2 * g.nh * g.np * pad64(g.nq);
-    if (want_d)
-      more += residue_syrk_res_bytes(g.nv) + (size_t)(RES_MOD - 5) * 2 * 2 * g.nv * pad64(small_terms_kmax(g.nc, g.na));
-    avail = std::max(avail / 4, avail > more ? avail - more : 0);
-  }
-  build_plan(g.nc, g.na, pair_cap_for_budget(g.nv, g.np, ks, rf, avail), P);
-  if (rf) {
-    int most = 1;
-    for (const Batch& b : P.batches) most = std::max(most, pair_tile_bound(RES_TILE, RES_TILE, g, b.npairs));
-    P.res_cap = std::min(P.res_cap, most);
-  }
-}
 
 static int run_pass(const Geometry& g, const double* B, const double* eps, const double* gamma1,
                     const double* lambda2, const Plan& P, PassBuffers& W, bool want_d, double* D,
@@ -461,7 +434,7 @@ static int nsplit_for(int nv, int ndesc, int ks) {
   return best;
 }
 
-// Carves the pass buffers out of the workspace (sizes must match pass_bytes).
+// Bytes of the pass buffers that carve_pass takes.
 static size_t pass_bytes(const Geometry& g, const Plan& P, bool want_d, int nsplit, int ks, int2 pform) {
   const size_t nv2 = (size_t)g.nv * g.nv;
   const int na = g.na, ns = na * (na + 1) / 2, nd = na * (na - 1) / 2;
@@ -482,7 +455,7 @@ static size_t pass_bytes(const Geometry& g, const Plan& P, bool want_d, int nspl
   b += ws_bytes(16, sizeof(int));
   if (ks) {
     const size_t rows = (size_t)g.nh * g.np;
-    const bool rf = residue_form(ks, pform);
+    const bool rf = P.residue;
     b += ws_bytes((size_t)(rf ? RES_MOD : ks) * rows * pad64(g.nq), 2) +
          (rf ? residue_exps_bytes(rows) : ws_bytes(rows, sizeof(int)));
     b += rf ? ws_bytes(P.res_cap * residue_tile_bytes(RES_MOD), 1) : doubles((size_t)P.max_pairs * g.np * g.np);
@@ -499,13 +472,45 @@ static size_t pass_bytes(const Geometry& g, const Plan& P, bool want_d, int nspl
     }
     b += ws_bytes(8, sizeof(int));
     size_t tiles = 0;
-    const int bm = pair_tile_rows(ks, pform), bn = pair_tile_cols(ks, pform);
+    const int bm = pair_tile_rows(P), bn = pair_tile_cols(P, pform);
     for (const Batch& bt : P.batches) tiles += (size_t)pair_tile_bound(bm, bn, g, bt.npairs);
     b += ws_bytes(tiles + 1, sizeof(int2)) + ws_bytes(P.batches.size() * (size_t)g.nh * g.nh + 1, sizeof(int));
   }
   return b;
 }
 
+// Batches of pairs that fit the budget.  The residues of 4096 output tiles (5.4
+// GB, 54 rounds of units on 76 pairs of SMs) lose nothing to the launches' last
+// rounds; a small budget holds an eighth of itself, at least 64 tiles.  What the
+// residue form holds beside the batches and five digit planes would not (ten
+// planes of B and of the small terms' operands, the update's residues) comes off
+// the budget, so that a pass's workspace is no larger than theirs: several batch
+// workers' passes stand beside each other and the inputs.  Where B is so large that
+// its ten planes and what the call holds beside the pass do not fit 2 1/6 of the
+// budget (0.975 of the free memory), the pass takes five digit planes: slower (319
+// against 154 ms at nvir 1200), but not refused.
+static void make_plan(const Geometry& g, int ks, int2 pform, size_t budget, bool want_d, size_t beside, Plan& P) {
+  P.residue = residue_form(ks, pform);
+  if (P.residue) {
+    const size_t tile = residue_tile_bytes(RES_MOD);
+    P.res_cap = (int)std::max<size_t>(64, std::min<size_t>(4096, budget / 8 / tile));
+    const size_t avail = budget - std::min(budget / 8, (size_t)P.res_cap * tile);
+    size_t more = (size_t)(RES_MOD - 5) * 2 * g.nh * g.np * pad64(g.nq);
+    if (want_d)
+      more += residue_syrk_res_bytes(g.nv) + (size_t)(RES_MOD - 5) * 2 * 2 * g.nv * pad64(small_terms_kmax(g.nc, g.na));
+    build_plan(g.nc, g.na, pair_cap_for_budget(g.nv, g.np, ks, true, std::max(avail / 4, avail > more ? avail - more : 0)), P);
+    int most = 1;
+    for (const Batch& b : P.batches) most = std::max(most, pair_tile_bound(RES_TILE, RES_TILE, g, b.npairs));
+    P.res_cap = std::min(P.res_cap, most);
+    if (beside + pass_bytes(g, P, want_d, 1, ks, pform) <= 2 * budget + budget / 6) return;
+    P = Plan{};
+    const size_t held = want_d ? residue_syrk_res_bytes(g.nv) : 0;
+    budget = std::max(budget / 4, budget > held ? budget - held : 0);
+  }
+  build_plan(g.nc, g.na, pair_cap_for_budget(g.nv, g.np, ks, false, budget), P);
+}
+
+// Carves the pass buffers out of the workspace (sizes must match pass_bytes).
 static int carve_pass(Workspace& ws, const Geometry& g, const Plan& P, bool want_d, int nsplit, int ks, int2 pform,
                       PassBuffers& W, cudaStream_t st) {
   const size_t nv2 = (size_t)g.nv * g.nv;
@@ -541,7 +546,7 @@ static int carve_pass(Workspace& ws, const Geometry& g, const Plan& P, bool want
     const size_t rows = (size_t)g.nh * g.np;
     W.kpad_q = pad64(g.nq);
     W.kpad_v = pad64(g.nv);
-    W.residue = residue_form(ks, pform);
+    W.residue = P.residue;
     W.planes_b = ws_take<__nv_bfloat16>(ws, (size_t)(W.residue ? RES_MOD : ks) * rows * W.kpad_q);
     if (W.residue) {
       W.exps_b = reinterpret_cast<int*>(ws_take<char>(ws, residue_exps_bytes(rows)));
@@ -576,7 +581,7 @@ static int carve_pass(Workspace& ws, const Geometry& g, const Plan& P, bool want
     std::vector<int2> all, one;
     std::vector<int> slots(P.batches.size() * (size_t)g.nh * g.nh, -1);
     size_t bound = 0;
-    const int bm = pair_tile_rows(ks, pform), bn = pair_tile_cols(ks, pform);
+    const int bm = pair_tile_rows(P), bn = pair_tile_cols(P, pform);
     for (size_t bi = 0; bi < P.batches.size(); ++bi) {
       const Batch& b = P.batches[bi];
       bound += (size_t)pair_tile_bound(bm, bn, g, b.npairs);
@@ -627,11 +632,9 @@ static int read_error_flag(const int* err, cudaStream_t st) {
 }
 
 // Energy-only pass for an arbitrary geometry (used for the MO and FNO bases).
-static int energy_pass(const Geometry& g, int ks, int2 pform, const double* B, const double* eps, const double* gamma1,
-                       const double* lambda2, Workspace& ws, size_t base_off, size_t budget, double* e_out,
+static int energy_pass(const Geometry& g, const Plan& P, int ks, int2 pform, const double* B, const double* eps,
+                       const double* gamma1, const double* lambda2, Workspace& ws, size_t base_off, double* e_out,
                        cudaStream_t st) {
-  Plan P;
-  make_plan(g, ks, pform, budget, false, P);
   ws.off = base_off;
   PassBuffers W{};
   size_t need = base_off + pass_bytes(g, P, false, 1, ks, pform);
@@ -643,12 +646,6 @@ static int energy_pass(const Geometry& g, int ks, int2 pform, const double* B, c
   return read_error_flag(W.err, st);
 }
 
-static size_t energy_pass_bytes(const Geometry& g, int ks, int2 pform, size_t budget) {
-  Plan P;
-  make_plan(g, ks, pform, budget, false, P);
-  return pass_bytes(g, P, false, 1, ks, pform);
-}
-
 int impl_pt2_energy(Workspace& ws, size_t budget, const dsrg_fno_problem* prob, double* e2_out, cudaStream_t st) {
   int s = validate(prob);
   if (s) return s;
@@ -656,11 +653,13 @@ int impl_pt2_energy(Workspace& ws, size_t budget, const dsrg_fno_problem* prob, 
   const Geometry g = geometry_of(prob);
   const int ks = slices_of(prob);
   const int2 pform = pair_form_of(prob, ks);
-  DSRG_TRY(ws_reserve(ws, energy_pass_bytes(g, ks, pform, budget) + ws_bytes(8, sizeof(int))));
+  const size_t fixed = ws_bytes(8, sizeof(int));
+  Plan P;
+  make_plan(g, ks, pform, budget, false, fixed, P);
+  DSRG_TRY(ws_reserve(ws, fixed + pass_bytes(g, P, false, 1, ks, pform)));
   int* flag = ws_take<int>(ws, 8);
   DSRG_TRY(check_inputs_finite(prob, flag, st));
-  return energy_pass(g, ks, pform, prob->B_hp, prob->eps, prob->gamma1, prob->lambda2, ws, ws.off, budget, e2_out,
-                     st);
+  return energy_pass(g, P, ks, pform, prob->B_hp, prob->eps, prob->gamma1, prob->lambda2, ws, ws.off, e2_out, st);
 }
 
 int impl_pt2_energy_mr(Workspace& ws, size_t budget, const dsrg_fno_problem* prob, const double* l3, double* e2_out,
@@ -674,7 +673,10 @@ int impl_pt2_energy_mr(Workspace& ws, size_t budget, const dsrg_fno_problem* pro
   const int ks = slices_of(prob);
   const int2 pform = pair_form_of(prob, ks);
   const size_t mr = mr_energy_work_doubles(g, ks);
-  DSRG_TRY(ws_reserve(ws, ws_bytes(8, sizeof(int)) + std::max(energy_pass_bytes(g, ks, pform, budget), doubles(mr))));
+  const size_t fixed = ws_bytes(8, sizeof(int));
+  Plan P;
+  make_plan(g, ks, pform, budget, false, fixed, P);
+  DSRG_TRY(ws_reserve(ws, fixed + std::max(pass_bytes(g, P, false, 1, ks, pform), doubles(mr))));
   int* flag = ws_take<int>(ws, 8);
   DSRG_TRY(check_inputs_finite(prob, flag, st));
   if (l3) {
@@ -687,7 +689,7 @@ int impl_pt2_energy_mr(Workspace& ws, size_t budget, const dsrg_fno_problem* pro
   }
   const size_t base = ws.off;
   double evv = 0.0;
-  DSRG_TRY(energy_pass(g, ks, pform, prob->B_hp, prob->eps, prob->gamma1, prob->lambda2, ws, base, budget, &evv, st));
+  DSRG_TRY(energy_pass(g, P, ks, pform, prob->B_hp, prob->eps, prob->gamma1, prob->lambda2, ws, base, &evv, st));
   ws.off = base;
   double* work = ws_take<double>(ws, mr);
   if (!work) return DSRG_FNO_ERR_NOMEM;
@@ -709,9 +711,6 @@ int impl_vv_opdm(Workspace& ws, size_t budget, const dsrg_fno_problem* prob, dou
   const Geometry g = geometry_of(prob);
   const int ks = slices_of(prob);
   const int2 pform = pair_form_of(prob, ks);
-  Plan P;
-  make_plan(g, ks, pform, budget, true, P);
-  const int nsplit = nsplit_for(g.nv, P.max_out, ks ? syrk_slices(ks) : 0);
   const size_t small = small_terms_work_doubles(g.nc, g.na, g.nv);
   const int kmax = small_terms_kmax(g.nc, g.na);
   const bool small_fast = ks > 0 && kmax >= SLICED_MIN_K;
@@ -721,9 +720,11 @@ int impl_vv_opdm(Workspace& ws, size_t budget, const dsrg_fno_problem* prob, dou
   const size_t small_out =
       small_res ? ws_bytes(residue_plain_bytes(RES_MOD, g.nv, g.nv), 1) : doubles((size_t)g.nv * g.nv);
   const size_t small_fast_bytes = small_fast ? ws_bytes(small_planes, 2) + 2 * small_exps + small_out : 0;
-  size_t need = ws_bytes(8, sizeof(int)) + pass_bytes(g, P, true, nsplit, ks, pform) + doubles((size_t)g.nh * g.nv) +
-                doubles(small + 1) + small_fast_bytes;
-  DSRG_TRY(ws_reserve(ws, need));
+  const size_t fixed = ws_bytes(8, sizeof(int)) + doubles((size_t)g.nh * g.nv) + doubles(small + 1) + small_fast_bytes;
+  Plan P;
+  make_plan(g, ks, pform, budget, true, fixed, P);
+  const int nsplit = nsplit_for(g.nv, P.max_out, ks ? syrk_slices(ks) : 0);
+  DSRG_TRY(ws_reserve(ws, fixed + pass_bytes(g, P, true, nsplit, ks, pform)));
   int* flag = ws_take<int>(ws, 8);
   DSRG_TRY(check_inputs_finite(prob, flag, st));
   if (l3) {
@@ -818,8 +819,6 @@ int impl_correction(Workspace& ws, size_t budget, const dsrg_fno_problem* prob, 
                  doubles(nk + 1);
   const int ks = slices_of(prob);
   const int2 pform = pair_form_of(prob, ks);
-  size_t pass_mo = e2_mo_in ? 0 : energy_pass_bytes(g, ks, pform, budget);
-  size_t pass_f = nk > 0 ? energy_pass_bytes(gf, ks, pform, budget) : 0;
   const int kpv = pad64(nv);
   // B' = B U enters E_vv(FNO) element by element and Delta E is a difference
   // of two large energies: the rotation takes 12 moduli (rows of norm 2^53) in
@@ -832,6 +831,16 @@ int impl_correction(Workspace& ws, size_t budget, const dsrg_fno_problem* prob, 
   // full-energy form: the rest terms of both bases (their work overlaps the passes) and f_hp rotated
   const size_t mr_work = mr ? doubles(mr_energy_work_doubles(g, ks)) : 0;
   const size_t ff_bytes = mr ? doubles((size_t)g.nh * gf.np + 1) : 0;
+  Plan plan_mo, plan_f;
+  size_t pass_mo = 0, pass_f = 0;
+  if (!e2_mo_in) {
+    make_plan(g, ks, pform, budget, false, fixed + ff_bytes, plan_mo);
+    pass_mo = pass_bytes(g, plan_mo, false, 1, ks, pform);
+  }
+  if (nk > 0) {
+    make_plan(gf, ks, pform, budget, false, fixed + ff_bytes, plan_f);
+    pass_f = pass_bytes(gf, plan_f, false, 1, ks, pform);
+  }
   DSRG_TRY(ws_reserve(ws, fixed + ff_bytes + std::max(std::max(pass_mo, pass_f), std::max(xform, mr_work))));
   int* flag = ws_take<int>(ws, 8);
   DSRG_TRY(check_inputs_finite(prob, flag, st));
@@ -858,8 +867,7 @@ int impl_correction(Workspace& ws, size_t budget, const dsrg_fno_problem* prob, 
   double e_mo = 0.0;
   if (e2_mo_in) e_mo = *e2_mo_in;
   else {
-    DSRG_TRY(energy_pass(g, ks, pform, prob->B_hp, prob->eps, prob->gamma1, prob->lambda2, ws, base, budget, &e_mo,
-                         st));
+    DSRG_TRY(energy_pass(g, plan_mo, ks, pform, prob->B_hp, prob->eps, prob->gamma1, prob->lambda2, ws, base, &e_mo, st));
     if (mr) {
       ws.off = base;
       double* work = ws_take<double>(ws, mr_energy_work_doubles(g, ks));
@@ -909,7 +917,7 @@ int impl_correction(Workspace& ws, size_t budget, const dsrg_fno_problem* prob, 
     DSRG_CUDA(cudaMemcpyAsync(epsf + g.nh, evals, sizeof(double) * nk, cudaMemcpyDeviceToDevice, st));
     if (eps_fno_out)
       DSRG_CUDA(cudaMemcpyAsync(eps_fno_out, evals, sizeof(double) * nk, cudaMemcpyDeviceToDevice, st));
-    DSRG_TRY(energy_pass(gf, ks, pform, Bf, epsf, prob->gamma1, prob->lambda2, ws, base, budget, &e_f, st));
+    DSRG_TRY(energy_pass(gf, plan_f, ks, pform, Bf, epsf, prob->gamma1, prob->lambda2, ws, base, &e_f, st));
   }
   if (mr) {
     // E^(2)(FNO) beyond its vv part: the active particles stay, the kept

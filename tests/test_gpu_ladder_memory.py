@@ -29,11 +29,14 @@ def run(nv, naux, npairs, megabytes=None):
     t = 0.05 * torch.randn((npairs, nv, nv), dtype=torch.float64, device="cuda", generator=gen)
     c = torch.full_like(t, float("nan"))
     hold = leave_free(megabytes) if megabytes else None
-    pkg.dsrg_fno_ladder(b, t, c)
-    torch.cuda.synchronize()
-    held = pkg.dsrg_fno_debug_workspace_bytes()
-    del hold
-    pkg.dsrg_fno_release()
+    try:
+        pkg.dsrg_fno_ladder(b, t, c)
+        torch.cuda.synchronize()
+    finally:
+        held = pkg.dsrg_fno_debug_workspace_bytes()
+        del hold
+        torch.cuda.empty_cache()
+        pkg.dsrg_fno_release()
     return c.cpu(), held
 
 
