@@ -406,11 +406,13 @@ static int run_pass(const Geometry& g, const double* B, const double* eps, const
 
 // Split of the dressed rank-K update over the dressed matrices: enough
 // upper-triangle tile jobs for two waves of the SMs, and a count that fills
-// its last wave (jobs = tiles x splits, the persistent grid has one CTA per SM).
+// its last wave (jobs = tiles x splits, the persistent grid has one CTA per SM).  ks:
+// planes of the update; with 5 it is in the residue form and has no partial sums.
 static int nsplit_for(int nv, int ndesc, int ks) {
+  if (ks == 5) return 0;
   int tiles;
-  if (ks) {  // 128 x BN tiles of the digit-plane kernel with some f >= e
-    const int bm = 128, bn = ks == 5 ? 48 : 64;
+  if (ks) {  // 128 x 64 tiles of the digit-plane kernel with some f >= e
+    const int bm = 128, bn = 64;
     const int ntm = ceil_div(nv, bm), ntn = ceil_div(nv, bn);
     tiles = 0;
     for (int m = 0; m < ntm; ++m) tiles += ntn - (m * bm) / bn;
@@ -723,7 +725,7 @@ int impl_vv_opdm(Workspace& ws, size_t budget, const dsrg_fno_problem* prob, dou
   const size_t fixed = ws_bytes(8, sizeof(int)) + doubles((size_t)g.nh * g.nv) + doubles(small + 1) + small_fast_bytes;
   Plan P;
   make_plan(g, ks, pform, budget, true, fixed, P);
-  const int nsplit = nsplit_for(g.nv, P.max_out, ks ? syrk_slices(ks) : 0);
+  const int nsplit = nsplit_for(g.nv, P.max_out, ks ? syrk_slices(ks) : 0);  // 0: the residue form splits by itself
   DSRG_TRY(ws_reserve(ws, fixed + pass_bytes(g, P, true, nsplit, ks, pform)));
   int* flag = ws_take<int>(ws, 8);
   DSRG_TRY(check_inputs_finite(prob, flag, st));
