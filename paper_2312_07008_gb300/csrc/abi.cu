@@ -674,7 +674,7 @@ int impl_pt2_energy_mr(Workspace& ws, size_t budget, const dsrg_fno_problem* pro
   const Geometry g = geometry_of(prob);
   const int ks = slices_of(prob);
   const int2 pform = pair_form_of(prob, ks);
-  const size_t mr = mr_energy_work_doubles(g, ks);
+  const size_t mr = mr_energy_work_doubles(g, ks, budget);
   const size_t fixed = ws_bytes(8, sizeof(int));
   Plan P;
   make_plan(g, ks, pform, budget, false, fixed, P);
@@ -696,7 +696,7 @@ int impl_pt2_energy_mr(Workspace& ws, size_t budget, const dsrg_fno_problem* pro
   double* work = ws_take<double>(ws, mr);
   if (!work) return DSRG_FNO_ERR_NOMEM;
   double rest = 0.0;
-  DSRG_TRY(mr_energy_rest(g, ks, prob->B_hp, prob->eps, prob->f_hp, prob->gamma1, prob->lambda2, l3, work, &rest, st));
+  DSRG_TRY(mr_energy_rest(g, ks, budget, prob->B_hp, prob->eps, prob->f_hp, prob->gamma1, prob->lambda2, l3, work, &rest, st));
   if (!isfinite(evv) || !isfinite(rest)) return DSRG_FNO_ERR_NONFINITE;
   *e2_out = evv + rest;
   if (evv_out) *evv_out = evv;
@@ -827,11 +827,16 @@ int impl_correction(Workspace& ws, size_t budget, const dsrg_fno_problem* prob, 
   // the fast form, the passes themselves keep ks.
   const int kx = ks ? RES_MOD_X : 0;
   size_t xform = 0;
-  if (kx && nk > 0)
-    xform = ws_bytes((size_t)kx * rows * kpv, 2) + residue_exps_bytes(rows) + ws_bytes((size_t)kx * nk * kpv, 2) +
-            residue_exps_bytes(nk) + ws_bytes(residue_plain_bytes(kx, rows, nk), 1) + ws_bytes(8, sizeof(int));
+  long xrows = rows;
+  int xcap = RES_PLAIN_CAP;
+  if (kx && nk > 0) {
+    xrows = residue_rows_at_a_time(kx, rows, kpv, budget);
+    xcap = residue_cap(kx, budget);
+    xform = ws_bytes((size_t)kx * xrows * kpv, 2) + residue_exps_bytes(xrows) + ws_bytes((size_t)kx * nk * kpv, 2) +
+            residue_exps_bytes(nk) + ws_bytes(residue_plain_bytes(kx, xrows, nk, xcap), 1) + ws_bytes(8, sizeof(int));
+  }
   // full-energy form: the rest terms of both bases (their work overlaps the passes) and f_hp rotated
-  const size_t mr_work = mr ? doubles(mr_energy_work_doubles(g, ks)) : 0;
+  const size_t mr_work = mr ? doubles(mr_energy_work_doubles(g, ks, budget)) : 0;
   const size_t ff_bytes = mr ? doubles((size_t)g.nh * gf.np + 1) : 0;
   Plan plan_mo, plan_f;
   size_t pass_mo = 0, pass_f = 0;
@@ -872,10 +877,10 @@ int impl_correction(Workspace& ws, size_t budget, const dsrg_fno_problem* prob, 
     DSRG_TRY(energy_pass(g, plan_mo, ks, pform, prob->B_hp, prob->eps, prob->gamma1, prob->lambda2, ws, base, &e_mo, st));
     if (mr) {
       ws.off = base;
-      double* work = ws_take<double>(ws, mr_energy_work_doubles(g, ks));
+      double* work = ws_take<double>(ws, mr_energy_work_doubles(g, ks, budget));
       double rest = 0.0;
       if (!work) return DSRG_FNO_ERR_NOMEM;
-      DSRG_TRY(mr_energy_rest(g, ks, prob->B_hp, prob->eps, prob->f_hp, prob->gamma1, prob->lambda2, mr->l3, work, &rest,
+      DSRG_TRY(mr_energy_rest(g, ks, budget, prob->B_hp, prob->eps, prob->f_hp, prob->gamma1, prob->lambda2, mr->l3, work, &rest,
                               st));
       e_mo += rest;
     }
@@ -896,19 +901,22 @@ int impl_correction(Workspace& ws, size_t budget, const dsrg_fno_problem* prob, 
     DSRG_TRY(copy_active(rows, g.na, g.np, gf.np, prob->B_hp, Bf, st));
     if (ks) {
       ws.off = base;
-      __nv_bfloat16* pa = ws_take<__nv_bfloat16>(ws, (size_t)kx * rows * kpv);
-      int* ea = reinterpret_cast<int*>(ws_take<char>(ws, residue_exps_bytes(rows)));
+      __nv_bfloat16* pa = ws_take<__nv_bfloat16>(ws, (size_t)kx * xrows * kpv);
+      int* ea = reinterpret_cast<int*>(ws_take<char>(ws, residue_exps_bytes(xrows)));
       __nv_bfloat16* pb = ws_take<__nv_bfloat16>(ws, (size_t)kx * nk * kpv);
       int* eb = reinterpret_cast<int*>(ws_take<char>(ws, residue_exps_bytes(nk)));
-      uint16_t* res = reinterpret_cast<uint16_t*>(ws_take<char>(ws, residue_plain_bytes(kx, rows, nk)));
+      uint16_t* res = reinterpret_cast<uint16_t*>(ws_take<char>(ws, residue_plain_bytes(kx, xrows, nk, xcap)));
       int* err = ws_take<int>(ws, 8);
       if (!err) return DSRG_FNO_ERR_NOMEM;
       DSRG_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
       // rows (Q, h) over the virtual index e, and U^T rows l over e
-      DSRG_TRY(residue_stage(kx, prob->B_hp + g.na, rows, nv, g.np, 1, kpv, pa, ea, st));
       DSRG_TRY(residue_stage(kx, U, nk, nv, 1, nk, kpv, pb, eb, st));
-      DSRG_TRY(residue_plain(kx, (int)rows, nk, pa, ea, rows, 0, pb, eb, kpv, 1.0, false, Bf + g.na, gf.np, 0, res,
-                             RES_PLAIN_CAP, err, st));
+      for (long r0 = 0; r0 < rows; r0 += xrows) {
+        const long n = std::min(xrows, rows - r0);
+        DSRG_TRY(residue_stage(kx, prob->B_hp + r0 * g.np + g.na, n, nv, g.np, 1, kpv, pa, ea, st));
+        DSRG_TRY(residue_plain(kx, (int)n, nk, pa, ea, n, 0, pb, eb, kpv, 1.0, false, Bf + r0 * gf.np + g.na, gf.np, 0, res,
+                               xcap, err, st));
+      }
       DSRG_TRY(read_error_flag(err, st));
     } else {
       DSRG_TRY(gemm_f64((int)rows, nk, nv, 1.0, prob->B_hp + g.na, g.np, true, U, nk, false, 0.0, Bf + g.na, gf.np,
@@ -938,10 +946,10 @@ int impl_correction(Workspace& ws, size_t budget, const dsrg_fno_problem* prob, 
       f_fno = ff;
     }
     ws.off = base;
-    double* work = ws_take<double>(ws, mr_energy_work_doubles(gf, ks));
+    double* work = ws_take<double>(ws, mr_energy_work_doubles(gf, ks, budget));
     double rest = 0.0;
     if (!work) return DSRG_FNO_ERR_NOMEM;
-    DSRG_TRY(mr_energy_rest(gf, ks, Bf, epsf, f_fno, prob->gamma1, prob->lambda2, mr->l3, work, &rest, st));
+    DSRG_TRY(mr_energy_rest(gf, ks, budget, Bf, epsf, f_fno, prob->gamma1, prob->lambda2, mr->l3, work, &rest, st));
     e_f += rest;
   }
   if (!isfinite(e_mo) || !isfinite(e_f)) return DSRG_FNO_ERR_NONFINITE;

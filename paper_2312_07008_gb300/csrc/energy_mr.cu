@@ -98,21 +98,28 @@ static size_t mr_dbl(size_t bytes) { return (bytes + 255) / 256 * 32; }
 
 static bool mr_tensor_gemm(const Geometry& g, int ks) { return ks > 0 && g.na > 0 && g.nq >= SLICED_MIN_K; }
 
-size_t mr_energy_work_doubles(const Geometry& g, int ks) {
+// rows (i, a) of the integrals' left operand staged at a time
+static long mr_rows_at_a_time(const Geometry& g, int ks, size_t budget) {
+  const long M = (long)g.nh * g.np;
+  return ks == 5 ? residue_rows_at_a_time(RES_MOD, M, pad64(g.nq), budget) : M;
+}
+
+size_t mr_energy_work_doubles(const Geometry& g, int ks, size_t budget) {
   const MRSizes z = mr_sizes(g);
   // nu (reused for tpp), tp, xp, z1; z2, z3; g2t, w3; t1, x1, tt1; gt1; BA; 2 x partials
   size_t n = 4 * mr_dbl(8 * (size_t)z.n4) + 2 * mr_dbl(8 * (size_t)z.n4a) + mr_dbl(8 * (size_t)z.ng2t) +
              mr_dbl(8 * (size_t)z.nw3) + 3 * mr_dbl(8 * (size_t)z.n1) + mr_dbl(8 * (size_t)z.ngt1) +
              mr_dbl(8 * (size_t)z.nba) + mr_dbl(8 * (2 * (size_t)MR_EBLOCKS + 16));
   if (mr_tensor_gemm(g, ks)) {
-    const size_t kp = pad64(g.nq), ra = (size_t)g.nh * g.np, rb = (size_t)g.nh * g.na, k = ks == 5 ? RES_MOD : ks;
-    n += mr_dbl(2 * k * ra * kp) + mr_dbl(2 * k * rb * kp) + mr_dbl(residue_exps_bytes(ra)) +
-         mr_dbl(residue_exps_bytes(rb)) + mr_dbl(32) + (ks == 5 ? mr_dbl(residue_plain_bytes(RES_MOD, ra, rb)) : 0);
+    const size_t kp = pad64(g.nq), rb = (size_t)g.nh * g.na, k = ks == 5 ? RES_MOD : ks;
+    const size_t ra = mr_rows_at_a_time(g, ks, budget);
+    n += mr_dbl(2 * k * ra * kp) + mr_dbl(2 * k * rb * kp) + mr_dbl(residue_exps_bytes(ra)) + mr_dbl(residue_exps_bytes(rb)) +
+         mr_dbl(32) + (ks == 5 ? mr_dbl(residue_plain_bytes(RES_MOD, ra, rb, residue_cap(RES_MOD, budget))) : 0);
   }
   return n;
 }
 
-int mr_energy_rest(const Geometry& g, int ks, const double* B, const double* eps, const double* f_hp,
+int mr_energy_rest(const Geometry& g, int ks, size_t budget, const double* B, const double* eps, const double* f_hp,
                    const double* g1, const double* l2, const double* l3, double* work, double* e_out,
                    cudaStream_t st) {
   *e_out = 0.0;
@@ -160,21 +167,26 @@ int mr_energy_rest(const Geometry& g, int ks, const double* B, const double* eps
     DSRG_LAUNCH_CHECK();
     const int M = g.nh * g.np, N = g.nh * g.na;
     if (mr_tensor_gemm(g, ks)) {
-      // rows (i, a) of B and (j, y) of BA, contraction over Q: exact digit planes
+      // rows (i, a) of B and (j, y) of BA, contraction over Q: exact residues (5 planes) or digit planes
       const int kp = pad64(g.nq);
+      const long ra = mr_rows_at_a_time(g, ks, budget);
       const size_t k = ks == 5 ? RES_MOD : ks;
-      __nv_bfloat16* pa = reinterpret_cast<__nv_bfloat16*>(take(2 * k * M * kp));
+      __nv_bfloat16* pa = reinterpret_cast<__nv_bfloat16*>(take(2 * k * ra * kp));
       __nv_bfloat16* pb = reinterpret_cast<__nv_bfloat16*>(take(2 * k * N * kp));
-      int* ea = reinterpret_cast<int*>(take(residue_exps_bytes(M)));
+      int* ea = reinterpret_cast<int*>(take(residue_exps_bytes(ra)));
       int* eb = reinterpret_cast<int*>(take(residue_exps_bytes(N)));
       int* err = reinterpret_cast<int*>(take(32));
       DSRG_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
       if (ks == 5) {
-        uint16_t* res = reinterpret_cast<uint16_t*>(take(residue_plain_bytes(RES_MOD, M, N)));
-        DSRG_TRY(residue_stage(RES_MOD, B, M, g.nq, 1, M, kp, pa, ea, st));
+        const int cap = residue_cap(RES_MOD, budget);
+        uint16_t* res = reinterpret_cast<uint16_t*>(take(residue_plain_bytes(RES_MOD, ra, N, cap)));
         DSRG_TRY(residue_stage(RES_MOD, BA, N, g.nq, 1, N, kp, pb, eb, st));
-        DSRG_TRY(residue_plain(RES_MOD, M, N, pa, ea, M, 0, pb, eb, kp, 1.0, false, nu, N, 0, res, RES_PLAIN_CAP, err,
-                               st));
+        for (long r0 = 0; r0 < M; r0 += ra) {
+          const long n = std::min(ra, M - r0);
+          DSRG_TRY(residue_stage(RES_MOD, B + r0, n, g.nq, 1, M, kp, pa, ea, st));
+          DSRG_TRY(residue_plain(RES_MOD, (int)n, N, pa, ea, n, 0, pb, eb, kp, 1.0, false, nu + r0 * N, N, 0, res, cap, err,
+                                 st));
+        }
       } else {
         DSRG_TRY(slice_rows(ks, B, M, g.nq, 1, M, kp, pa, ea, st));
         DSRG_TRY(slice_rows(ks, BA, N, g.nq, 1, N, kp, pb, eb, st));

@@ -2,6 +2,8 @@
 #pragma once
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace dsrg {
@@ -182,7 +184,18 @@ int residue_pair(const Geometry& g, const __nv_bfloat16* planes, const int* exps
                  const int* slot_of, const float2* hp, uint16_t* res, int cap, float2* tau, float2* kap, double* ts,
                  int* err, cudaStream_t st);
 constexpr int RES_PLAIN_CAP = 1024;  // output tiles of a product whose residues are held at a time
-size_t residue_plain_bytes(int nm, long M, long N);  // residues of an M x N product (at most RES_PLAIN_CAP tiles)
+size_t residue_plain_bytes(int nm, long M, long N, int cap = RES_PLAIN_CAP);  // residues of an M x N product (at most cap tiles)
+// A long operand goes through a product in parts where the budget of a call is small:
+// its planes take at most half of that (the other operand is staged once) and the
+// residues an eighth.  Rows in parts of whole tiles, at least one.
+inline long residue_rows_at_a_time(int nm, long rows, int Kpad, size_t budget) {
+  const long fit = (long)(budget / 2 / ((size_t)nm * 2 * Kpad)) / RES_TILE * RES_TILE;
+  return fit >= rows ? rows : (fit > RES_TILE ? fit : std::min<long>(rows, RES_TILE));
+}
+inline int residue_cap(int nm, size_t budget) {
+  const size_t fit = budget / 8 / residue_tile_bytes(nm);
+  return fit >= (size_t)RES_PLAIN_CAP ? RES_PLAIN_CAP : (fit > 8 ? (int)fit : 8);  // 8: a unit for every pair of SMs
+}
 int residue_plain(int nm, int M, int N, const __nv_bfloat16* pa, const int* ea, long rows_a, int a0,
                   const __nv_bfloat16* pb, const int* eb, int Kpad, double alpha, bool add, double* C, long ldc, int swap,
                   uint16_t* res, int cap, int* err, cudaStream_t st);
@@ -233,8 +246,8 @@ bool is_device_ptr(const void* p);
 
 // Full multi-reference PT2 energy beyond E_vv, float64 (energy_mr.cu).
 // ks > 0: the integral GEMM on the digit-plane tensor-core path with ks planes (naux >= SLICED_MIN_K).
-size_t mr_energy_work_doubles(const Geometry& g, int ks);
-int mr_energy_rest(const Geometry& g, int ks, const double* B, const double* eps, const double* f_hp,
+size_t mr_energy_work_doubles(const Geometry& g, int ks, size_t budget);
+int mr_energy_rest(const Geometry& g, int ks, size_t budget, const double* B, const double* eps, const double* f_hp,
                    const double* g1, const double* l2, const double* l3, double* work, double* e_out,
                    cudaStream_t st);
 

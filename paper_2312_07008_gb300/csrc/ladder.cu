@@ -66,7 +66,7 @@ static LadderPlan ladder_plan(const Workspace& ws, int nv, int naux, int npairs)
   if (ladder_bytes(nv, naux, P) <= ws.cap) return P;
   const size_t budget = device_budget(ws.cap);
   if (ladder_bytes(nv, naux, P) <= budget) return P;
-  P.cap = (int)std::max<size_t>(64, std::min<size_t>(RES_PLAIN_CAP, budget / 8 / residue_tile_bytes(RES_MOD)));
+  P.cap = residue_cap(RES_MOD, budget);
   while (P.A > least && ladder_bytes(nv, naux, P) > budget) --P.A;
   while (P.A > 1 && ladder_bytes(nv, naux, P) > 2 * budget) --P.A;
   while (P.pairs > RES_TILE && ladder_bytes(nv, naux, P) > 2 * budget) P.pairs = std::max(RES_TILE, P.pairs / 2);

@@ -27,20 +27,30 @@ int impl_naf(Workspace& ws, int32_t nh, int32_t np, int32_t naux, const double* 
   const size_t n2 = (size_t)naux * naux;
   const bool fast = precision == DSRG_FNO_SLICED_BF16;
   const int kw = RES_MOD, kb = RES_MOD_X;
-  const int lpad = pad64((int)L), qpad = pad64(naux);
-  size_t planes = 0;
-  if (fast) {
-    // the metric's planes, then (reusing the space) the rotation's
-    const size_t p1 = ws_bytes((size_t)kw * naux * lpad, 2) + residue_exps_bytes(naux) + ws_bytes(16, sizeof(int)) +
-                      ws_bytes(residue_plain_bytes(kw, naux, naux), 1);
-    const size_t p2 = ws_bytes((size_t)kb * L * qpad, 2) + ws_bytes((size_t)kb * naux * qpad, 2) + residue_exps_bytes(L) +
-                      residue_exps_bytes(naux) + ws_bytes(16, sizeof(int)) + ws_bytes(residue_plain_bytes(kb, naux, L), 1);
-    planes = std::max(p1, p2);
+  const int qpad = pad64(naux);
+  const size_t fixed = 3 * ws_bytes(n2, sizeof(double)) + ws_bytes(eig_work_doubles(naux), sizeof(double)) +
+                       ws_bytes(naux + 16, sizeof(double)) + ws_bytes(naux + 16, sizeof(int)) + ws_bytes(8, sizeof(int));
+  // Fast form: pairs ia that pass through the metric (its contraction index) and the
+  // rotation (rows) at a time, all of them unless the memory that calls plan with is
+  // too small; the planes of the one, then (reusing the space) of the other.
+  long lw = L, lb = L;
+  int capw = RES_PLAIN_CAP, capb = RES_PLAIN_CAP;
+  auto planes = [&] {
+    const size_t p1 = ws_bytes((size_t)kw * naux * pad64((int)lw), 2) + residue_exps_bytes(naux) + ws_bytes(16, sizeof(int)) +
+                      ws_bytes(residue_plain_bytes(kw, naux, naux, capw), 1);
+    const size_t p2 = ws_bytes((size_t)kb * lb * qpad, 2) + ws_bytes((size_t)kb * naux * qpad, 2) + residue_exps_bytes(lb) +
+                      residue_exps_bytes(naux) + ws_bytes(16, sizeof(int)) + ws_bytes(residue_plain_bytes(kb, naux, lb, capb), 1);
+    return std::max(p1, p2);
+  };
+  if (fast && fixed + planes() > ws.cap) {
+    const size_t budget = device_budget(ws.cap);
+    lw = residue_rows_at_a_time(kw, L, qpad, budget);
+    lb = residue_rows_at_a_time(kb, L, qpad, budget);
+    capw = residue_cap(kw, budget);
+    capb = residue_cap(kb, budget);
   }
-  const size_t need = 3 * ws_bytes(n2, sizeof(double)) + ws_bytes(eig_work_doubles(naux), sizeof(double)) +
-                      ws_bytes(naux + 16, sizeof(double)) + ws_bytes(naux + 16, sizeof(int)) + planes +
-                      ws_bytes(8, sizeof(int));
-  DSRG_TRY(ws_reserve(ws, need));
+  const int lpad = pad64((int)lw);
+  DSRG_TRY(ws_reserve(ws, fixed + (fast ? planes() : 0)));
   {
     int* flag = ws_take<int>(ws, 8);
     int h = 0;
@@ -67,13 +77,15 @@ int impl_naf(Workspace& ws, int32_t nh, int32_t np, int32_t naux, const double* 
       ws.off = base;
       __nv_bfloat16* pl = ws_take<__nv_bfloat16>(ws, (size_t)kw * naux * lpad);
       int* ex = reinterpret_cast<int*>(ws_take<char>(ws, residue_exps_bytes(naux)));
-      uint16_t* res = reinterpret_cast<uint16_t*>(ws_take<char>(ws, residue_plain_bytes(kw, naux, naux)));
+      uint16_t* res = reinterpret_cast<uint16_t*>(ws_take<char>(ws, residue_plain_bytes(kw, naux, naux, capw)));
       int* err = ws_take<int>(ws, 16);
       if (!err) return DSRG_FNO_ERR_NOMEM;
       DSRG_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
-      DSRG_TRY(residue_stage(kw, B, naux, (int)L, L, 1, lpad, pl, ex, st));
-      DSRG_TRY(residue_plain(kw, naux, naux, pl, ex, naux, 0, pl, ex, lpad, 1.0, false, W, naux, 0, res, RES_PLAIN_CAP,
-                             err, st));
+      for (long l0 = 0; l0 < L; l0 += lw) {
+        const int n = (int)std::min(lw, L - l0), kp = pad64(n);
+        DSRG_TRY(residue_stage(kw, B + l0, naux, n, L, 1, kp, pl, ex, st));
+        DSRG_TRY(residue_plain(kw, naux, naux, pl, ex, naux, 0, pl, ex, kp, 1.0, l0 > 0, W, naux, 0, res, capw, err, st));
+      }
       int h = 0;
       DSRG_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, st));
       DSRG_CUDA(cudaStreamSynchronize(st));
@@ -100,19 +112,21 @@ int impl_naf(Workspace& ws, int32_t nh, int32_t np, int32_t naux, const double* 
     DSRG_PHASE("phase_naf_rotate", st);
     if (fast) {
       ws.off = base;
-      __nv_bfloat16* pb = ws_take<__nv_bfloat16>(ws, (size_t)kb * L * qpad);
+      __nv_bfloat16* pb = ws_take<__nv_bfloat16>(ws, (size_t)kb * lb * qpad);
       __nv_bfloat16* pu = ws_take<__nv_bfloat16>(ws, (size_t)kb * naux * qpad);
-      int* eb = reinterpret_cast<int*>(ws_take<char>(ws, residue_exps_bytes(L)));
+      int* eb = reinterpret_cast<int*>(ws_take<char>(ws, residue_exps_bytes(lb)));
       int* eu = reinterpret_cast<int*>(ws_take<char>(ws, residue_exps_bytes(naux)));
-      uint16_t* res = reinterpret_cast<uint16_t*>(ws_take<char>(ws, residue_plain_bytes(kb, naux, L)));
+      uint16_t* res = reinterpret_cast<uint16_t*>(ws_take<char>(ws, residue_plain_bytes(kb, naux, lb, capb)));
       int* err = ws_take<int>(ws, 16);
       if (!err) return DSRG_FNO_ERR_NOMEM;
       DSRG_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
       // rows of U^T (eigenvector K over Q: stride naux) and of B2^T (column ia over Q: stride L)
       DSRG_TRY(residue_stage(kb, U, k, naux, 1, naux, qpad, pu, eu, st));
-      DSRG_TRY(residue_stage(kb, B, L, naux, 1, L, qpad, pb, eb, st));
-      DSRG_TRY(residue_plain(kb, k, (int)L, pu, eu, k, 0, pb, eb, qpad, 1.0, false, B_out, L, 0, res, RES_PLAIN_CAP, err,
-                             st));
+      for (long l0 = 0; l0 < L; l0 += lb) {
+        const int n = (int)std::min(lb, L - l0);
+        DSRG_TRY(residue_stage(kb, B + l0, n, naux, 1, L, qpad, pb, eb, st));
+        DSRG_TRY(residue_plain(kb, k, n, pu, eu, k, 0, pb, eb, qpad, 1.0, false, B_out + l0, L, 0, res, capb, err, st));
+      }
       int h = 0;
       DSRG_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, st));
       DSRG_CUDA(cudaStreamSynchronize(st));

@@ -892,9 +892,9 @@ int residue_stage(int nm, const double* src, long R, int K, long rs, long ks, in
   return DSRG_FNO_ERR_ARG;
 }
 
-size_t residue_plain_bytes(int nm, long M, long N) {
+size_t residue_plain_bytes(int nm, long M, long N, int cap) {
   const long tiles = (long)ceil_div(M, GT_M) * ceil_div(N, GT_M);
-  return (size_t)std::min<long>(tiles, RES_PLAIN_CAP) * residue_tile_bytes(nm);
+  return (size_t)std::min<long>(tiles, cap) * residue_tile_bytes(nm);
 }
 
 size_t residue_tile_bytes(int nm) { return (size_t)nm * GT_M * GT_M * sizeof(uint16_t); }
