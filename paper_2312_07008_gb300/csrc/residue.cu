@@ -36,14 +36,16 @@ __global__ void __launch_bounds__(256) row_norm_kernel(const T* __restrict__ src
   const long row0 = (long)blockIdx.x * 32;
   double s = 0.0;
   uint32_t hi = 0;
+  auto take = [&](const T* p, int k, long step) {
+    for (; k < k1; k += 8) {
+      const T v = p[k * step];
+      s += square_of(v);
+      hi = max(hi, high_word(v));
+    }
+  };
   if (ks == 1) {  // 8 threads per row
     const long row = row0 + (threadIdx.x >> 3);
-    if (row < R)
-      for (int k = k0 + (threadIdx.x & 7); k < k1; k += 8) {
-        const T v = src[row * rs + k];
-        s += square_of(v);
-        hi = max(hi, high_word(v));
-      }
+    if (row < R) take(src + row * rs, k0 + (threadIdx.x & 7), 1);
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) {
       s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -57,12 +59,7 @@ __global__ void __launch_bounds__(256) row_norm_kernel(const T* __restrict__ src
   __shared__ uint32_t red_hi[8][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const long row = row0 + lane;
-  if (row < R)
-    for (int k = k0 + w; k < k1; k += 8) {
-      const T v = src[row * rs + (long)k * ks];
-      s += square_of(v);
-      hi = max(hi, high_word(v));
-    }
+  if (row < R) take(src + row * rs, k0 + w, ks);
   red[w][lane] = s;
   red_hi[w][lane] = hi;
   __syncthreads();
