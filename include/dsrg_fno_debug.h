@@ -57,7 +57,8 @@ int dsrg_fno_debug_mma_schedule(int32_t nslices, int32_t* entries, int32_t max_e
 
 /* Output tiles of the pair contraction for one batch of hole pairs, host
  * only: pairs[2k], pairs[2k+1] = (i, j), i <= j < ncore + nact; the tiles are
- * 128-row x N-column blocks (N = 48 for 5 planes, 64 for 3 or 4) of the
+ * 128-row x N-column blocks (N = 48 for 5 planes, 64 for 3 or 4), or with
+ * nslices = 10 the 256 x 256 blocks of the residue form (what 5 slices run), of the
  * (nh np) x (nh np) matrix of all hole-particle rows; energy_only restricts
  * the needed elements to virtual x virtual.  tiles[2t], tiles[2t+1] = (row
  * tile, column tile) in the kernel's order.  Returns the tile count, or

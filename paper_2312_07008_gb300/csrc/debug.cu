@@ -181,7 +181,8 @@ extern "C" int64_t dsrg_fno_debug_workspace_allocations(void) { return ws_alloca
 extern "C" int dsrg_fno_debug_pair_tiles(int32_t nslices, int32_t ncore, int32_t nact, int32_t nvir,
                                          const int32_t* pairs, int32_t npairs, int32_t energy_only,
                                          int32_t* tiles, int32_t max_tiles) {
-  if (nslices < 3 || nslices > 5 || ncore < 0 || nact < 0 || nvir <= 0 || ncore + nact <= 0 || npairs < 0 ||
+  const bool residue = nslices == RES_MOD;
+  if ((!residue && (nslices < 3 || nslices > 5)) || ncore < 0 || nact < 0 || nvir <= 0 || ncore + nact <= 0 || npairs < 0 ||
       (npairs > 0 && !pairs) || !tiles)
     return DSRG_FNO_ERR_ARG;
   Geometry g{};
@@ -195,9 +196,9 @@ extern "C" int dsrg_fno_debug_pair_tiles(int32_t nslices, int32_t ncore, int32_t
     pr[k] = make_int2(pairs[2 * k], pairs[2 * k + 1]);
     if (pr[k].x < 0 || pr[k].y < pr[k].x || pr[k].y >= g.nh) return DSRG_FNO_ERR_ARG;
   }
-  const int bn = pair_tile_n(FORM_DIGITS, nslices);
-  DSRG_TRY(pair_tiles(PAIR_TILE_M, bn, g, pr.data(), npairs, energy_only != 0, out));
-  if ((long)out.size() > max_tiles || (long)out.size() > pair_tile_bound(PAIR_TILE_M, bn, g, npairs)) return DSRG_FNO_ERR_ARG;
+  const int bm = residue ? RES_TILE : PAIR_TILE_M, bn = residue ? RES_TILE : pair_tile_n(FORM_DIGITS, nslices);
+  DSRG_TRY(pair_tiles(bm, bn, g, pr.data(), npairs, energy_only != 0, out));
+  if ((long)out.size() > max_tiles || (long)out.size() > pair_tile_bound(bm, bn, g, npairs)) return DSRG_FNO_ERR_ARG;
   for (size_t t = 0; t < out.size(); ++t) {
     tiles[2 * t] = out[t].x;
     tiles[2 * t + 1] = out[t].y;
