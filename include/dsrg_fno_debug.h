@@ -99,6 +99,11 @@ int dsrg_fno_debug_set_eig_colpair(int32_t on);
  * Allocates device memory; DSRG_FNO_ERR_NOCONV if a solve did not converge. */
 int dsrg_fno_debug_eig_batch(int32_t count, const int32_t* n, double* const* A, double* const* V);
 
+/* 1 / x, 1 / sqrt(x) and sqrt(x) of the divide and conquer's iterations for n
+ * positive x (host arrays): each from a float32 estimate and one step of third
+ * order, the library's functions outside float32's range. */
+int dsrg_fno_debug_dc_roots(int32_t n, const double* x, double* rcp, double* rsqrt, double* sqrt);
+
 /* Bytes of device workspace the single-instance calls hold on the current
  * device (grow-only; 0 before the first call and after dsrg_fno_release()).
  * Host only: reads the library's bookkeeping, launches nothing. */

@@ -39,6 +39,7 @@ EXPORTED = (
     "dsrg_fno_debug_slice_rows_dd",
     "dsrg_fno_debug_regularizer",
     "dsrg_fno_debug_mma_schedule",
+    "dsrg_fno_debug_dc_roots",
     "dsrg_fno_debug_workspace_bytes",
     "dsrg_fno_debug_workspace_allocations",
     "dsrg_fno_debug_eig_batch",
@@ -151,6 +152,8 @@ def load(path: str = LIB_PATH):
     lib.dsrg_fno_debug_eig_batch.argtypes = [i32, ctypes.POINTER(i32), ctypes.POINTER(ctypes.POINTER(d)),
                                              ctypes.POINTER(ctypes.POINTER(d))]
     lib.dsrg_fno_debug_eig_batch.restype = ctypes.c_int
+    lib.dsrg_fno_debug_dc_roots.argtypes = [i32, dp, dp, dp, dp]
+    lib.dsrg_fno_debug_dc_roots.restype = ctypes.c_int
     lib.dsrg_fno_debug_workspace_allocations.argtypes = []
     lib.dsrg_fno_debug_workspace_allocations.restype = ctypes.c_int64
     lib.dsrg_fno_debug_workspace_bytes.argtypes = []

@@ -171,6 +171,20 @@ extern "C" int dsrg_fno_debug_eig_batch(int32_t count, const int32_t* n, double*
   return DSRG_FNO_OK;
 }
 
+extern "C" int dsrg_fno_debug_dc_roots(int32_t n, const double* x, double* rcp, double* rsqrt, double* sqrt) {
+  if (n <= 0 || !x || !rcp || !rsqrt || !sqrt) return DSRG_FNO_ERR_ARG;
+  DevBuf d;
+  const size_t bytes = sizeof(double) * n;
+  DSRG_CUDA(cudaMalloc(&d.p, 4 * bytes));
+  double* p = (double*)d.p;
+  DSRG_CUDA(cudaMemcpy(p, x, bytes, cudaMemcpyHostToDevice));
+  DSRG_TRY(eig_dc_roots_test(n, p, p + n, p + 2 * (size_t)n, p + 3 * (size_t)n, 0));
+  DSRG_CUDA(cudaMemcpy(rcp, p + n, bytes, cudaMemcpyDeviceToHost));
+  DSRG_CUDA(cudaMemcpy(rsqrt, p + 2 * (size_t)n, bytes, cudaMemcpyDeviceToHost));
+  DSRG_CUDA(cudaMemcpy(sqrt, p + 3 * (size_t)n, bytes, cudaMemcpyDeviceToHost));
+  return DSRG_FNO_OK;
+}
+
 extern "C" int64_t dsrg_fno_debug_workspace_bytes(void) {
   std::lock_guard<std::mutex> lk(workspace_mutex());
   return (int64_t)workspace_for_current_device().cap;

@@ -734,7 +734,21 @@ __global__ void __launch_bounds__(256) dc_back_kernel(int n, const double* __res
   }
 }
 
+__global__ void dc_roots_test_kernel(int n, const double* x, double* rcp, double* rsqrt, double* root) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    rcp[i] = dc_rcp(x[i]);
+    rsqrt[i] = dc_rsqrt(x[i]);
+    root[i] = dc_sqrt(x[i]);
+  }
+}
+
 }  // namespace
+
+int eig_dc_roots_test(int n, const double* x, double* rcp, double* rsqrt, double* sqrt, cudaStream_t st) {
+  dc_roots_test_kernel<<<ceil_div(n, 256), 256, 0, st>>>(n, x, rcp, rsqrt, sqrt);
+  DSRG_LAUNCH_CHECK();
+  return DSRG_FNO_OK;
+}
 
 // A (n x n, symmetric) is destroyed: on return its diagonal holds the
 // eigenvalues (any order) and V's columns the eigenvectors.  work:

@@ -39,8 +39,11 @@ DC_HD int dc_node_rows(int n, int l) { return (n + (1 << l) - 1) >> l; }
 constexpr int DC_DEFLATE_ROW_BYTES = 8 + 8 + 8 + 4 + 1 + 1;
 DC_HD int dc_deflate_bytes(int n, int l) { return DC_DEFLATE_ROW_BYTES * dc_node_rows(n, l); }
 
-// 1 / x, 1 / sqrt(x) and sqrt(x) from a float32 estimate and one step of third
-// order (relative error of a few 2^-53): chains of 3 to 5 float64 instructions
+// 1 / x, 1 / sqrt(x) and sqrt(x) from a float32 estimate r and the binomial series in
+// what it leaves, e = 1 - x r and 1 - x r^2: 1 / x = r (1 - e)^-1 = r (1 + e + e^2 +
+// ...), 1 / sqrt(x) = r (1 - e)^-1/2 = r (1 + e / 2 + 3 e^2 / 8 + ...), up to e^2.  With
+// |e| below 2^-22 and 2^-20 the rest is under 2^-60, the roundings leave relative
+// errors of 1, 3/2 and 5/2 units of 2^-53.  Chains of 3 to 5 float64 instructions
 // where the library's take 15 to 30; an SM has two float64 lanes, and a chain of
 // float64 operations is what most steps of the solver wait for.
 DC_HD double dc_rcp(double x) {

@@ -82,6 +82,7 @@ constexpr size_t eig_work_doubles(int n) {
 constexpr int EIG_DC_MIN_N = 33, EIG_DC_MAX_N = 7700;
 int eig_dc(int n, double* A, double* V, double* work, unsigned* bar, int* status_dev, long long spin_limit, bool shared,
            cudaStream_t st);
+int eig_dc_roots_test(int n, const double* x, double* rcp, double* rsqrt, double* sqrt, cudaStream_t st);
 int eig_set_barrier_limit(long long spins);
 void set_eig_colpair(bool on);
 int eig_sym_jacobi(int n, double* A, double* V, double* work, int* status_dev, int max_sweeps,
