@@ -23,8 +23,6 @@ __global__ void reg_tables_fill_kernel() {
     g_reg.T[j] = dd_from_double(exp2(-j / 64.0));
     g_reg.C[j] = dd_from_double(-expm1(-j * 0.69314718055994530942 / 64.0));
   }
-  if (threadIdx.x == 0) {
-  }
 }
 
 __device__ __forceinline__ void reg_tables_load(RegTables& R) {

@@ -666,15 +666,15 @@ int dispatch_gemm(int KS, const void* pa, long rows_a, const void* pb, long rows
     switch (KS) {
       case 3: return launch_gemm<3, 64, 3, FORM_DIGITS_T>(pa, rows_a, pb, rows_b, Kpad, P, st);
       case 4: return launch_gemm<4, 64, 2, FORM_DIGITS_T>(pa, rows_a, pb, rows_b, Kpad, P, st);
-      case 5: return launch_gemm<5, 48, 2, FORM_DIGITS_T>(pa, rows_a, pb, rows_b, Kpad, P, st);
-      default: return DSRG_FNO_ERR_ARG;
+      default: return DSRG_FNO_ERR_ARG;  // 5 planes: the residue form
     }
   }
   switch (KS) {
     case 3: return launch_gemm<3, 64, 3>(pa, rows_a, pb, rows_b, Kpad, P, st);
     case 4: return launch_gemm<4, 64, 2>(pa, rows_a, pb, rows_b, Kpad, P, st);
+    // 5 planes: the pair contraction where the ten residue planes do not fit the device
     case 5: return launch_gemm<5, 48, 2>(pa, rows_a, pb, rows_b, Kpad, P, st);
-    // 6 planes (21 products): TMEM allows N = 32, shared memory one stage
+    // 6 planes (test hook) (21 products): TMEM allows N = 32, shared memory one stage
     case 6: return P.mode == MODE_PLAIN ? launch_gemm<6, 32, 1>(pa, rows_a, pb, rows_b, Kpad, P, st)
                                         : DSRG_FNO_ERR_ARG;
     default: return DSRG_FNO_ERR_ARG;
