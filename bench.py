@@ -648,7 +648,7 @@ def main():
         "vs_baseline": None, "dtype": dtype_of(args.nslices),
         "data": "synthetic",
         "config": dict(single_config(p, args.workload, cuts, args.nslices),
-                       epilogue="fused" if args.fused_epilogue else "separate kernel"),
+                       epilogue="fused" if args.fused_epilogue and args.nslices in (3, 4) else "separate kernel"),
         "gflops": flops * value / 1e9,
         "s_per_solve": ms_max / args.steps / 1e3,
         "roofline": roofline,

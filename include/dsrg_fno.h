@@ -53,7 +53,8 @@ typedef enum {
  * power-of-two scale, whose products run on the tensor cores (tcgen05) with
  * exact float32 sums.  With 5 planes (the default) the contractions are formed
  * modulo 10 coprime numbers (residue form, rows scaled to a 2-norm of 2^44) and
- * put together by the Chinese remainder theorem; otherwise the
+ * put together by the Chinese remainder theorem (a pass whose B is too large for
+ * the ten planes takes five digit planes for its contraction); otherwise the
  * integers are split into `nslices` exact bfloat16 digit planes, whose level
  * sums are merged into double-float accumulators (float32 hi + lo pairs, about
  * 48 bits); the
@@ -130,9 +131,10 @@ int dsrg_fno_pt2_energy(const dsrg_fno_problem* prob, double* e2_out, void* stre
  * In the single-reference limit (nact = 0) E^(2) = E_vv plus the singles of
  * f_hp.  Errors as for dsrg_fno_pt2_energy; a host lambda3 gives
  * DSRG_FNO_ERR_ARG, a non-finite one DSRG_FNO_ERR_NONFINITE.  Device
- * workspace: about 32 nh^2 np nact bytes beyond the E_vv pass, plus the digit
- * planes of B (2 nslices nh np naux bytes) on the tensor-core path (grow-only,
- * freed by dsrg_fno_release).  Synchronises `stream`. */
+ * workspace: about 32 nh^2 np nact bytes beyond the E_vv pass, plus the planes
+ * of B on the tensor-core path (20 nh np naux bytes with 5 slices, in parts where
+ * memory is short; 2 nslices nh np naux otherwise; grow-only, freed by
+ * dsrg_fno_release).  Synchronises `stream`. */
 int dsrg_fno_pt2_energy_mr(const dsrg_fno_problem* prob, const double* lambda3, double* e2_out,
                            double* evv_out, void* stream);
 
@@ -248,8 +250,9 @@ int dsrg_fno_truncate_noalloc(int32_t nvir, const double* dvv, int32_t mode, dou
  *   T          device [npairs][nv][nv]: T[p][c][d] = T^{ij}_{cd} of hole pair p.
  *   precision  DSRG_FNO_FP64 or DSRG_FNO_SLICED_BF16 (residue form, 10 moduli).
  *   C_out      device [npairs][nv][nv].
- * The 4-index integrals are formed for 16 values of a at a time and never
- * stored whole.  Errors: DSRG_FNO_ERR_ARG for bad sizes, null or host
+ * The 4-index integrals are formed for a block of values of a at a time: 16 in
+ * FP64; in the fast form up to 2^28 integrals (all of a small basis) within the
+ * memory that is free.  Errors: DSRG_FNO_ERR_ARG for bad sizes, null or host
  * pointers; DSRG_FNO_ERR_NONFINITE for a NaN/Inf in B_vv or T; sizes with
  * nv^3 * 16 or npairs * nv^2 >= 2^31 and other precisions give
  * DSRG_FNO_ERR_UNSUPPORTED. */

@@ -18,11 +18,13 @@ extern "C" {
 /* enable != 0 starts recording (and clears earlier records); 0 stops. */
 void dsrg_fno_profile_enable(int32_t enable);
 
-/* Totals over the recorded launches of kernel `name` ("sliced_gemm_pair",
- * "sliced_gemm_syrk", "sliced_gemm_plain", "pair_gemm_f64", or a phase
+/* Totals over the recorded launches of kernel `name` ("residue_gemm_pair",
+ * "residue_gemm_syrk", "residue_gemm_plain": 5 slices; "sliced_gemm_pair",
+ * "sliced_gemm_syrk", "sliced_gemm_plain": digit planes; "pair_gemm_f64"; or a phase
  * "phase_*"): summed event time (ms), number of launches, and summed executed
  * flops.  Counters without timing ("eig_sweeps_large" / "eig_sweeps_small":
- * Jacobi sweeps of matrices with n >= 256 / n < 256) report calls in
+ * Jacobi sweeps of matrices with n >= 256 / n < 256; none from 33 to 7700 rows, which
+ * divide and conquer solves) report calls in
  * `launches` and the summed count in `flops`.  Returns 0. */
 int dsrg_fno_profile_query(const char* name, double* total_ms, int64_t* launches, double* flops);
 

@@ -199,8 +199,8 @@ struct PassBuffers {
   int* status;
   int nsplit;
   // fast form
-  int ks;             // digit planes (0 = float64 form)
-  int ks_d;           // digit planes of the dressed matrices (rank-K update)
+  int ks;             // slices (0 = float64 form; 5: residues, 3 and 4: digit planes)
+  int ks_d;           // slices of the dressed matrices (rank-K update)
   int2 pform;         // form and parts of the B.B contraction
   int kpad_q, kpad_v; // padded contraction lengths (naux, nvir)
   __nv_bfloat16 *planes_b, *planes_s;
@@ -212,7 +212,7 @@ struct PassBuffers {
   float2* nu;        // double-float contraction tiles
   float2* eps_dd;    // orbital energies as double-float
   unsigned* rowmax;  // max |hi| per row of the dressed matrices (float bits)
-  float2* hp;        // [nh np] eps_i - eps_a, double-float (fused epilogue)
+  float2* hp;        // [nh np] eps_i - eps_a, double-float (fused epilogue, residue form)
   const RegTables* reg;
   bool fused;        // Eq. A7 epilogue inside the contraction kernel
   bool residue;      // B.B contraction in the residue form
@@ -327,7 +327,7 @@ static int run_pass(const Geometry& g, const double* B, const double* eps, const
   }
   const int ntd = ceil_div(g.nv, 32);
   if (W.ks) {
-    // digit planes of B: rows (hole, particle), contraction over Q
+    // planes of B (residues, digits or literal parts): rows (hole, particle), contraction over Q
     const long rows = (long)g.nh * g.np;
     DSRG_PHASE("phase_stage_b", st);
     if (W.residue)

@@ -1,10 +1,10 @@
 // Symmetric eigensolver (Eq. 8: Gamma V = n V) and helpers: the dispatch, the
 // Jacobi kernels and the sorting.  From EIG_DC_MIN_N = 33 rows on the solver is
-// divide and conquer in float64 (eig_dc.cu): at 34 rows it takes 0.72 ms
-// against 0.78 ms here, at 80 1.3 against 5.1, at 203 3.1 against 9.1, at 1200
-// 27 against 97 (D_vv-like matrices; errors 2e-15 of the largest eigenvalue
-// against 1e-13).  The Jacobi kernels keep the smaller matrices, those above
-// EIG_DC_MAX_N, and the density step's, which share one launch.
+// divide and conquer in float64 (eig_dc.cu): at 90 rows it takes 0.80 ms against
+// 2.7 ms here, at 203 1.6 against 9.1, at 1200 16.8 against 97 (D_vv-like matrices;
+// errors 2e-15 of the largest eigenvalue against 1e-13; in its first form, twice as
+// slow, it was level with Jacobi at 34 rows).  The Jacobi kernels keep the smaller
+// matrices, of which a density step's share one launch, and those above EIG_DC_MAX_N.
 //
 // Cyclic two-sided Jacobi with round-robin pair ordering: in each round the
 // indices form m/2 disjoint pairs (m = n rounded up to even, a padding index

@@ -6,8 +6,8 @@
 //   1. BA[Q][j][y] = B[Q][j][y] for the active particles y (gather), and the
 //      integrals <ay|ij> = sum_Q B[Q][i][a] BA[Q][j][y] as one GEMM (M = nh np
 //      rows (i, a), N = nh na columns (j, y), K = naux): in the fast form on
-//      the tensor cores from exact bf16 digit planes of both operands (the
-//      plain mode of the digit-plane contraction kernel), else float64.
+//      the tensor cores from exact bf16 residues (5 slices) or digit planes of
+//      both operands (the plain mode of either contraction kernel), else float64.
 //   2. Eq. A7 amplitudes tp and the vertex xp; Eq. A6 singles t1 and x1.
 //   3. The images of T under Theta (particles) and Gamma (holes): z1, tpp,
 //      z2, z3, g2t, w3, tt1, gt1.

@@ -760,7 +760,7 @@ __device__ __forceinline__ Pieces2 pieces2_of(float4 v, float fa, float fb) {
 
 // Residue planes [RES_MOD_S][nr][nv][Kpad] of the dressed matrices (double-float
 // rows, contiguous), scaled by their segment's row exponents.  Bound by memory: 8
-// bytes read and 18 written per element; float32 arithmetic in packed pairs, about
+// bytes read and 20 written per element; float32 arithmetic in packed pairs, about
 // 50 instructions per element (165 with 64-bit integers; nvir 600 with 40 core and
 // 10 active orbitals 4.99 -> 3.96 ms, 6.5 TB/s).  Exponents beyond +-126 need two
 // factors.

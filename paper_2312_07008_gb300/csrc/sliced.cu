@@ -1,7 +1,7 @@
 // Contractions by exact bfloat16 digit planes on the tcgen05 tensor cores (the
 // planes are staged by stage.cu): the fast form with 3 or 4 planes, and the
 // literal forms of the precision study.  With 5 planes the residue form
-// (residue.cu) takes its place.
+// (residue.cu) takes its place, except in passes whose B is too large for its planes.
 //
 // Products.  For two rows a, b:  x_a . x_b = 2^-14 sum_L 2^-8L S_L with the
 // level sums S_L = sum_{s+t=L} sum_k d_s(a,k) d_t(b,k).  Only levels
@@ -674,7 +674,7 @@ int dispatch_gemm(int KS, const void* pa, long rows_a, const void* pb, long rows
     case 4: return launch_gemm<4, 64, 2>(pa, rows_a, pb, rows_b, Kpad, P, st);
     // 5 planes: the pair contraction where the ten residue planes do not fit the device
     case 5: return launch_gemm<5, 48, 2>(pa, rows_a, pb, rows_b, Kpad, P, st);
-    // 6 planes (test hook) (21 products): TMEM allows N = 32, shared memory one stage
+    // 6 planes (21 products; test hook): TMEM allows N = 32, shared memory one stage
     case 6: return P.mode == MODE_PLAIN ? launch_gemm<6, 32, 1>(pa, rows_a, pb, rows_b, Kpad, P, st)
                                         : DSRG_FNO_ERR_ARG;
     default: return DSRG_FNO_ERR_ARG;
