@@ -866,10 +866,10 @@ def naf_timing(pkg, dev, nslices, keep_frac=0.75):
 TRAFFIC = {
     "sa_cas10_ncore60_nvir1200_naux3600": {
         # small-case capture (energy pass of ncore 20 / nact 4 / nvir 700 / naux 3600):
-        # 8.185 GB read + 3.013 GB written for 1.1088e13 executed flops
-        "bytes_per_exec_flop": (8.185194e9 + 3.013085e9) / 1.10883137e13,
+        # 8.72 GB read + 3.01 GB written for 1.1088e13 executed flops
+        "bytes_per_exec_flop": (8.72e9 + 3.01e9) / 1.10883137e13,
         "sha256": {"paper_2312_07008_gb300/csrc/residue.cu":
-                   "5d8747b7cdab178808ca87171877d8a45d952ba3e06d7de1af612db0eabb2e88",
+                   "1efe718f3fa64ac134295b31e96ea115a5205dc74a1e6d0d918494debcd52377",
                    "paper_2312_07008_gb300/csrc/tc_ptx.cuh":
                    "1759ad784a427ead3781e6d492cf0fa7ab5e5d37e44eb1bb38bc52f14c94e780"},
     },
